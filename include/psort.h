@@ -70,6 +70,9 @@ typedef enum {
 
 /* Tuning parameters.  0 in a field means "choose automatically" (a tuned
  * entry from ps_autotune, else the library's size-binned default).
+ * A keys-only sort with every field automatic and no trace may sort its input
+ * as one block whatever ps_resolve_params reports (the result is the same);
+ * n_B and n_P then matter to sorts that fix them or ask for a trace.
  * n_blocks = n_B and n_parts = n_P of Sec. 2; both may exceed n (empty blocks
  * or partitions are legal).  Limits: 1 <= n_blocks <= 4096,
  * 1 <= n_parts <= 1048576.
@@ -322,8 +325,10 @@ int ps_debug_fail_alloc(int count);
  * global and shared-memory index in its kernels; the first out-of-range
  * access is not performed but recorded.  ps_debug_violation waits for
  * nothing, reads and clears that record: it returns 1 and fills out[0..3]
- * with (site + 100 * key family, index, bound, CTA) if a violation was seen,
- * 0 if none (always 0 in an ordinary build), or a negative status. */
+ * with (site + 100 * kernel family, index, bound, CTA) if a violation was seen,
+ * 0 if none, or a negative status.  An ordinary build reports one thing only:
+ * site 90 (index = tile), a radix pass's bounded wait for an earlier tile that
+ * gave up (it never does in a correct run; the sort's output is then wrong). */
 int ps_debug_violation(uint64_t* out);
 
 /* ---- profiling (library-wide, off by default) ---------------------------

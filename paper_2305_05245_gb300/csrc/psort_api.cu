@@ -304,6 +304,30 @@ static int log_level()
     return lvl;
 }
 
+// Keys-only sorts whose blocks are the library's choice sort their input as
+// one block, by radix (the result is the same whatever the blocks are, and
+// nothing is left to partition or merge), from this many keys on.  Measured,
+// tiles and multiway merges against radix: 2^17 int32 keys 72 / 74 us (below,
+// the launches of the digit passes cost more than the merges), 3,000,001
+// float32 251 / 102 us, 2^26 int32 1.90 / 1.13 ms, 2^30 int64 54.7 / 47.4 ms
+// (a copy of the keys included in the last three).
+#ifndef PS_RADIX_MIN
+#define PS_RADIX_MIN 100000
+#endif
+static bool free_params(const ps_params* p, const ps_trace* trace)
+{
+    if (trace) return false;
+    return !p || (p->n_blocks <= 0 && p->n_parts <= 0 && p->items_per_thread == 0 && p->block_threads == 0);
+}
+static bool radix_takes(const SortArgs& a)
+{
+    if (a.dtype < 0 || a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
+    const bool one = a.n_B == 1 && a.n_P == 1 && !a.trace && a.items == 0 && a.threads == 0;
+    if (!a.free_blocks && !one) return false;
+    if (a.n_inst != 1 || a.inst_ptrs || a.src_keys || a.dst_keys || a.inst_base) return false;
+    return a.n >= PS_RADIX_MIN;
+}
+
 static int dispatch(SortArgs& a)
 {
     if (log_level() >= 1)
@@ -313,6 +337,7 @@ static int dispatch(SortArgs& a)
     int rc = PS_OK;
     const ShapeEntry* sh = shape_of(a.dtype, a.items, a.threads, &rc);
     if (rc != PS_OK) return rc;
+    if (radix_takes(a)) return tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
     if (sh) return sh->run(a);
     switch (a.dtype) {
     case PS_I32: case PS_F32: case PS_U32: return run_sort_u32(a);
@@ -349,6 +374,7 @@ static int sort_common(void* keys, uint32_t* payload, int64_t n, int dtype, int 
     a.threads = r.block_threads;
     a.trace = trace;
     a.stream = (cudaStream_t)stream;
+    a.free_blocks = free_params(params, trace);
     return dispatch(a);
 }
 
@@ -362,14 +388,32 @@ static size_t dtype_size(int dtype)
     return (dtype == PS_I32 || dtype == PS_F32 || dtype == PS_U32) ? 4 : 8;
 }
 
+// Workspace of the radix block sort of n keys as one block (0: it does not
+// take them).
+static size_t radix_bytes(int64_t n, int dtype)
+{
+    SortArgs a;
+    a.keys = nullptr;
+    a.payload = nullptr;
+    a.n = n;
+    a.dtype = dtype;
+    a.mode = PS_PIVOT_EXACT;
+    a.n_B = a.n_P = 1;
+    a.trace = nullptr;
+    a.stream = nullptr;
+    if (!radix_takes(a)) return 0;
+    return tune_family(dtype) == 0 ? radix_bytes_u32(a) : radix_bytes_u64(a);
+}
+
 size_t sort_ws_bytes(int64_t n, int dtype)
 {
     ps_params r;
     resolve(n, dtype, nullptr, &r);
     switch (dtype) {
-    case PS_I32: case PS_F32: case PS_U32: return ws_bytes_u32(n, r.n_blocks, r.n_parts);
+    case PS_I32: case PS_F32: case PS_U32:
+        return std::max(radix_bytes(n, dtype), ws_bytes_u32(n, r.n_blocks, r.n_parts));
     case -1: return ws_bytes_rec(n, r.n_blocks, r.n_parts);
-    default: return ws_bytes_u64(n, r.n_blocks, r.n_parts);
+    default: return std::max(radix_bytes(n, dtype), ws_bytes_u64(n, r.n_blocks, r.n_parts));
     }
 }
 
@@ -1054,7 +1098,7 @@ int ps_workspace_bytes(int64_t n, int dtype, const ps_params* params, size_t* ou
         a.n_P = r.n_parts;
         a.trace = nullptr;
         a.stream = nullptr;
-        *out = sh->ws(a);
+        *out = std::max(sh->ws(a), free_params(params, nullptr) ? radix_bytes(n, dtype) : (size_t)0);
         return PS_OK;
     }
     switch (dtype) {
@@ -1062,6 +1106,8 @@ int ps_workspace_bytes(int64_t n, int dtype, const ps_params* params, size_t* ou
     case -1: *out = ws_bytes_rec(n, r.n_blocks, r.n_parts); break;
     default: *out = ws_bytes_u64(n, r.n_blocks, r.n_parts); break;
     }
+    if (free_params(params, nullptr) || (r.n_blocks == 1 && r.n_parts == 1))
+        *out = std::max(*out, radix_bytes(n, dtype));
     return PS_OK;
 }
 
@@ -1138,9 +1184,10 @@ int ps_debug_violation(uint64_t* out)
 {
     if (!out) return PS_ERR_INVALID_ARG;
     unsigned long long v[4];
-    int (*readers[3])(unsigned long long*) = {viol_read_u32, viol_read_u64, viol_read_rec};
+    int (*readers[])(unsigned long long*) = {viol_read_u32, viol_read_u64, viol_read_rec, viol_read_radix_u32,
+                                             viol_read_radix_u64};
     int found = 0;
-    for (int f = 0; f < 3; f++) {
+    for (int f = 0; f < (int)(sizeof(readers) / sizeof(readers[0])); f++) {
         int rc = readers[f](v);
         if (rc < 0) return rc;
         if (rc == 1 && !found) {

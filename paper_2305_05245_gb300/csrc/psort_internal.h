@@ -61,6 +61,9 @@ struct SortArgs {
     // last pass writes it back there; `keys` (extent keys, laid out by
     // inst_base) only carries the passes in between.
     void* const* inst_ptrs = nullptr;
+    // n_B and n_P are the library's choice and no intermediates are asked for:
+    // the block sort may take the whole input as one block (radix_takes).
+    bool free_blocks = false;
 };
 
 // Workspace from the library's stream-ordered pool.
@@ -94,6 +97,8 @@ size_t ws_bytes_rec(int64_t n, int64_t n_B, int64_t n_P);
 int viol_read_u32(unsigned long long* out);
 int viol_read_u64(unsigned long long* out);
 int viol_read_rec(unsigned long long* out);
+int viol_read_radix_u32(unsigned long long* out);
+int viol_read_radix_u64(unsigned long long* out);
 // Batched sort of the segments [off[i], off[i+1]) of keys (host offsets).
 // pinned (optional): page-locked host scratch of pinned_cap int64 for the
 // instance table; when given, the call does not wait for the stream.
@@ -123,6 +128,12 @@ int run_sort_u64_on(const SortArgs& a, char* ws, size_t cap);
 int run_front_u32(const SortArgs* t, const SortArgs* sm, unsigned long long* next);
 int run_front_u64(const SortArgs* t, const SortArgs* sm, unsigned long long* next);
 constexpr int64_t SMALL_SEG = 1024;
+// The radix block sort (psort_radix.cuh) of every instance as one block, and
+// the workspace it takes.
+int run_radix_u32(const SortArgs& a);
+int run_radix_u64(const SortArgs& a);
+size_t radix_bytes_u32(const SortArgs& a);
+size_t radix_bytes_u64(const SortArgs& a);
 // Workspace bytes of the sort a describes (batched instances included).
 size_t ws_bytes_args_u32(const SortArgs& a);
 size_t ws_bytes_args_u64(const SortArgs& a);

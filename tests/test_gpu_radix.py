@@ -1,0 +1,99 @@
+"""The radix block sort (one block, keys only) against the plain definition of
+the result (the unique ascending order of the keys' bits, oracle.reference_sort):
+sizes around its tiles and its smallest size, every key type, distributions
+that leave digits out (all keys equal, one varying byte, few values) or that
+fill a digit with one value, unaligned buffers, and repeated runs."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+T32, T64 = 512 * 24, 512 * 16  # keys per tile of a digit pass
+MIN = 100000                   # smallest size the radix block sort takes
+
+
+@pytest.fixture(scope="module")
+def ps():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2305_05245_gb300 as ps
+    assert torch.cuda.is_available()
+    return ps
+
+
+def check(ps, ora, host, mode="exact", offset=0, **kw):
+    """Sort host on the device (starting `offset` elements into a buffer)."""
+    import torch
+    st = {"uint32": np.int32, "uint64": np.int64}.get(str(host.dtype), host.dtype)
+    buf = torch.zeros(host.size + offset + 3, dtype=torch.from_numpy(host[:1].view(st)).dtype, device="cuda")
+    x = buf[offset:offset + host.size]
+    x.copy_(torch.from_numpy(host.view(st)))
+    y = x.view(getattr(torch, str(host.dtype))) if st != host.dtype else x
+    ps.sort(y, mode, **kw)
+    torch.cuda.synchronize()
+    got = x.cpu().numpy().view(host.dtype)
+    want = ora.reference_sort(host)
+    assert got.tobytes() == want.tobytes()
+    assert not buf[:offset].any() and not buf[offset + host.size:].any()
+
+
+SIZES = [MIN - 1, MIN, MIN + 1, 9 * T32 - 1, 9 * T32, 9 * T32 + 1, 13 * T64 - 1, 13 * T64, 13 * T64 + 1, 1 << 20,
+         3000017]
+
+
+@pytest.mark.parametrize("dtype", sorted(synth.DTYPES))
+@pytest.mark.parametrize("n", SIZES)
+def test_sizes(ps, ora, dtype, n):
+    check(ps, ora, synth.keys(n, dtype, "uniform", seed=synth.seed_for("radix", n)))
+
+
+@pytest.mark.parametrize("dtype", sorted(synth.DTYPES))
+@pytest.mark.parametrize("dist", ["sorted", "reverse", "few_unique", "gaussian", "almost_sorted", "three_valued"])
+def test_distributions(ps, ora, dtype, dist):
+    if dist == "gaussian" and not dtype.startswith("float"):
+        pytest.skip("gaussian keys are floating point")
+    check(ps, ora, synth.keys(400003, dtype, dist, seed=synth.seed_for("radix", dist)), mode="regular")
+
+
+@pytest.mark.parametrize("dtype", ["int32", "uint32", "int64", "uint64"])
+@pytest.mark.parametrize("bytes_", [(), (0,), (1,), (0, 3), (1, 2, 3), (-1,), (2, -1)])
+def test_varying_bytes(ps, ora, dtype, bytes_):
+    """Only the named bytes of the keys vary: none to three passes have work."""
+    width = np.dtype(dtype).itemsize
+    z = synth.splitmix64(7, 250001)
+    u = np.full(z.size, 0x0123456789ABCDEF, dtype=np.uint64)
+    for b in bytes_:
+        s = np.uint64(8 * (b % width))
+        u = (u & ~(np.uint64(255) << s)) | (((z >> s) & np.uint64(255)) << s)
+    host = (u & np.uint64(0xFFFFFFFF)).astype(np.uint32).view(dtype) if width == 4 else u.view(dtype)
+    check(ps, ora, np.ascontiguousarray(host))
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+def test_float_specials(ps, ora, dtype):
+    x = synth.keys(200001, dtype, "gaussian", seed=5)
+    info = np.finfo(dtype)
+    sp = np.array([0.0, -0.0, np.inf, -np.inf, info.max, info.min, info.tiny, -info.tiny,
+                   info.smallest_subnormal, -info.smallest_subnormal], dtype=dtype)
+    x[::17] = sp[np.arange(x[::17].size) % sp.size]
+    check(ps, ora, x)
+
+
+@pytest.mark.parametrize("dtype,offset", [("int32", 1), ("float32", 3), ("int64", 1), ("float64", 1)])
+def test_unaligned_buffers(ps, ora, dtype, offset):
+    check(ps, ora, synth.keys(150007, dtype, "uniform", seed=9), offset=offset)
+
+
+def test_one_block_given_by_the_caller(ps, ora):
+    check(ps, ora, synth.keys(300007, "int32", "uniform", seed=3), n_blocks=1, n_parts=1)
+
+
+def test_repeated_runs_are_identical(ps, ora):
+    host = synth.keys(1 << 20, "int64", "few_unique", seed=11)
+    for _ in range(10):
+        check(ps, ora, host)
