@@ -11,6 +11,8 @@
 // digit counts, sums the counts of the tiles before it and publishes the sum.
 #pragma once
 
+#include <type_traits>
+
 #include "psort_kernels.cuh"
 
 namespace ps {
@@ -30,6 +32,8 @@ template <> struct Rx<uint32_t> {
         return up & ~((1u << (8 * lo)) - 1);
     }
     __device__ static __forceinline__ bool lt(uint32_t a, uint32_t b, M m) { return (a & m) < (b & m); }
+    __device__ static __forceinline__ bool same(uint32_t a, uint32_t b, M m) { return ((a ^ b) & m) == 0; }
+    __device__ static __forceinline__ uint64_t word(uint32_t a, M m) { return a & m; }
 };
 template <> struct Rx<uint64_t> {
     static constexpr int D = 8;
@@ -44,6 +48,8 @@ template <> struct Rx<uint64_t> {
         return up & ~((1ull << (8 * lo)) - 1);
     }
     __device__ static __forceinline__ bool lt(uint64_t a, uint64_t b, M m) { return (a & m) < (b & m); }
+    __device__ static __forceinline__ bool same(uint64_t a, uint64_t b, M m) { return ((a ^ b) & m) == 0; }
+    __device__ static __forceinline__ uint64_t word(uint64_t a, M m) { return a & m; }
 };
 
 // What one segment's passes do: digits dig[0..npass), ascending.
@@ -54,8 +60,9 @@ struct RxPlan {
 };
 
 // Device tables and buffers of one radix sort.  Pass 0 reads `first`, pass i
-// writes b (i even) or a (i odd); the last pass (which has an odd index)
-// writes `last`.
+// writes b (i even) or a (i odd); a last pass of odd index writes `last`
+// instead of a.  (A last pass of even index leaves the keys in b: only when
+// low digits were left out, k_rx_fix then moves them to `last`.)
 template <typename K> struct RxArgs {
     GBuf<K> first, a, b, last;
     Inst in;
@@ -70,6 +77,10 @@ template <typename K> struct RxArgs {
     unsigned* ticket;        // [D]: next tile of each pass
     int64_t chunk;           // keys per counting chunk
     int64_t RC;              // chunk slots per segment
+    int sample;              // sampled keys (0: none, every digit is sorted)
+    unsigned* hits;          // [D]: the sample's hits per choice of the lowest digit
+    uint8_t* flags;          // [fix tiles], see k_rx_fix
+    unsigned* nflag;         // number of flagged tiles
     int min_pass;            // least number of passes (a sort between two buffers needs some)
     bool keep;               // the last pass leaves order keys
 };
@@ -91,6 +102,74 @@ template <typename K> __device__ __forceinline__ GBuf<K> rx_sub(const GBuf<K>& g
 // The first look-back wait that gave up (tile + 1), recorded like an index
 // violation; 0 in every correct run.
 static __device__ unsigned long long rx_stall;
+
+// ------------------------------------------------------------ sampling
+// How many low bytes the passes may leave out (wide keys of one segment).
+// Sorting by the leading bytes alone leaves runs of keys that agree in them;
+// where such runs are short, putting them in order afterwards (k_rx_fix) costs
+// less than the passes it saves: 2^30 uniform 64-bit keys are nearly distinct
+// in their leading four bytes.  The sample tells: S keys at hashed positions
+// enter one hash table per choice of `lo` (open addressing, keyed by the bytes
+// lo and above); a key that meets an earlier one of the same leading bytes
+// which it follows or precedes in the wrong order counts as a hit.  S keys
+// have S^2/2 pairs, half of which would be in the wrong order, so a key has
+// about 4 * hits * n / S^2 others in its run that are out of order; the
+// smallest number of leading bytes that keeps this at PS_RX_RUN or less wins.
+// A wrong guess costs time, never order.  Measured: 2^30 int64 uniform 47.4 ->
+// 27.3 ms, 2^26 float64 Gaussian 3.03 -> 2.3 ms (five leading bytes), a copy of
+// the keys included.
+#ifndef PS_RX_RUN
+#define PS_RX_RUN 1
+#endif
+constexpr int RX_SAMPLE_MAX = 1 << 16;
+__device__ __forceinline__ uint64_t rx_mix(uint64_t z)
+{
+    // SplitMix64's finaliser (Steele, Lea & Flood 2014)
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+// blockIdx.y: the choice of lo, less 1.  tab: [D][2 * S] entries (sample + 1).
+template <typename K, int XF>
+__global__ void __launch_bounds__(128) k_rx_sample(RxArgs<K> A, unsigned* tab)
+{
+    const int S = A.sample;
+    constexpr int D = Rx<K>::D;
+    const int64_t n = A.in.n0;
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    auto at = [&](int j) { return (int64_t)__umul64hi(rx_mix((uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull), (uint64_t)n); };
+    const bool in = i < S;
+    const int64_t pi = in ? at(i) : 0;
+    const K x = A.first.template ldx<XF>(pi);
+    const int lo = 1 + blockIdx.y;
+    const typename Rx<K>::M m = Rx<K>::mask(lo, D - 1);
+    bool hit = false;
+    unsigned* t = tab + (size_t)lo * 2 * S;
+    unsigned q = (unsigned)rx_mix(Rx<K>::word(x, m)) & (unsigned)(2 * S - 1);
+    for (int probe = 0; in && probe < 2 * S; probe++) {
+        const unsigned cur = atomicCAS(&t[q], 0u, (unsigned)(i + 1));
+        if (cur == 0) break;
+        const int64_t pj = at((int)cur - 1);
+        const K y = A.first.template ldx<XF>(pj);
+        if (Rx<K>::same(x, y, m)) {
+            hit = pi < pj ? key_lt(y, x) : key_lt(x, y);
+            break;
+        }
+        q = (q + 1) & (unsigned)(2 * S - 1);
+    }
+    const unsigned c = __popc(__ballot_sync(0xFFFFFFFFu, hit));
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&A.hits[lo], c);
+}
+// The choice, by one warp: the largest lo up to which no prefix has too many hits.
+template <typename K> __device__ __forceinline__ int rx_choose_lo(const RxArgs<K>& A)
+{
+    constexpr int D = Rx<K>::D;
+    if (A.sample == 0) return 0;
+    const int q = (threadIdx.x & 31) + 1;
+    const double h = q <= D - 2 ? (double)__ldcg(&A.hits[q]) : 0.0;
+    const bool ok = q <= D - 2 && h * 4.0 * (double)A.in.n0 <= (double)PS_RX_RUN * (double)A.sample * (double)A.sample;
+    return __ffs(~__ballot_sync(0xFFFFFFFFu, ok)) - 1;
+}
 
 // ------------------------------------------------------------ counting
 // One CTA counts G digits (group blockIdx.y) of one chunk of one segment.
@@ -115,6 +194,8 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     if (c0 >= len) return;
     const int n = (int)(len - c0 < A.chunk ? len - c0 : A.chunk);
     const int g0 = blockIdx.y * G;
+    const int lo0 = D > G ? rx_choose_lo(A) : 0;
+    if (g0 + G <= lo0) return;
     for (int i = threadIdx.x; i < G * 4096; i += NT) cnt[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -122,6 +203,7 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     auto add = [&](const K& k) {
 #pragma unroll
         for (int d = 0; d < G; d++) {
+            if (D > G && g0 + d < lo0) continue;
             const unsigned v = Rx<K>::dig(k, g0 + d);
             atomicAdd(&cnt[d * 4096 + ((v >> 1) << 5) + lane], (v & 1) ? 65536u : 1u);
         }
@@ -152,7 +234,7 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned parts = (unsigned)((len + A.chunk - 1) / A.chunk) * gridDim.y;
+        const unsigned parts = (unsigned)((len + A.chunk - 1) / A.chunk) * (gridDim.y - lo0 / G);
         s_last = atomicAdd(&A.done[seg], 1u) == parts - 1;
     }
     __syncthreads();
@@ -188,16 +270,17 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     __syncthreads();
     if (threadIdx.x == 0) {
         RxPlan p;
-        p.lo = 0;
+        p.lo = lo0;
         int act = 0;
-        for (int d = 0; d < D; d++) act += !s_all[d];
+        for (int d = lo0; d < D; d++) act += !s_all[d];
         // the passes alternate between two buffers: an even number of them,
-        // filled up with digits that change nothing
-        int want = act + (act & 1);
+        // filled up with digits that change nothing, unless k_rx_fix can move
+        // the keys
+        int want = lo0 ? act : act + (act & 1);
         if (want < A.min_pass) want = A.min_pass;
         int fill = want - act;
         p.npass = 0;
-        for (int d = 0; d < D; d++) {
+        for (int d = lo0; d < D; d++) {
             if (s_all[d] && fill <= 0) continue;
             if (s_all[d]) fill--;
             p.dig[p.npass++] = (uint8_t)d;
@@ -258,7 +341,7 @@ constexpr unsigned RX_SPINS = 1u << 24;  // looks at one predecessor before a wa
 //
 // Bound by shared-memory wavefronts and their latency (L1 data pipe 72%, 50
 // instructions per 32 keys at 2^26 uint32).  Measured at 2^28 uniform keys per
-// pass: 0.79 ms for uint32 (2.7 TB/s), 1.20 ms for uint64 (3.6 TB/s).  Ranks by
+// pass: 0.84 ms for uint32 (2.6 TB/s), 1.17 ms for uint64 (3.7 TB/s).  Ranks by
 // ballots alone took 1.37 and 1.76 ms (ALU bound, 97 instructions per 32
 // keys), __match_any_sync 2.20 ms, matching through shared-memory OR 0.99 ms;
 // the check costs 2-3%.
@@ -297,7 +380,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
         const GBuf<K> own = A.iptr ? GBuf<K>{A.iptr[seg], len} : rx_sub(A.a, off, len);
         const GBuf<K> oth = rx_sub(A.b, off, len);
         const GBuf<K> src = head ? (A.iptr ? own : rx_sub(A.first, off, len)) : (slot & 1) ? oth : own;
-        const GBuf<K> dst = tail ? (A.iptr ? own : rx_sub(A.last, off, len)) : (slot & 1) ? own : oth;
+        const GBuf<K> dst = !(slot & 1) ? oth : (tail && !A.iptr) ? rx_sub(A.last, off, len) : own;
         const int n = (int)(len - o < T ? len - o : T);
         const bool full = n == T;
         const int p0 = w * 32 * E + lane;
@@ -317,19 +400,31 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             }
         };
         load();
+        // the items that hold one digit value, found ahead of the atomics so that
+        // the matches, and then the atomics, overlap
+        uint32_t same = 0;
 #pragma unroll
         for (int j = 0; j < E; j++) {
-            const unsigned v = Rx<K>::dig(k[j], d);
-            int same;
-            __match_all_sync(0xFFFFFFFFu, v, &same);
-            if (same && full) {
-                const uint32_t old = my[v];
-                __syncwarp();
-                if (lane == 0) my[v] = old + 32;
-                __syncwarp();
-                rk[j] = old + lane;
-            } else if (full || p0 + j * 32 < n) {
-                rk[j] = atomicAdd(&my[v], 1u);
+            int s;
+            __match_all_sync(0xFFFFFFFFu, Rx<K>::dig(k[j], d), &s);
+            same |= (uint32_t)(s != 0) << j;
+        }
+        if (full && same == 0) {
+#pragma unroll
+            for (int j = 0; j < E; j++) rk[j] = atomicAdd(&my[Rx<K>::dig(k[j], d)], 1u);
+        } else {
+#pragma unroll
+            for (int j = 0; j < E; j++) {
+                const unsigned v = Rx<K>::dig(k[j], d);
+                if (full && ((same >> j) & 1)) {
+                    const uint32_t old = my[v];
+                    __syncwarp();
+                    if (lane == 0) my[v] = old + 32;
+                    __syncwarp();
+                    rk[j] = old + lane;
+                } else if (full || p0 + j * 32 < n) {
+                    rk[j] = atomicAdd(&my[v], 1u);
+                }
             }
         }
         __syncthreads();
@@ -365,11 +460,10 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
         }
         __syncthreads();
 #pragma unroll
+        for (int j = 0; j < E; j++) rk[j] += my[Rx<K>::dig(k[j], d)];
+#pragma unroll
         for (int j = 0; j < E; j++)
-            if (full || p0 + j * 32 < n) {
-                const uint32_t q = my[Rx<K>::dig(k[j], d)] + rk[j];
-                if (PS_IN(q, T, 51)) sk[q] = k[j];
-            }
+            if ((full || p0 + j * 32 < n) && PS_IN(rk[j], T, 51)) sk[rk[j]] = k[j];
         if (tid < 256) {
             CT excl = 0;
             if (lt == 0) {
@@ -405,23 +499,44 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
         __syncthreads();
         const typename Rx<K>::M m = Rx<K>::mask(pl.lo, d);
         const bool inv = tail && !A.keep;
-        auto store = [&]() {
+        // The tile arrives in the order of the digits before this one: when its
+        // first and last key agree in them, all its keys do and any order within
+        // a group is right.
+        const typename Rx<K>::M mb = d > pl.lo ? Rx<K>::mask(pl.lo, d - 1) : 0;
+        const bool check = !head && !Rx<K>::same(src.ld(o), src.ld(o + n - 1), mb);
+        // (a stale sum after an abandoned wait must not leave the segment)
+        auto store_as = [&](auto ordered, auto inverse) {
+            constexpr int U = E % 8 == 0 ? 8 : E % 6 == 0 ? 6 : 4;
+            static_assert(E % U == 0, "keys per thread are a multiple of the store batch");
             bool bad = false;
 #pragma unroll
-            for (int q = 0; q < E; q++) {
-                const int i = tid + q * NT;
-                if (full || i < n) {
-                    const K x = sk[i];
-                    if (!head) bad |= Rx<K>::lt(x, sk[i > 0 ? i - 1 : 0], m);
-                    const CT p = gb[Rx<K>::dig(x, d)] + (CT)i;
-                    // (a stale sum after an abandoned wait must not leave the segment)
-                    if (p < (CT)len) {
-                        if (inv) dst.template stx<XF>((int64_t)p, x);
-                        else dst.st((int64_t)p, x);
+            for (int q0 = 0; q0 < E; q0 += U) {
+                K x[U], y[U];
+                CT p[U];
+#pragma unroll
+                for (int q = 0; q < U; q++) {
+                    const int i = tid + (q0 + q) * NT;
+                    const bool in = full || i < n;
+                    x[q] = sk[in ? i : 0];
+                    if constexpr (decltype(ordered)::value) y[q] = sk[in && i > 0 ? i - 1 : 0];
+                }
+#pragma unroll
+                for (int q = 0; q < U; q++) p[q] = gb[Rx<K>::dig(x[q], d)] + (CT)(tid + (q0 + q) * NT);
+#pragma unroll
+                for (int q = 0; q < U; q++) {
+                    if (!full && tid + (q0 + q) * NT >= n) continue;
+                    if constexpr (decltype(ordered)::value) bad |= Rx<K>::lt(x[q], y[q], m);
+                    if (p[q] < (CT)len) {
+                        if constexpr (decltype(inverse)::value) dst.template stx<XF>((int64_t)p[q], x[q]);
+                        else dst.st((int64_t)p[q], x[q]);
                     }
                 }
             }
             return bad;
+        };
+        auto store = [&]() {
+            if (!check) return inv ? store_as(std::false_type{}, std::true_type{}) : store_as(std::false_type{}, std::false_type{});
+            return inv ? store_as(std::true_type{}, std::true_type{}) : store_as(std::true_type{}, std::false_type{});
         };
         if (__syncthreads_or(store())) {
 #pragma unroll 1
@@ -448,6 +563,296 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             __syncthreads();
             store();
             __syncthreads();
+        }
+    }
+}
+
+// ------------------------------------------------------- left-out digits
+// After passes over the digits lo and above, keys that agree in them stand in
+// runs, in an order that the low digits have not had a say in.  One CTA owns
+// the runs that start in its FT positions.  It lists them (most keys are runs
+// of their own and need nothing more), one thread sorts each listed run of at
+// most FL keys by insertion in shared memory, and runs that changed are
+// written back.  Keys of a run all stay inside it, so the leading bytes at a
+// position never change and CTAs do not disturb each other's view of the runs,
+// even in place.  Longer runs are left to k_rx_long: a tile in which one of
+// them is out of order gets a flag (1: a run from an earlier tile, 2: one that
+// starts here and goes on into the next tile, 4: one inside the tile).
+// An odd number of passes left the keys in b: every key is then moved to
+// `last`.  Measured on 2^28 uniform uint64 keys, in place: 0.64 ms (every
+// position tested by its own thread with run scans of its own: 1.0 ms).
+constexpr int FT = 4096, FN = 256, FL = 64;
+template <typename K, int XF>
+__global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
+{
+    const RxPlan& pl = A.plan[0];
+    if (pl.lo == 0) return;
+    extern __shared__ __align__(16) char smem[];
+    K* sk = (K*)smem;                                 // [FT + 2 * FL + 1]
+    uint16_t* runs = (uint16_t*)(sk + FT + 2 * FL + 1);  // [FT / 2 + 1]
+    __shared__ unsigned s_runs, s_flag, s_long, s_end;
+    __shared__ int s_in;  // first position of the tile after an earlier tile's short run
+    const int64_t len = A.in.n0;
+    const bool move = pl.npass & 1;
+    const GBuf<K> src = move ? A.b : A.last, dst = A.last;
+    const typename Rx<K>::M m = Rx<K>::mask(pl.lo, Rx<K>::D - 1);
+    const bool inv = !A.keep;
+    const int64_t t0 = (int64_t)blockIdx.x * FT, t1 = t0 + FT < len ? t0 + FT : len;
+    if (t0 >= len) return;
+    const int64_t base = t0 - FL > 0 ? t0 - FL : 0;
+    const int end = (int)((t1 + FL + 1 < len ? t1 + FL + 1 : len) - base);  // keys held
+    const int h0 = (int)(t0 - base), h1 = (int)(t1 - base);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        s_runs = s_flag = s_long = 0;
+        s_end = (unsigned)h1;
+        s_in = h0;
+    }
+    if (inv) {
+#pragma unroll 8
+        for (int i = tid; i < end; i += FN) sk[i] = src.template ldx<XF>(base + i);
+    } else {
+#pragma unroll 8
+        for (int i = tid; i < end; i += FN) sk[i] = src.ld(base + i);
+    }
+    __syncthreads();
+    auto put = [&](int i, const K& x) {
+        if (inv) dst.template stx<XF>(base + i, x);
+        else dst.st(base + i, x);
+    };
+#pragma unroll 4
+    for (int i = h0 + tid; i < h1; i += FN) {
+        const K x = sk[i];
+        const bool next = i + 1 < end && Rx<K>::same(sk[i + 1], x, m);
+        if (next && !(i > 0 && Rx<K>::same(sk[i - 1], x, m))) runs[atomicAdd(&s_runs, 1u)] = (uint16_t)i;
+    }
+    if (tid == 0 && h0 > 0 && Rx<K>::same(sk[h0 - 1], sk[h0], m)) {
+        // the tile begins inside an earlier tile's run
+        const K x = sk[h0];
+        int s = h0 - 1;
+        while (s > 0 && Rx<K>::same(sk[s - 1], x, m)) s--;
+        if (s == 0 || (s + FL < end && Rx<K>::same(sk[s + FL], x, m))) {
+            s_long = 1;
+        } else {
+            int e = h0;
+            while (e < end && Rx<K>::same(sk[e], x, m)) e++;
+            s_in = e;
+        }
+    }
+    __syncthreads();
+    for (unsigned q = tid; q < s_runs; q += FN) {
+        const int s = runs[q];
+        const K x = sk[s];
+        int e = s + 2;
+        bool moved = key_lt(sk[s + 1], x);
+        while (e < end && e <= s + FL && Rx<K>::same(sk[e], x, m)) {
+            moved |= key_lt(sk[e], sk[e - 1]);
+            e++;
+        }
+        if (e > s + FL) {
+            s_long = 1;
+            continue;
+        }
+        if (moved) {
+            for (int i = s + 1; i < e; i++) {
+                const K v = sk[i];
+                int j = i;
+                for (; j > s && key_lt(v, sk[j - 1]); j--) sk[j] = sk[j - 1];
+                sk[j] = v;
+            }
+            if (!move)
+                for (int i = s; i < e; i++) put(i, sk[i]);
+        }
+        if (e > h1) s_end = (unsigned)e;  // (only the last run reaches beyond the tile)
+    }
+    __syncthreads();
+    if (move) {
+        const int i1 = (int)s_end < end ? (int)s_end : end;
+        for (int i = s_in + tid; i < i1; i += FN) put(i, sk[i]);
+    }
+    if (!s_long) return;
+    for (int i = h0 + tid; i < h1; i += FN) {
+        if (i == 0) continue;
+        const K x = sk[i], y = sk[i - 1];
+        if (!Rx<K>::same(y, x, m) || !key_lt(x, y)) continue;  // (short runs are in order by now)
+        if (i < s_in) continue;
+        atomicOr(&s_flag, h0 > 0 && Rx<K>::same(sk[h0 - 1], x, m) ? 1u
+                          : h1 < end && Rx<K>::same(sk[h1], x, m) ? 2u
+                                                                  : 4u);
+    }
+    __syncthreads();
+    if (tid == 0 && s_flag) {
+        A.flags[blockIdx.x] = (uint8_t)s_flag;
+        atomicAdd(A.nflag, 1u);
+    }
+}
+
+// Stable radix sort of x[s, e) by the bytes below lo, by one CTA, with y[s, e)
+// as scratch; both hold keys as the user sees them when inv.
+template <int NT, typename K, int XF>
+__device__ void rx_sort_run(const GBuf<K>& x, const GBuf<K>& y, int64_t s, int64_t e, int lo, bool inv, uint32_t* wt,
+                            unsigned long long* cnt)
+{
+    constexpr int W = NT / 32, E = 4;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    auto ld = [&](const GBuf<K>& b, int64_t i) { return inv ? b.template ldx<XF>(i) : b.ld(i); };
+    bool swapped = false;
+    for (int d = 0; d < lo; d++) {
+        const GBuf<K> src = swapped ? y : x, dst = swapped ? x : y;
+        for (int i = tid; i < 256; i += NT) cnt[i] = 0;
+        __syncthreads();
+        for (int64_t i = s + tid; i < e; i += NT) atomicAdd(&cnt[Rx<K>::dig(ld(src, i), d)], 1ull);
+        __syncthreads();
+        bool all = false;
+        for (int i = tid; i < 256; i += NT) all |= cnt[i] == (unsigned long long)(e - s);
+        if (__syncthreads_or(all)) continue;  // one value: nothing to do
+        if (tid < 32) {  // exclusive sums
+            unsigned long long v[8], t = 0;
+            for (int q = 0; q < 8; q++) t += v[q] = cnt[lane * 8 + q];
+            unsigned long long z = t;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long u = __shfl_up_sync(0xFFFFFFFFu, z, o);
+                if (lane >= o) z += u;
+            }
+            z -= t;
+            for (int q = 0; q < 8; q++) {
+                cnt[lane * 8 + q] = z;
+                z += v[q];
+            }
+        }
+        for (int64_t c = s; c < e; c += NT * E) {
+            for (int i = tid; i < W * 256; i += NT) wt[i] = 0;
+            __syncthreads();
+            K k[E];
+            uint32_t rk[E];
+            for (int j = 0; j < E; j++) {
+                const int64_t i = c + w * 32 * E + j * 32 + lane;
+                const bool in = i < e;
+                k[j] = ld(src, in ? i : s);
+                const unsigned v = Rx<K>::dig(k[j], d);
+                unsigned mt = __ballot_sync(0xFFFFFFFFu, in);
+                for (int b = 0; b < 8; b++) {
+                    const bool bit = (v >> b) & 1;
+                    const unsigned u = __ballot_sync(0xFFFFFFFFu, bit);
+                    mt &= bit ? u : ~u;
+                }
+                const unsigned r = __popc(mt & ((1u << lane) - 1));
+                const uint32_t old = wt[w * 256 + v];
+                __syncwarp();
+                if (in && r == 0) wt[w * 256 + v] = old + __popc(mt);
+                __syncwarp();
+                rk[j] = old + r;
+            }
+            __syncthreads();
+            uint32_t tot = 0;
+            if (tid < 256)
+                for (int q = 0; q < W; q++) {
+                    const uint32_t t = wt[q * 256 + tid];
+                    wt[q * 256 + tid] = tot;
+                    tot += t;
+                }
+            __syncthreads();
+            for (int j = 0; j < E; j++) {
+                if (c + w * 32 * E + j * 32 + lane >= e) continue;
+                const unsigned v = Rx<K>::dig(k[j], d);
+                const int64_t p = s + (int64_t)cnt[v] + wt[w * 256 + v] + rk[j];
+                if (p >= e) continue;
+                if (inv) dst.template stx<XF>(p, k[j]);
+                else dst.st(p, k[j]);
+            }
+            __syncthreads();
+            if (tid < 256) cnt[tid] += tot;
+            __syncthreads();
+        }
+        swapped = !swapped;
+    }
+    if (swapped)
+        for (int64_t i = s + tid; i < e; i += NT) x.st(i, y.ld(i));
+    __syncthreads();
+}
+
+// The long runs that k_rx_fix left out of order, one CTA each (the sample
+// makes them rare).  Who sorts a run that spans tiles: the tile where it
+// starts if that tile saw it out of order, else the first later tile that did.
+// The flags and the leading bytes do not change here, so every CTA decides
+// alike.
+template <typename K, int XF>
+__global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
+{
+    constexpr int NT = 512;
+    if (*A.nflag == 0) return;
+    __shared__ uint32_t wt[(NT / 32) * 256];
+    __shared__ unsigned long long cnt[256];
+    __shared__ unsigned long long s_min;
+    const RxPlan& pl = A.plan[0];
+    const int64_t len = A.in.n0, nt = (len + FT - 1) / FT;
+    const typename Rx<K>::M m = Rx<K>::mask(pl.lo, Rx<K>::D - 1);
+    const bool inv = !A.keep;
+    const GBuf<K> x = A.last, y = A.b;
+    auto ld = [&](int64_t i) { return inv ? x.template ldx<XF>(i) : x.ld(i); };
+    // first position of [a, b) whose leading bytes are not below (not above) v's
+    auto lower = [&](int64_t a, int64_t b, const K& v) {
+        while (a < b) {
+            const int64_t q = a + ((b - a) >> 1);
+            if (Rx<K>::lt(ld(q), v, m)) a = q + 1;
+            else b = q;
+        }
+        return a;
+    };
+    auto upper = [&](int64_t a, int64_t b, const K& v) {
+        while (a < b) {
+            const int64_t q = a + ((b - a) >> 1);
+            if (!Rx<K>::lt(v, ld(q), m)) a = q + 1;
+            else b = q;
+        }
+        return a;
+    };
+    for (int64_t f0 = (int64_t)blockIdx.x * 32; f0 < nt; f0 += (int64_t)gridDim.x * 32) {
+        const int fl = threadIdx.x < 32 && f0 + threadIdx.x < nt ? A.flags[f0 + threadIdx.x] : 0;
+        if (!__syncthreads_or(fl)) continue;
+        for (int64_t f = f0; f < f0 + 32 && f < nt; f++) {
+            const int g = A.flags[f];
+            if (g == 0) continue;
+            const int64_t t0 = f * FT, t1 = t0 + FT < len ? t0 + FT : len;
+            if (g & 4) {
+                for (int64_t from = t0 + 1;;) {
+                    if (threadIdx.x == 0) s_min = ~0ull;
+                    __syncthreads();
+                    for (int64_t i = from + threadIdx.x; i < t1; i += NT) {
+                        const K v = ld(i), u = ld(i - 1);
+                        if (!Rx<K>::same(u, v, m) || !key_lt(v, u)) continue;
+                        if (t0 > 0 && Rx<K>::same(ld(t0 - 1), v, m)) continue;
+                        if (t1 < len && Rx<K>::same(ld(t1), v, m)) continue;
+                        atomicMin(&s_min, (unsigned long long)i);
+                    }
+                    __syncthreads();
+                    const unsigned long long at = s_min;
+                    __syncthreads();
+                    if (at == ~0ull) break;
+                    const K v = ld((int64_t)at);
+                    const int64_t s = lower(t0, (int64_t)at, v), e = upper((int64_t)at, t1, v);
+                    __syncthreads();
+                    rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
+                    from = e;
+                }
+            }
+            if (g & 2) {
+                const K v = ld(t1 - 1);
+                const int64_t s = lower(t0, t1 - 1, v), e = upper(t1, len, v);
+                __syncthreads();
+                rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
+            }
+            if (g & 1) {
+                const K v = ld(t0);
+                const int64_t s = lower(0, t0, v), fs = s / FT;
+                bool other = threadIdx.x == 0 && (A.flags[fs] & 2);
+                for (int64_t q = fs + 1 + threadIdx.x; q < f; q += NT) other |= (A.flags[q] & 1) != 0;
+                if (!__syncthreads_or(other)) {
+                    const int64_t e = upper(t0, len, v);
+                    __syncthreads();
+                    rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
+                }
+            }
         }
     }
 }

@@ -8,19 +8,40 @@
 
 namespace ps {
 
-// Threads, keys per thread and CTAs per SM of a digit pass.
+// Threads, keys per thread and CTAs per SM of a digit pass.  Large tiles spread
+// the fixed work of a tile (digit tables, look-back, barriers) over more keys;
+// sorts of few tiles want more of them at once.  Measured per sort: uint32,
+// 384 x 32 / 512 x 16 / 512 x 8: 2^30 keys 15.1 / 16.4 / 24.1 ms, 2^22 140 / 129 /
+// 147 us, 2^18 79 / 71 / 62 us; uint64, 256 x 24 / 512 x 16 / 512 x 8: 2^30 24.6 /
+// 26.0 / 33.2 ms, 2^20 136 / 137 / 138 us, 2^17 114 / 119 / 107 us.
+template <int NT_, int E_, int CTAS_> struct RxShape {
+    static constexpr int NT = NT_, E = E_, CTAS = CTAS_, T = NT_ * E_;
+};
 template <typename K> struct RxCfg;
-template <> struct RxCfg<uint32_t> { static constexpr int NT = 512, E = 24, CTAS = 2; };
-template <> struct RxCfg<uint64_t> { static constexpr int NT = 512, E = 16, CTAS = 2; };
+template <> struct RxCfg<uint32_t> {
+    using Small = RxShape<512, 8, 2>;
+    using Mid = RxShape<512, 16, 2>;
+    using Large = RxShape<384, 32, 2>;
+    static constexpr int64_t small = int64_t(1) << 18, mid = int64_t(1) << 23;  // up to so many keys
+};
+template <> struct RxCfg<uint64_t> {
+    using Small = RxShape<512, 8, 2>;
+    using Mid = RxShape<256, 24, 3>;
+    using Large = RxShape<256, 24, 3>;
+    static constexpr int64_t small = int64_t(1) << 18, mid = int64_t(1) << 18;
+};
 
 template <typename K> struct Radix {
     using C = RxCfg<K>;
-    static constexpr int D = Rx<K>::D, T = C::NT * C::E;
+    static constexpr int D = Rx<K>::D;
     static constexpr int G = 4, CNT = 512;  // digits and threads of a counting CTA
 
     struct Layout {
+        int T;  // keys per tile
         int64_t nseg, R, ntiles, chunk, RC;
         bool wide;  // 64-bit look-back words
+        int S;      // sampled keys (0: every digit is sorted)
+        size_t o_nflag, o_hits, o_tab, o_flags;
         size_t o_hist, o_done, o_ticket, o_lb0, zero_bytes, o_lb1, o_plan, o_data, total;
     };
     static Layout layout(const SortArgs& a)
@@ -28,13 +49,21 @@ template <typename K> struct Radix {
         Layout y;
         const int64_t nmax = a.inst_base ? a.n_max : a.n, extent = a.inst_base ? a.extent : a.n;
         y.nseg = a.n_inst;
-        y.R = (nmax + T - 1) / T;
+        y.T = nmax <= C::small ? C::Small::T : nmax <= C::mid ? C::Mid::T : C::Large::T;
+        y.R = (nmax + y.T - 1) / y.T;
         y.ntiles = y.nseg * y.R;
         y.wide = nmax >= (int64_t(1) << 30);
         // counting chunks: about four per SM, 4096 to 2^20 keys
         const int64_t want = (nmax * y.nseg) / (152 * 4);
         y.chunk = std::min<int64_t>(int64_t(1) << 20, std::max<int64_t>(4096, (want + 4095) / 4096 * 4096));
         y.RC = (nmax + y.chunk - 1) / y.chunk;
+        // sqrt(8 n) sampled keys: runs of about one key out of order then give
+        // two hits, the least that tells them from none
+        y.S = 0;
+        if (D > 4 && y.nseg == 1) {
+            y.S = 256;
+            while (y.S < RX_SAMPLE_MAX && (int64_t)y.S * y.S < 8 * nmax) y.S *= 2;
+        }
         const size_t lb = align256((size_t)y.ntiles * 256 * (y.wide ? 8 : 4));
         size_t o = 0;
         y.o_hist = o;
@@ -43,6 +72,13 @@ template <typename K> struct Radix {
         o += align256((size_t)y.nseg * 4);
         y.o_ticket = o;
         o += 256;
+        y.o_nflag = o;
+        y.o_hits = o + 8;
+        o += 256;
+        y.o_tab = o;
+        o += align256((size_t)(y.S ? D : 0) * 2 * y.S * 4);
+        y.o_flags = o;
+        o += align256(y.S ? (size_t)(nmax + FT - 1) / FT : 0);
         y.o_lb0 = o;
         o += lb;
         y.zero_bytes = o;  // everything up to here starts as zeros
@@ -56,27 +92,61 @@ template <typename K> struct Radix {
         return y;
     }
 
-    template <int XF, typename CT>
-    static cudaError_t passes(const SortArgs& a, const Layout& y, const RxArgs<K>& A, char* ws, int grid_sms)
+    template <int XF, typename CT, typename SH>
+    static cudaError_t digits(const Layout& y, const RxArgs<K>& A, char* ws, int grid_sms, cudaStream_t s)
     {
-        cudaStream_t s = a.stream;
-        auto fc = k_rx_count<CNT, G, K, XF>;
-        const size_t cb = (size_t)G * 4096 * 4;
-        cudaError_t e = smem_attr(fc, cb);
+        auto fp = k_rx_pass<K, XF, CT, SH::NT, SH::E, SH::CTAS>;
+        constexpr size_t sb = rx_smem<K, CT, SH::NT, SH::E>();
+        cudaError_t e = smem_attr(fp, sb);
         if (e != cudaSuccess) return e;
-        {
-            ProfScope ps_("radix_count", s);
-            fc<<<dim3((unsigned)(y.nseg * y.RC), D / G), CNT, cb, s>>>(A);
-        }
-        auto fp = k_rx_pass<K, XF, CT, C::NT, C::E, C::CTAS>;
-        constexpr size_t sb = rx_smem<K, CT, C::NT, C::E>();
-        if ((e = smem_attr(fp, sb)) != cudaSuccess) return e;
-        const unsigned grid = (unsigned)std::min<int64_t>(y.ntiles, (int64_t)grid_sms * C::CTAS);
+        const unsigned grid = (unsigned)std::min<int64_t>(y.ntiles, (int64_t)grid_sms * SH::CTAS);
         CT* l0 = (CT*)(ws + y.o_lb0);
         CT* l1 = (CT*)(ws + y.o_lb1);
         for (int i = 0; i < D; i++) {
             ProfScope ps_("radix_pass", s);
-            fp<<<grid, C::NT, sb, s>>>(A, i, (i & 1) ? l1 : l0, (i & 1) ? l0 : l1);
+            fp<<<grid, SH::NT, sb, s>>>(A, i, (i & 1) ? l1 : l0, (i & 1) ? l0 : l1);
+        }
+        return cudaGetLastError();
+    }
+
+    template <int XF, typename CT>
+    static cudaError_t passes(const SortArgs& a, const Layout& y, const RxArgs<K>& A, char* ws, int grid_sms)
+    {
+        cudaStream_t s = a.stream;
+        cudaError_t e;
+        if constexpr (D > 4) {
+            if (y.S) {
+                ProfScope ps_("radix_sample", s);
+                k_rx_sample<K, XF><<<dim3((unsigned)((y.S + 127) / 128), D - 2), 128, 0, s>>>(
+                    A, (unsigned*)(ws + y.o_tab));
+            }
+        }
+        auto fc = k_rx_count<CNT, G, K, XF>;
+        const size_t cb = (size_t)G * 4096 * 4;
+        if ((e = smem_attr(fc, cb)) != cudaSuccess) return e;
+        {
+            ProfScope ps_("radix_count", s);
+            fc<<<dim3((unsigned)(y.nseg * y.RC), D / G), CNT, cb, s>>>(A);
+        }
+        if (std::is_same<CT, uint32_t>::value && y.T == C::Small::T)
+            e = digits<XF, uint32_t, typename C::Small>(y, A, ws, grid_sms, s);
+        else if (std::is_same<CT, uint32_t>::value && y.T == C::Mid::T)
+            e = digits<XF, uint32_t, typename C::Mid>(y, A, ws, grid_sms, s);
+        else
+            e = digits<XF, CT, typename C::Large>(y, A, ws, grid_sms, s);
+        if (e != cudaSuccess) return e;
+        if constexpr (D > 4) {
+            if (y.S) {
+                {
+                    auto ff = k_rx_fix<K, XF>;
+                    constexpr size_t fb = sizeof(K) * (FT + 2 * FL + 1) + 2 * (FT / 2 + 2);
+                    if ((e = smem_attr(ff, fb)) != cudaSuccess) return e;
+                    ProfScope ps_("radix_fix", s);
+                    ff<<<(unsigned)((A.in.n0 + FT - 1) / FT), FN, fb, s>>>(A);
+                }
+                ProfScope ps_("radix_long", s);
+                k_rx_long<K, XF><<<(unsigned)grid_sms, 512, 0, s>>>(A);
+            }
         }
         return cudaGetLastError();
     }
@@ -108,6 +178,10 @@ template <typename K> struct Radix {
         A.ticket = (unsigned*)(ws + y.o_ticket);
         A.chunk = y.chunk;
         A.RC = y.RC;
+        A.sample = y.S;
+        A.hits = (unsigned*)(ws + y.o_hits);
+        A.nflag = (unsigned*)(ws + y.o_nflag);
+        A.flags = (uint8_t*)(ws + y.o_flags);
         A.keep = a.keep_order_keys;
         // a sort between two buffers, or one that leaves order keys, moves
         // (and transforms) the keys even when they are all equal

@@ -12,7 +12,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-T32, T64 = 512 * 24, 512 * 16  # keys per tile of a digit pass
+T32, T64 = 384 * 32, 256 * 24  # keys per tile of a digit pass (large sorts; smaller ones: 4096, 8192)
 MIN = 100000                   # smallest size the radix block sort takes
 
 
@@ -42,7 +42,8 @@ def check(ps, ora, host, mode="exact", offset=0, **kw):
     assert not buf[:offset].any() and not buf[offset + host.size:].any()
 
 
-SIZES = [MIN - 1, MIN, MIN + 1, 9 * T32 - 1, 9 * T32, 9 * T32 + 1, 13 * T64 - 1, 13 * T64, 13 * T64 + 1, 1 << 20,
+SIZES = [MIN - 1, MIN, MIN + 1, 683 * T32 - 1, 683 * T32, 683 * T32 + 1, 43 * T64 - 1, 43 * T64,
+         43 * T64 + 1, 26 * 4096 + 1, 1 << 18, (1 << 18) + 1, 1 << 20, (1 << 23) + 1,
          3000017]
 
 
@@ -97,3 +98,52 @@ def test_repeated_runs_are_identical(ps, ora):
     host = synth.keys(1 << 20, "int64", "few_unique", seed=11)
     for _ in range(10):
         check(ps, ora, host)
+
+
+def clustered(n, sizes, top, seed):
+    """n uniform uint64 keys, of which sizes[c] share the leading `top` bytes of
+    one key and differ in the others (runs that the leading bytes alone leave in
+    input order)."""
+    u = synth.splitmix64(seed, n)
+    place = np.argsort(synth.splitmix64(seed + 1, n))[:sum(sizes)]
+    low = np.uint64((1 << (64 - 8 * top)) - 1)
+    at = 0
+    for c, m in enumerate(sizes):
+        idx = place[at:at + m]
+        u[idx] = (u[idx[0]] & ~low) | (u[idx] & low)
+        at += m
+    return u
+
+
+@pytest.mark.parametrize("n,sizes,top", [
+    (1 << 20, (2, 63, 64, 65, 66, 127, 128, 129), 5),   # around the length a run is ranked in place
+    (1 << 20, (700, 40, 300, 2, 3), 4),
+    (1 << 20, (300,) * 2, 7),
+    (1 << 25, (9000,), 5),                              # runs over several tiles of the fix kernel
+    (1 << 25, (5000, 70), 6),
+    (1 << 18, (1 << 18,), 3),                           # one run: the sample sees it
+    (300001, (100000, 50000), 6),
+])
+def test_runs_of_equal_leading_bytes(ps, ora, n, sizes, top):
+    u = clustered(n, sizes, top, seed=n + top)
+    check(ps, ora, u)
+    if n < (1 << 25):
+        check(ps, ora, u.view(np.int64), mode="regular")
+
+
+def test_runs_of_equal_keys(ps, ora):
+    """Long runs of identical keys among distinct ones (never out of order)."""
+    u = synth.splitmix64(3, 1 << 20)
+    u[::5] = u[0]
+    u[1::5] = u[0] ^ np.uint64(1)  # and a neighbour that differs in the last byte only
+    check(ps, ora, u)
+    u[1::5] = u[0]
+    check(ps, ora, u)
+
+
+@pytest.mark.parametrize("n", [110592 - 1, 110592, 110592 + 1, 110592 + 64, 110592 + 65])
+def test_fix_tile_edges(ps, ora, n):
+    """Keys of 24 leading bits that come in pairs and triples, sizes around the
+    fix kernel's tiles of 4096 positions."""
+    z = synth.splitmix64(n, n)
+    check(ps, ora, ((z >> np.uint64(44)) << np.uint64(44)) | (z & np.uint64(255)))
