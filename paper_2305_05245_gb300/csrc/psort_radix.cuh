@@ -52,6 +52,56 @@ template <> struct Rx<uint64_t> {
     __device__ static __forceinline__ uint64_t word(uint64_t a, M m) { return a & m; }
 };
 
+template <> struct Rx<Rec> {
+    static constexpr int D = 12;
+    __device__ static __forceinline__ unsigned dig(const Rec& r, int d)
+    {
+        return d < 4 ? __byte_perm(r.p, 0, 0x4440 | d) : Rx<uint64_t>::dig(r.k, d - 4);
+    }
+    struct M {
+        uint64_t k;
+        uint32_t p;
+    };
+    __device__ static M mask(int lo, int d)
+    {
+        return M{d < 4 ? 0 : Rx<uint64_t>::mask(lo < 4 ? 0 : lo - 4, d - 4),
+                 lo > 3 ? 0 : Rx<uint32_t>::mask(lo, d > 3 ? 3 : d)};
+    }
+    __device__ static __forceinline__ bool lt(const Rec& a, const Rec& b, M m)
+    {
+        return (a.k & m.k) < (b.k & m.k) || ((a.k & m.k) == (b.k & m.k) && (a.p & m.p) < (b.p & m.p));
+    }
+    __device__ static __forceinline__ bool same(const Rec& a, const Rec& b, M m)
+    {
+        return ((a.k ^ b.k) & m.k) == 0 && ((a.p ^ b.p) & m.p) == 0;
+    }
+    __device__ static __forceinline__ uint64_t word(const Rec& a, M m)
+    {
+        return (a.k & m.k) + (uint64_t)(a.p & m.p) * 0x9E3779B97F4A7C15ull;
+    }
+};
+
+// Keys of one tile in shared memory.
+template <typename K> struct RxTile {
+    K* a;
+    static constexpr size_t bytes(int n) { return sizeof(K) * n; }
+    __device__ RxTile(char*& sp, int n) : a((K*)sp) { sp += bytes(n); }
+    __device__ __forceinline__ K ld(int i) const { return a[i]; }
+    __device__ __forceinline__ void st(int i, const K& v) const { a[i] = v; }
+};
+template <> struct RxTile<Rec> {
+    uint64_t* k;
+    uint32_t* p;
+    static constexpr size_t bytes(int n) { return 12 * (size_t)n; }
+    __device__ RxTile(char*& sp, int n) : k((uint64_t*)sp), p((uint32_t*)(sp + 8 * (size_t)n)) { sp += bytes(n); }
+    __device__ __forceinline__ Rec ld(int i) const { return Rec{k[i], p[i]}; }
+    __device__ __forceinline__ void st(int i, const Rec& v) const
+    {
+        k[i] = v.k;
+        p[i] = v.p;
+    }
+};
+
 // What one segment's passes do: digits dig[0..npass), ascending.
 struct RxPlan {
     int npass;
@@ -97,6 +147,23 @@ template <typename K> __device__ __forceinline__ void rx_seg(const RxArgs<K>& A,
 template <typename K> __device__ __forceinline__ GBuf<K> rx_sub(const GBuf<K>& g, int64_t off, int64_t len)
 {
     return GBuf<K>{g.p + off, len};
+}
+template <> __device__ __forceinline__ GBuf<Rec> rx_sub(const GBuf<Rec>& g, int64_t off, int64_t len)
+{
+    return GBuf<Rec>{g.k + off, g.p + off, len};
+}
+// The segment's part of its instance's own buffer (keys only).
+template <typename K> __device__ __forceinline__ GBuf<K> rx_own(K* const* iptr, int64_t seg, int64_t off, int64_t len)
+{
+    return GBuf<K>{iptr[seg] + off, len};
+}
+template <> __device__ __forceinline__ GBuf<Rec> rx_own(Rec* const*, int64_t, int64_t, int64_t) { return GBuf<Rec>{nullptr, nullptr, 0}; }
+// A key of which only the digits of group g0.. matter.
+template <int XF, typename K> __device__ __forceinline__ K rx_ld_digits(const GBuf<K>& b, int64_t i, int) { return b.template ldx<XF>(i); }
+template <int XF> __device__ __forceinline__ Rec rx_ld_digits(const GBuf<Rec>& b, int64_t i, int g0)
+{
+    if (!PS_IN(i, b.n, 1)) return Rec{0, 0};
+    return g0 < 4 ? Rec{0, b.p[i]} : Rec{b.k[i], 0};
 }
 
 // The first look-back wait that gave up (tile + 1), recorded like an index
@@ -199,7 +266,7 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     for (int i = threadIdx.x; i < G * 4096; i += NT) cnt[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const GBuf<K> src = A.iptr ? GBuf<K>{A.iptr[seg] + c0, (int64_t)n} : rx_sub(A.first, off + c0, (int64_t)n);
+    const GBuf<K> src = A.iptr ? rx_own(A.iptr, seg, c0, (int64_t)n) : rx_sub(A.first, off + c0, (int64_t)n);
     auto add = [&](const K& k) {
 #pragma unroll
         for (int d = 0; d < G; d++) {
@@ -213,11 +280,11 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     for (; i + (U - 1) * NT < n; i += U * NT) {
         K k[U];
 #pragma unroll
-        for (int u = 0; u < U; u++) k[u] = src.template ldx<XF>(i + u * NT);
+        for (int u = 0; u < U; u++) k[u] = rx_ld_digits<XF>(src, i + u * NT, g0);
 #pragma unroll
         for (int u = 0; u < U; u++) add(k[u]);
     }
-    for (; i < n; i += NT) add(src.template ldx<XF>(i));
+    for (; i < n; i += NT) add(rx_ld_digits<XF>(src, i, g0));
     __syncthreads();
     unsigned long long* h = A.hist + seg * (D * 256);
     for (int r = threadIdx.x; r < G * 128; r += NT) {
@@ -316,11 +383,40 @@ template <typename CT> struct Lb {
     }
 };
 
+// One segment's part in one pass.
+template <typename K> struct RxSegPass {
+    GBuf<K> src, dst;
+    int64_t len;
+    typename Rx<K>::M m, mb;  // the digits sorted after this pass, and before it
+    int npass, d;
+    bool inv;  // the pass writes the keys as the user sees them
+};
+template <typename K>
+__device__ __forceinline__ void rx_seg_pass(const RxArgs<K>& A, int64_t seg, int slot, RxSegPass<K>& sg)
+{
+    int64_t off, len;
+    rx_seg(A, seg, off, len);
+    const RxPlan& pl = A.plan[seg];
+    sg.len = len;
+    sg.npass = len > 0 ? pl.npass : 0;
+    if (slot >= sg.npass) return;
+    const int d = pl.dig[slot];
+    const bool tail = slot + 1 == sg.npass;
+    const GBuf<K> own = A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.a, off, len);
+    const GBuf<K> oth = rx_sub(A.b, off, len);
+    sg.d = d;
+    sg.src = slot == 0 ? (A.iptr ? own : rx_sub(A.first, off, len)) : (slot & 1) ? oth : own;
+    sg.dst = !(slot & 1) ? oth : (tail && !A.iptr) ? rx_sub(A.last, off, len) : own;
+    sg.inv = tail && !A.keep;
+    sg.m = Rx<K>::mask(pl.lo, d);
+    sg.mb = d > pl.lo ? Rx<K>::mask(pl.lo, d - 1) : typename Rx<K>::M{};
+}
+
 // Shared memory of one pass CTA: the tile's keys grouped by digit, one digit
 // table per warp, and every digit's destination.
 template <typename K, typename CT, int NT, int E> constexpr size_t rx_smem()
 {
-    return sizeof(K) * NT * E + (NT / 32) * 1024 + 256 * sizeof(CT) + 64;
+    return RxTile<K>::bytes(NT * E) + (NT / 32) * 1024 + 256 * sizeof(CT) + 64;
 }
 
 constexpr unsigned RX_SPINS = 1u << 24;  // looks at one predecessor before a wait gives up
@@ -341,7 +437,10 @@ constexpr unsigned RX_SPINS = 1u << 24;  // looks at one predecessor before a wa
 //
 // Bound by shared-memory wavefronts and their latency (L1 data pipe 72%, 50
 // instructions per 32 keys at 2^26 uint32).  Measured at 2^28 uniform keys per
-// pass: 0.84 ms for uint32 (2.6 TB/s), 1.17 ms for uint64 (3.7 TB/s).  Ranks by
+// pass: 0.77 ms for uint32 (2.8 TB/s), 1.10 ms for uint64 (3.9 TB/s), 1.7 ms for
+// records (3.8 TB/s).  What a tile costs whatever it holds is kept small: its
+// number is fetched ahead, the segment's constants sit in shared memory and ranks
+// two to a register (all of them in registers spilled: 1.04 ms for uint32).  Ranks by
 // ballots alone took 1.37 and 1.76 ms (ALU bound, 97 instructions per 32
 // keys), __match_any_sync 2.20 ms, matching through shared-memory OR 0.99 ms;
 // the check costs 2-3%.
@@ -351,48 +450,57 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
     constexpr int T = NT * E, W = NT / 32, LB = 8;
     static_assert(NT >= 256, "one thread per digit value");
     extern __shared__ __align__(16) char smem[];
-    K* sk = (K*)smem;
-    uint32_t* wt = (uint32_t*)(sk + T);  // [W][256]
+    char* sp = smem;
+    const RxTile<K> sk(sp, T);
+    uint32_t* wt = (uint32_t*)sp;        // [W][256]
     CT* gb = (CT*)(wt + W * 256);        // [256]: destination of the digit's group, less its place in the tile
     __shared__ unsigned s_tile, s_w[8];
+    __shared__ __align__(16) char s_seg[sizeof(RxSegPass<K>)];
+    RxSegPass<K>& sg = *(RxSegPass<K>*)s_seg;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     uint32_t* my = wt + w * 256;
-    const bool single = A.nseg == 1;
+    const bool single = A.nseg == 1, head = slot == 0;
     if (single && slot >= A.plan[0].npass) return;
-    for (;;) {
-        if (tid == 0) s_tile = atomicAdd(&A.ticket[slot], 1u);
-        ((uint4*)my)[lane] = make_uint4(0, 0, 0, 0);
-        ((uint4*)my)[lane + 32] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
-        const int64_t tile = s_tile;
-        if (tile >= A.ntiles) return;
+    if (tid == 0) s_tile = atomicAdd(&A.ticket[slot], 1u);
+    __syncthreads();
+    int64_t cur = -1;
+    for (int64_t tile = s_tile; tile < A.ntiles;) {
         const int64_t seg = single ? 0 : tile / A.R, lt = single ? tile : tile - seg * A.R;
-        int64_t off, len;
-        rx_seg(A, seg, off, len);
-        const int64_t o = lt * T;
-        const RxPlan& pl = A.plan[seg];
-        if (o >= len || slot >= pl.npass) {
+        if (seg != cur) {
+            cur = seg;
             __syncthreads();
+            if (tid == 0) rx_seg_pass(A, seg, slot, sg);
+            __syncthreads();
+        }
+        const int64_t o = lt * T;
+        if (slot >= sg.npass || o >= sg.len) {
+            __syncthreads();
+            if (tid == 0) s_tile = atomicAdd(&A.ticket[slot], 1u);
+            __syncthreads();
+            tile = s_tile;
             continue;
         }
-        const int d = pl.dig[slot];
-        const bool head = slot == 0, tail = slot + 1 == pl.npass;
-        const GBuf<K> own = A.iptr ? GBuf<K>{A.iptr[seg], len} : rx_sub(A.a, off, len);
-        const GBuf<K> oth = rx_sub(A.b, off, len);
-        const GBuf<K> src = head ? (A.iptr ? own : rx_sub(A.first, off, len)) : (slot & 1) ? oth : own;
-        const GBuf<K> dst = !(slot & 1) ? oth : (tail && !A.iptr) ? rx_sub(A.last, off, len) : own;
-        const int n = (int)(len - o < T ? len - o : T);
+        const int d = sg.d;
+        // the next tile's number, fetched while this tile is ranked
+        unsigned next = 0;
+        if (tid == NT - 1) next = atomicAdd(&A.ticket[slot], 1u);
+        ((uint4*)my)[lane] = make_uint4(0, 0, 0, 0);
+        ((uint4*)my)[lane + 32] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+        const int n = (int)(sg.len - o < T ? sg.len - o : T);
         const bool full = n == T;
         const int p0 = w * 32 * E + lane;
         K k[E];
-        uint32_t rk[E];
+        uint32_t rk[E / 2] = {};  // two ranks a register
+        auto put_rank = [&](int j, uint32_t r) { rk[j / 2] = (j & 1) ? __byte_perm(rk[j / 2], r, 0x5410) : r; };
         auto load = [&]() {
+            const GBuf<K> src = sg.src;
             if (full) {
 #pragma unroll
                 for (int j = 0; j < E; j++) k[j] = src.ld(o + p0 + j * 32);
             } else {
 #pragma unroll
-                for (int j = 0; j < E; j++) k[j] = p0 + j * 32 < n ? src.ld(o + p0 + j * 32) : K(0);
+                for (int j = 0; j < E; j++) k[j] = p0 + j * 32 < n ? src.ld(o + p0 + j * 32) : K{};
             }
             if (head) {
 #pragma unroll
@@ -400,43 +508,44 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             }
         };
         load();
-        // the items that hold one digit value, found ahead of the atomics so that
-        // the matches, and then the atomics, overlap
-        uint32_t same = 0;
+        // Items of one digit value come in crowds (sorted input, few values): a
+        // warp looks at four of its items and takes the careful path for all of
+        // them if one is uniform.
+        bool crowd = !full;
 #pragma unroll
-        for (int j = 0; j < E; j++) {
+        for (int j = 0; j < E; j += E / 4) {
             int s;
             __match_all_sync(0xFFFFFFFFu, Rx<K>::dig(k[j], d), &s);
-            same |= (uint32_t)(s != 0) << j;
+            crowd |= s != 0;
         }
-        if (full && same == 0) {
+        if (!crowd) {
 #pragma unroll
-            for (int j = 0; j < E; j++) rk[j] = atomicAdd(&my[Rx<K>::dig(k[j], d)], 1u);
+            for (int j = 0; j < E; j++) put_rank(j, atomicAdd(&my[Rx<K>::dig(k[j], d)], 1u));
         } else {
 #pragma unroll
             for (int j = 0; j < E; j++) {
                 const unsigned v = Rx<K>::dig(k[j], d);
-                if (full && ((same >> j) & 1)) {
-                    const uint32_t old = my[v];
+                int s;
+                __match_all_sync(0xFFFFFFFFu, v, &s);
+                uint32_t r = 0;
+                if (full && s) {
+                    r = my[v] + lane;
                     __syncwarp();
-                    if (lane == 0) my[v] = old + 32;
+                    if (lane == 0) my[v] = r + 32;
                     __syncwarp();
-                    rk[j] = old + lane;
                 } else if (full || p0 + j * 32 < n) {
-                    rk[j] = atomicAdd(&my[v], 1u);
+                    r = atomicAdd(&my[v], 1u);
                 }
+                put_rank(j, r);
             }
         }
         __syncthreads();
+        if (tid == NT - 1) s_tile = next;
         uint32_t tot = 0, ex = 0;
         CT* row = lb + tile * 256;
         if (tid < 256) {
 #pragma unroll
-            for (int i = 0; i < W; i++) {
-                const uint32_t c = wt[i * 256 + tid];
-                wt[i * 256 + tid] = tot;
-                tot += c;
-            }
+            for (int i = 0; i < W; i++) tot += wt[i * 256 + tid];
             const CT start = lt == 0 ? (CT)A.hist[(seg * Rx<K>::D + d) * 256 + tid] : 0;
             if (lt == 0) gb[tid] = start;
             Lb<CT>::st(row + tid, lt == 0 ? (Lb<CT>::SUM | (start + tot)) : (Lb<CT>::OWN | (CT)tot));
@@ -455,15 +564,28 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
 #pragma unroll
             for (int i = 0; i < 7; i++)
                 if (i < w) ex += s_w[i];
+            uint32_t at = ex;
 #pragma unroll
-            for (int i = 0; i < W; i++) wt[i * 256 + tid] += ex;
+            for (int i0 = 0; i0 < W; i0 += 4) {
+                uint32_t c[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) c[i] = wt[(i0 + i) * 256 + tid];
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    wt[(i0 + i) * 256 + tid] = at;
+                    at += c[i];
+                }
+            }
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < E; j++) rk[j] += my[Rx<K>::dig(k[j], d)];
+        for (int j = 0; j < E; j += 2)
+            rk[j / 2] += my[Rx<K>::dig(k[j], d)] + (my[Rx<K>::dig(k[j + 1], d)] << 16);
 #pragma unroll
-        for (int j = 0; j < E; j++)
-            if ((full || p0 + j * 32 < n) && PS_IN(rk[j], T, 51)) sk[rk[j]] = k[j];
+        for (int j = 0; j < E; j++) {
+            const uint32_t q = (j & 1) ? rk[j / 2] >> 16 : rk[j / 2] & 0xFFFFu;
+            if ((full || p0 + j * 32 < n) && PS_IN(q, T, 51)) sk.st(q, k[j]);
+        }
         if (tid < 256) {
             CT excl = 0;
             if (lt == 0) {
@@ -497,18 +619,19 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             gb[tid] = excl - ex;
         }
         __syncthreads();
-        const typename Rx<K>::M m = Rx<K>::mask(pl.lo, d);
-        const bool inv = tail && !A.keep;
+        const unsigned after = s_tile;
         // The tile arrives in the order of the digits before this one: when its
         // first and last key agree in them, all its keys do and any order within
         // a group is right.
-        const typename Rx<K>::M mb = d > pl.lo ? Rx<K>::mask(pl.lo, d - 1) : 0;
-        const bool check = !head && !Rx<K>::same(src.ld(o), src.ld(o + n - 1), mb);
+        const bool check = !head && !Rx<K>::same(sg.src.ld(o), sg.src.ld(o + n - 1), sg.mb);
         // (a stale sum after an abandoned wait must not leave the segment)
         auto store_as = [&](auto ordered, auto inverse) {
-            constexpr int U = E % 8 == 0 ? 8 : E % 6 == 0 ? 6 : 4;
+            constexpr int U = sizeof(K) == 4 ? 8 : sizeof(K) == 8 ? 4 : 2;  // store batch
             static_assert(E % U == 0, "keys per thread are a multiple of the store batch");
             bool bad = false;
+            const GBuf<K> dst = sg.dst;
+            const typename Rx<K>::M m = sg.m;
+            const CT len = (CT)sg.len;
 #pragma unroll
             for (int q0 = 0; q0 < E; q0 += U) {
                 K x[U], y[U];
@@ -517,8 +640,8 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
                 for (int q = 0; q < U; q++) {
                     const int i = tid + (q0 + q) * NT;
                     const bool in = full || i < n;
-                    x[q] = sk[in ? i : 0];
-                    if constexpr (decltype(ordered)::value) y[q] = sk[in && i > 0 ? i - 1 : 0];
+                    x[q] = sk.ld(in ? i : 0);
+                    if constexpr (decltype(ordered)::value) y[q] = sk.ld(in && i > 0 ? i - 1 : 0);
                 }
 #pragma unroll
                 for (int q = 0; q < U; q++) p[q] = gb[Rx<K>::dig(x[q], d)] + (CT)(tid + (q0 + q) * NT);
@@ -526,7 +649,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
                 for (int q = 0; q < U; q++) {
                     if (!full && tid + (q0 + q) * NT >= n) continue;
                     if constexpr (decltype(ordered)::value) bad |= Rx<K>::lt(x[q], y[q], m);
-                    if (p[q] < (CT)len) {
+                    if (p[q] < len) {
                         if constexpr (decltype(inverse)::value) dst.template stx<XF>((int64_t)p[q], x[q]);
                         else dst.st((int64_t)p[q], x[q]);
                     }
@@ -535,14 +658,16 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             return bad;
         };
         auto store = [&]() {
+            const bool inv = sg.inv;
             if (!check) return inv ? store_as(std::false_type{}, std::true_type{}) : store_as(std::false_type{}, std::false_type{});
             return inv ? store_as(std::true_type{}, std::true_type{}) : store_as(std::true_type{}, std::false_type{});
         };
-        if (__syncthreads_or(store())) {
+        const bool bad = store();
+        if (check && __syncthreads_or(bad)) {
 #pragma unroll 1
             for (int j = 0; j < E; j++) {
                 const int i = p0 + j * 32;
-                const K x = i < n ? (head ? src.template ldx<XF>(o + i) : src.ld(o + i)) : K(0);
+                const K x = i < n ? (head ? sg.src.template ldx<XF>(o + i) : sg.src.ld(o + i)) : K{};
                 const unsigned v = Rx<K>::dig(x, d);
                 unsigned mt = __ballot_sync(0xFFFFFFFFu, i < n);
 #pragma unroll
@@ -556,7 +681,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
                 __syncwarp();
                 if (i < n) {
                     if (r == 0) my[v] = old + __popc(mt);
-                    if (PS_IN(old + r, T, 52)) sk[old + r] = x;
+                    if (PS_IN(old + r, T, 52)) sk.st(old + r, x);
                 }
                 __syncwarp();
             }
@@ -564,6 +689,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
             store();
             __syncthreads();
         }
+        tile = after;
     }
 }
 

@@ -11,9 +11,10 @@ namespace ps {
 // Threads, keys per thread and CTAs per SM of a digit pass.  Large tiles spread
 // the fixed work of a tile (digit tables, look-back, barriers) over more keys;
 // sorts of few tiles want more of them at once.  Measured per sort: uint32,
-// 384 x 32 / 512 x 16 / 512 x 8: 2^30 keys 15.1 / 16.4 / 24.1 ms, 2^22 140 / 129 /
-// 147 us, 2^18 79 / 71 / 62 us; uint64, 256 x 24 / 512 x 16 / 512 x 8: 2^30 24.6 /
-// 26.0 / 33.2 ms, 2^20 136 / 137 / 138 us, 2^17 114 / 119 / 107 us.
+// 512 x 24 / 384 x 32 / 256 x 32 / 512 x 16: 2^28 keys 3.48 / 3.50 / 3.53 / 4.00
+// ms, 2^22 129 / 135 / 141 / 124 us, and 512 x 8 against 512 x 16 at 2^18 62 / 71
+// us; uint64, 384 x 24 / 256 x 32 / 512 x 16: 2^28 5.54 / 5.58 / 5.64 ms; records,
+// 384 x 16 / 256 x 24 / 512 x 12: 2^28 8.90 / 9.00 / 9.05 ms.
 template <int NT_, int E_, int CTAS_> struct RxShape {
     static constexpr int NT = NT_, E = E_, CTAS = CTAS_, T = NT_ * E_;
 };
@@ -21,13 +22,19 @@ template <typename K> struct RxCfg;
 template <> struct RxCfg<uint32_t> {
     using Small = RxShape<512, 8, 2>;
     using Mid = RxShape<512, 16, 2>;
-    using Large = RxShape<384, 32, 2>;
+    using Large = RxShape<512, 24, 2>;
     static constexpr int64_t small = int64_t(1) << 18, mid = int64_t(1) << 23;  // up to so many keys
 };
 template <> struct RxCfg<uint64_t> {
     using Small = RxShape<512, 8, 2>;
-    using Mid = RxShape<256, 24, 3>;
-    using Large = RxShape<256, 24, 3>;
+    using Mid = RxShape<384, 24, 2>;
+    using Large = RxShape<384, 24, 2>;
+    static constexpr int64_t small = int64_t(1) << 18, mid = int64_t(1) << 18;
+};
+template <> struct RxCfg<Rec> {
+    using Small = RxShape<512, 8, 2>;
+    using Mid = RxShape<384, 16, 2>;
+    using Large = RxShape<384, 16, 2>;
     static constexpr int64_t small = int64_t(1) << 18, mid = int64_t(1) << 18;
 };
 
@@ -171,7 +178,7 @@ template <typename K> struct Radix {
         A.nseg = y.nseg;
         A.R = y.R;
         A.ntiles = y.ntiles;
-        A.iptr = (K* const*)a.inst_ptrs;
+        A.iptr = std::is_same<K, Rec>::value ? nullptr : (K* const*)a.inst_ptrs;
         A.hist = (unsigned long long*)(ws + y.o_hist);
         A.plan = (RxPlan*)(ws + y.o_plan);
         A.done = (unsigned*)(ws + y.o_done);
@@ -196,10 +203,14 @@ template <typename K> struct Radix {
         const int rc = ws_alloc((void**)&ws, y.total, a.stream);
         if (rc != PS_OK) return rc;
         cudaError_t e;
-        switch (xf_of(a.dtype)) {
-        case 1: e = run_xf<1>(a, y, ws); break;
-        case 2: e = run_xf<2>(a, y, ws); break;
-        default: e = run_xf<0>(a, y, ws); break;
+        if constexpr (std::is_same<K, Rec>::value) {
+            e = run_xf<0>(a, y, ws);
+        } else {
+            switch (xf_of(a.dtype)) {
+            case 1: e = run_xf<1>(a, y, ws); break;
+            case 2: e = run_xf<2>(a, y, ws); break;
+            default: e = run_xf<0>(a, y, ws); break;
+            }
         }
         ws_free(ws, a.stream);
         return e == cudaSuccess ? PS_OK : fail_cuda(e);
