@@ -304,7 +304,7 @@ static int log_level()
     return lvl;
 }
 
-// Keys-only sorts whose blocks are the library's choice sort their input as
+// Sorts whose blocks are the library's choice sort their input as
 // one block, by radix (the result is the same whatever the blocks are, and
 // nothing is left to partition or merge), from this many keys on.  Measured,
 // tiles and multiway merges against radix: 2^17 int32 keys 72 / 74 us (below,
@@ -321,7 +321,7 @@ static bool free_params(const ps_params* p, const ps_trace* trace)
 }
 static bool radix_takes(const SortArgs& a)
 {
-    if (a.dtype < 0 || a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
+    if (a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
     const bool one = a.n_B == 1 && a.n_P == 1 && !a.trace && a.items == 0 && a.threads == 0;
     if (!a.free_blocks && !one) return false;
     if (a.n_inst != 1 || a.inst_ptrs || a.src_keys || a.dst_keys || a.inst_base) return false;
@@ -337,7 +337,8 @@ static int dispatch(SortArgs& a)
     int rc = PS_OK;
     const ShapeEntry* sh = shape_of(a.dtype, a.items, a.threads, &rc);
     if (rc != PS_OK) return rc;
-    if (radix_takes(a)) return tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
+    if (radix_takes(a))
+        return a.dtype < 0 ? run_radix_rec(a) : tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
     if (sh) return sh->run(a);
     switch (a.dtype) {
     case PS_I32: case PS_F32: case PS_U32: return run_sort_u32(a);
@@ -402,7 +403,7 @@ static size_t radix_bytes(int64_t n, int dtype)
     a.trace = nullptr;
     a.stream = nullptr;
     if (!radix_takes(a)) return 0;
-    return tune_family(dtype) == 0 ? radix_bytes_u32(a) : radix_bytes_u64(a);
+    return dtype < 0 ? radix_bytes_rec(a) : tune_family(dtype) == 0 ? radix_bytes_u32(a) : radix_bytes_u64(a);
 }
 
 size_t sort_ws_bytes(int64_t n, int dtype)
@@ -412,7 +413,7 @@ size_t sort_ws_bytes(int64_t n, int dtype)
     switch (dtype) {
     case PS_I32: case PS_F32: case PS_U32:
         return std::max(radix_bytes(n, dtype), ws_bytes_u32(n, r.n_blocks, r.n_parts));
-    case -1: return ws_bytes_rec(n, r.n_blocks, r.n_parts);
+    case -1: return std::max(radix_bytes(n, dtype), ws_bytes_rec(n, r.n_blocks, r.n_parts));
     default: return std::max(radix_bytes(n, dtype), ws_bytes_u64(n, r.n_blocks, r.n_parts));
     }
 }
@@ -1185,7 +1186,7 @@ int ps_debug_violation(uint64_t* out)
     if (!out) return PS_ERR_INVALID_ARG;
     unsigned long long v[4];
     int (*readers[])(unsigned long long*) = {viol_read_u32, viol_read_u64, viol_read_rec, viol_read_radix_u32,
-                                             viol_read_radix_u64};
+                                             viol_read_radix_u64, viol_read_radix_rec};
     int found = 0;
     for (int f = 0; f < (int)(sizeof(readers) / sizeof(readers[0])); f++) {
         int rc = readers[f](v);

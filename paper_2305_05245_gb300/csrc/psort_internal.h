@@ -99,6 +99,7 @@ int viol_read_u64(unsigned long long* out);
 int viol_read_rec(unsigned long long* out);
 int viol_read_radix_u32(unsigned long long* out);
 int viol_read_radix_u64(unsigned long long* out);
+int viol_read_radix_rec(unsigned long long* out);
 // Batched sort of the segments [off[i], off[i+1]) of keys (host offsets).
 // pinned (optional): page-locked host scratch of pinned_cap int64 for the
 // instance table; when given, the call does not wait for the stream.
@@ -132,6 +133,8 @@ constexpr int64_t SMALL_SEG = 1024;
 // the workspace it takes.
 int run_radix_u32(const SortArgs& a);
 int run_radix_u64(const SortArgs& a);
+int run_radix_rec(const SortArgs& a);
+size_t radix_bytes_rec(const SortArgs& a);
 size_t radix_bytes_u32(const SortArgs& a);
 size_t radix_bytes_u64(const SortArgs& a);
 // Workspace bytes of the sort a describes (batched instances included).

@@ -12,7 +12,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-T32, T64 = 384 * 32, 256 * 24  # keys per tile of a digit pass (large sorts; smaller ones: 4096, 8192)
+T32, T64 = 512 * 24, 384 * 24  # keys per tile of a digit pass (large sorts; smaller ones: 4096, 8192)
 MIN = 100000                   # smallest size the radix block sort takes
 
 
@@ -147,3 +147,41 @@ def test_fix_tile_edges(ps, ora, n):
     fix kernel's tiles of 4096 positions."""
     z = synth.splitmix64(n, n)
     check(ps, ora, ((z >> np.uint64(44)) << np.uint64(44)) | (z & np.uint64(255)))
+
+
+def check_records(ps, k, p, mode="exact"):
+    """Records against numpy's order by (key, payload)."""
+    import torch
+    tk = torch.from_numpy(k.view(np.int64).copy()).cuda()
+    tp = torch.from_numpy(p.view(np.int32).copy()).cuda()
+    ps.sort_pairs(tk, tp, mode)
+    torch.cuda.synchronize()
+    o = np.lexsort((p, k))
+    assert tk.cpu().numpy().view(np.uint64).tobytes() == k[o].tobytes()
+    assert tp.cpu().numpy().view(np.uint32).tobytes() == p[o].tobytes()
+
+
+@pytest.mark.parametrize("n", [MIN - 1, MIN, MIN + 1, 43 * 6144 - 1, 43 * 6144, 43 * 6144 + 1, 1000003])
+@pytest.mark.parametrize("kind", ["uniform", "index", "few", "few_index", "one_key", "all_equal"])
+def test_records(ps, n, kind):
+    """Payloads that are the input position, or random, or few; keys distinct,
+    few or all equal: passes over key bytes, payload bytes, both or none."""
+    z = synth.splitmix64(n, 2 * n)
+    k, p = z[:n].copy(), (z[n:] >> np.uint64(32)).astype(np.uint32)
+    if kind in ("index", "few_index"):
+        p = np.arange(n, dtype=np.uint32)
+    if kind in ("few", "few_index"):
+        k = z[:16][(z[:n] >> np.uint64(60)).astype(np.int64)]
+    if kind == "one_key":
+        k[:] = k[0]
+    if kind == "all_equal":
+        k[:], p[:] = k[0], p[0]
+    check_records(ps, k, p, "regular" if n & 1 else "exact")
+
+
+@pytest.mark.parametrize("sizes,top", [((2, 63, 64, 65, 66, 129), 5), ((700, 300, 3), 4), ((300, 300), 7)])
+def test_record_runs_of_equal_leading_bytes(ps, sizes, top):
+    n = 1 << 20
+    k = clustered(n, sizes, top, seed=top)
+    k[5::1000] = k[5]  # some equal keys, ordered by payload
+    check_records(ps, k, (synth.splitmix64(9, n) >> np.uint64(40)).astype(np.uint32))
