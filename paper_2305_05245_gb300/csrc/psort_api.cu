@@ -321,6 +321,7 @@ static bool free_params(const ps_params* p, const ps_trace* trace)
 }
 static bool radix_takes(const SortArgs& a)
 {
+    if (a.radix) return true;
     if (a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
     const bool one = a.n_B == 1 && a.n_P == 1 && !a.trace && a.items == 0 && a.threads == 0;
     if (!a.free_blocks && !one) return false;
@@ -421,8 +422,9 @@ size_t sort_ws_bytes(int64_t n, int dtype)
 // Batched sorts.  A batch plan bins the segments [off[i], off[i+1]) by length
 // and fixes each bin's parameters and its part of the instance table (per
 // bin: all starts, then all lengths); launching a plan queues one persistent
-// launch for the segments of at most one tile (both short bins together) and
-// one multi-instance pipeline per longer bin.
+// launch for the segments of at most one tile (both short bins together), one
+// multi-instance pipeline per longer bin and one radix sort of all segments
+// beyond those.
 struct BatchBin {
     size_t at;                // offset of the bin's starts in the instance table
     int64_t cnt, nmax, nsum;  // instances, longest, total keys
@@ -430,6 +432,7 @@ struct BatchBin {
     int items, threads;       // launch shape (0, 0: automatic)
     bool small;               // at most SMALL_SEG keys each (one warp each)
     bool front;               // at most one tile each: sorted by the persistent front kernel
+    bool radix;               // longer than batch_radix_min: every segment one block, sorted by radix
 };
 struct BatchPlan {
     int dtype = 0, mode = 0;
@@ -439,6 +442,20 @@ struct BatchPlan {
     std::vector<BatchBin> bins;
     size_t counter_at = 0;       // the front kernel's work counter (last table slot), if a front bin exists
 };
+
+// Segments longer than this sort as one block each, by radix, all of them
+// together (the launches no longer depend on the number of size bins).
+// Measured on 2^26 keys in segments of 1.4 * 2^k, tiles and merges / radix:
+// int32, k = 17: 1.21 / 1.35 ms, 18: 1.54 / 1.35, 21: 2.04 / 1.37; int64, k = 16:
+// 2.02 / 2.07, 17: 2.12 / 2.04, 21: 3.35 / 2.09.  (Up to these lengths one merge
+// pass after the tiles finishes a segment.)
+#ifndef PS_BATCH_RADIX32
+#define PS_BATCH_RADIX32 262144
+#endif
+#ifndef PS_BATCH_RADIX64
+#define PS_BATCH_RADIX64 131072
+#endif
+static int64_t batch_radix_min(int dtype) { return tune_family(dtype) == 0 ? PS_BATCH_RADIX32 : PS_BATCH_RADIX64; }
 
 // own (optional): one device pointer per segment; segment i then lives in its
 // own buffer, and off only lays the segments out for the workspace.
@@ -458,15 +475,17 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
     bp->table.clear();
     bp->bins.clear();
     // bins: 0 = at most SMALL_SEG keys (a warp each); 1 = fits one tile (a
-    // CTA each); b >= 2 = lengths in (T*2^(b-2), T*2^(b-1)]
-    const int64_t tile = 8192;
-    std::vector<std::vector<int64_t>> bins(48);
+    // CTA each); b >= 2 = lengths in (T*2^(b-2), T*2^(b-1)], up to
+    // batch_radix_min keys; the last bin = all longer ones
+    const int64_t tile = 8192, rmin = std::max(tile, batch_radix_min(dtype));
+    std::vector<std::vector<int64_t>> bins(49);
     for (int64_t i = 0; i < n_segs; i++) {
         const int64_t len = off[i + 1] - off[i];
         if (len <= 1) continue;
         int b = 1;
         if (len <= SMALL_SEG) b = 0;
         while (len > (tile << (b - 1)) && b > 0) b++;
+        if (!force && len > rmin) b = (int)bins.size() - 1;
         bins[b].push_back(i);
     }
     for (size_t b = 0; b < bins.size(); b++) {
@@ -486,8 +505,9 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
             for (int64_t i : bins[b]) bp->table.push_back((int64_t)(uintptr_t)(*own)[(size_t)i]);
         ps_params r;
         memset(&r, 0, sizeof(r));
-        if (b <= 1) {
-            r.n_blocks = r.n_parts = 1;  // one tile: the block sort is the whole sort
+        bb.radix = b + 1 == bins.size();
+        if (b <= 1 || bb.radix) {
+            r.n_blocks = r.n_parts = 1;  // the block sort is the whole sort
         } else if (force) {
             r = *force;
         } else {
@@ -495,8 +515,8 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         }
         bb.n_B = r.n_blocks;
         bb.n_P = r.n_parts;
-        bb.items = b <= 1 ? 0 : r.items_per_thread;
-        bb.threads = b <= 1 ? 0 : r.block_threads;
+        bb.items = r.items_per_thread;
+        bb.threads = r.block_threads;
         bb.small = b == 0;
         bb.front = b <= 1;
         bp->bins.push_back(bb);
@@ -525,13 +545,16 @@ static SortArgs batch_bin_args(const BatchPlan& bp, const BatchBin& bb, const in
     a.threads = bb.threads;
     a.trace = nullptr;
     a.stream = s;
-    a.inst_base = dev_table + bb.at;
-    a.inst_n = dev_table + bb.at + bb.cnt;
+    // (sizing only, without a device table: any address that is not null marks a batch)
+    const int64_t* table = dev_table ? dev_table : (const int64_t*)sizeof(int64_t);
+    a.inst_base = table + bb.at;
+    a.inst_n = table + bb.at + bb.cnt;
     if (bp.own && dev_table) a.inst_ptrs = (void* const*)(dev_table + bb.at + 2 * bb.cnt);
     a.n_inst = bb.cnt;
     a.n_max = bb.nmax;
     a.n_sum = bb.nsum;
     a.extent = bp.extent;
+    a.radix = bb.radix;
     return a;
 }
 
@@ -567,7 +590,9 @@ static int batch_launch(const BatchPlan& bp, const int64_t* dev_table, void* key
     for (size_t i = 0; i < bp.bins.size() && rc == PS_OK; i++) {
         if (bp.bins[i].front) continue;
         SortArgs a = batch_bin_args(bp, bp.bins[i], dev_table, keys, s);
-        if (ws) {
+        if (ws && a.radix) {
+            rc = narrow ? run_radix_u32(a, ws, cap) : run_radix_u64(a, ws, cap);
+        } else if (ws) {
             const ShapeEntry* sh = shape_of(a.dtype, a.items, a.threads, &rc);
             if (rc == PS_OK)
                 rc = sh ? sh->run_on(a, ws, cap) : narrow ? run_sort_u32_on(a, ws, cap) : run_sort_u64_on(a, ws, cap);
@@ -963,6 +988,10 @@ int ps_batch_plan_create(const int64_t* host_seg_offsets, int64_t n_segs, int dt
         if (bb.front) continue;
         SortArgs a = batch_bin_args(p->plan, bb, nullptr, nullptr, nullptr);
         int src = PS_OK;
+        if (bb.radix) {
+            ws = std::max(ws, narrow_dtype(dtype) ? radix_bytes_u32(a) : radix_bytes_u64(a));
+            continue;
+        }
         const ShapeEntry* sh = shape_of(dtype, a.items, a.threads, &src);
         if (src != PS_OK && rc == PS_OK) rc = src;
         ws = std::max(ws, sh ? sh->ws(a) : narrow_dtype(dtype) ? ws_bytes_args_u32(a) : ws_bytes_args_u64(a));

@@ -64,6 +64,8 @@ struct SortArgs {
     // n_B and n_P are the library's choice and no intermediates are asked for:
     // the block sort may take the whole input as one block (radix_takes).
     bool free_blocks = false;
+    // Several instances, each sorted as one block by radix.
+    bool radix = false;
 };
 
 // Workspace from the library's stream-ordered pool.
@@ -130,9 +132,9 @@ int run_front_u32(const SortArgs* t, const SortArgs* sm, unsigned long long* nex
 int run_front_u64(const SortArgs* t, const SortArgs* sm, unsigned long long* next);
 constexpr int64_t SMALL_SEG = 1024;
 // The radix block sort (psort_radix.cuh) of every instance as one block, and
-// the workspace it takes.
-int run_radix_u32(const SortArgs& a);
-int run_radix_u64(const SortArgs& a);
+// the workspace it takes (ws: on a caller's workspace of cap bytes, allocating nothing).
+int run_radix_u32(const SortArgs& a, char* ws = nullptr, size_t cap = 0);
+int run_radix_u64(const SortArgs& a, char* ws = nullptr, size_t cap = 0);
 int run_radix_rec(const SortArgs& a);
 size_t radix_bytes_rec(const SortArgs& a);
 size_t radix_bytes_u32(const SortArgs& a);

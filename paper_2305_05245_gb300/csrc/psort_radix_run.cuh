@@ -45,33 +45,32 @@ template <typename K> struct Radix {
 
     struct Layout {
         int T;  // keys per tile
-        int64_t nseg, R, ntiles, chunk, RC;
-        bool wide;  // 64-bit look-back words
-        int S;      // sampled keys (0: every digit is sorted)
-        size_t o_nflag, o_hits, o_tab, o_flags;
-        size_t o_hist, o_done, o_ticket, o_lb0, zero_bytes, o_lb1, o_plan, o_data, total;
+        int64_t nseg, tiles, chunk, chunks, fixes, S;  // (several segments: upper bounds)
+        bool wide;     // 64-bit look-back words
+        size_t o_hist, o_done, o_ticket, o_misc, o_hits, o_tab, o_flags, o_lb0, zero_bytes, o_lb1, o_plan, o_at, o_tile,
+            o_chunk, o_fix, o_data, total;
     };
     static Layout layout(const SortArgs& a)
     {
         Layout y;
-        const int64_t nmax = a.inst_base ? a.n_max : a.n, extent = a.inst_base ? a.extent : a.n;
+        const bool multi = a.inst_base != nullptr;
+        const int64_t nmax = multi ? a.n_max : a.n, nsum = multi ? a.n_sum : a.n, extent = multi ? a.extent : a.n;
         y.nseg = a.n_inst;
-        y.T = nmax <= C::small ? C::Small::T : nmax <= C::mid ? C::Mid::T : C::Large::T;
-        y.R = (nmax + y.T - 1) / y.T;
-        y.ntiles = y.nseg * y.R;
+        const int64_t extra = y.nseg == 1 ? 0 : y.nseg;
+        auto parts = [&](int64_t u) { return y.nseg == 1 ? (nsum + u - 1) / u : nsum / u + extra; };
+        y.T = nsum <= C::small ? C::Small::T : nsum <= C::mid ? C::Mid::T : C::Large::T;
+        y.tiles = parts(y.T);
         y.wide = nmax >= (int64_t(1) << 30);
-        // counting chunks: about four per SM, 4096 to 2^20 keys
-        const int64_t want = (nmax * y.nseg) / (152 * 4);
-        y.chunk = std::min<int64_t>(int64_t(1) << 20, std::max<int64_t>(4096, (want + 4095) / 4096 * 4096));
-        y.RC = (nmax + y.chunk - 1) / y.chunk;
-        // sqrt(8 n) sampled keys: runs of about one key out of order then give
-        // two hits, the least that tells them from none
-        y.S = 0;
-        if (D > 4 && y.nseg == 1) {
-            y.S = 256;
-            while (y.S < RX_SAMPLE_MAX && (int64_t)y.S * y.S < 8 * nmax) y.S *= 2;
-        }
-        const size_t lb = align256((size_t)y.ntiles * 256 * (y.wide ? 8 : 4));
+        // counting chunks: about four per SM, 4096 to 2^20 keys (2^16 for several segments)
+        const int64_t want = nsum / (152 * 4);
+        y.chunk = std::min<int64_t>(int64_t(1) << (extra ? 16 : 20), std::max<int64_t>(4096, (want + 4095) / 4096 * 4096));
+        y.chunks = parts(y.chunk);
+        const bool sampled = D > 4;
+        y.fixes = sampled ? parts(FT) : 0;
+        y.S = sampled ? rx_samples(nmax) : 0;
+        // hash tables: S < 2 sqrt(8 n), or 128, keys of each segment
+        const double many = y.nseg == 1 ? (double)y.S : 2.0 * std::sqrt(8.0 * (double)y.nseg * (double)nsum) + 128.0 * y.nseg;
+        const size_t lb = align256((size_t)y.tiles * 256 * (y.wide ? 8 : 4));
         size_t o = 0;
         y.o_hist = o;
         o += align256((size_t)y.nseg * D * 256 * 8);
@@ -79,13 +78,14 @@ template <typename K> struct Radix {
         o += align256((size_t)y.nseg * 4);
         y.o_ticket = o;
         o += 256;
-        y.o_nflag = o;
-        y.o_hits = o + 8;
+        y.o_misc = o;  // most passes, flagged tiles, totals
         o += 256;
+        y.o_hits = o;
+        o += align256(sampled ? (size_t)y.nseg * RX_TRY * 4 : 0);
         y.o_tab = o;
-        o += align256((size_t)(y.S ? D : 0) * 2 * y.S * 4);
+        o += align256(sampled ? (size_t)many * RX_TRY * 2 * 4 : 0);
         y.o_flags = o;
-        o += align256(y.S ? (size_t)(nmax + FT - 1) / FT : 0);
+        o += align256((size_t)y.fixes);
         y.o_lb0 = o;
         o += lb;
         y.zero_bytes = o;  // everything up to here starts as zeros
@@ -93,6 +93,14 @@ template <typename K> struct Radix {
         o += lb;
         y.o_plan = o;
         o += align256((size_t)y.nseg * sizeof(RxPlan));
+        y.o_at = o;
+        o += align256((size_t)extra * sizeof(RxSegAt));
+        y.o_tile = o;
+        o += align256(extra ? (size_t)y.tiles * 4 : 0);
+        y.o_chunk = o;
+        o += align256(extra ? (size_t)y.chunks * 4 : 0);
+        y.o_fix = o;
+        o += align256(extra ? (size_t)y.fixes * 4 : 0);
         y.o_data = o;
         o += align256((size_t)extent * GStore<K>::bytes + 256);
         y.total = o;
@@ -106,7 +114,7 @@ template <typename K> struct Radix {
         constexpr size_t sb = rx_smem<K, CT, SH::NT, SH::E>();
         cudaError_t e = smem_attr(fp, sb);
         if (e != cudaSuccess) return e;
-        const unsigned grid = (unsigned)std::min<int64_t>(y.ntiles, (int64_t)grid_sms * SH::CTAS);
+        const unsigned grid = (unsigned)std::min<int64_t>(y.tiles, (int64_t)grid_sms * SH::CTAS);
         CT* l0 = (CT*)(ws + y.o_lb0);
         CT* l1 = (CT*)(ws + y.o_lb1);
         for (int i = 0; i < D; i++) {
@@ -121,19 +129,27 @@ template <typename K> struct Radix {
     {
         cudaStream_t s = a.stream;
         cudaError_t e;
+        if (y.nseg > 1) {
+            ProfScope ps_("radix_segments", s);
+            k_rx_at<1024, K><<<1, 1024, 0, s>>>(A);
+            k_rx_lists<K><<<(unsigned)((y.nseg + 7) / 8), 256, 0, s>>>(A);
+        }
+        if constexpr (std::is_same<K, Rec>::value) {
+            ProfScope ps_("radix_descents", s);
+            const int64_t g = (A.in.n0 + 4095) / 4096;
+            k_rx_descents<512><<<(unsigned)std::min<int64_t>(g, grid_sms * 4), 512, 0, s>>>(A.first.p, A.in.n0, A.descents);
+        }
         if constexpr (D > 4) {
-            if (y.S) {
-                ProfScope ps_("radix_sample", s);
-                k_rx_sample<K, XF><<<dim3((unsigned)((y.S + 127) / 128), D - 2), 128, 0, s>>>(
-                    A, (unsigned*)(ws + y.o_tab));
-            }
+            ProfScope ps_("radix_sample", s);
+            const unsigned z = (unsigned)std::min<int64_t>((y.S + 127) / 128, y.nseg == 1 ? 512 : 16);
+            k_rx_sample<K, XF><<<dim3((unsigned)y.nseg, RX_TRY, z), 128, 0, s>>>(A);
         }
         auto fc = k_rx_count<CNT, G, K, XF>;
         const size_t cb = (size_t)G * 4096 * 4;
         if ((e = smem_attr(fc, cb)) != cudaSuccess) return e;
         {
             ProfScope ps_("radix_count", s);
-            fc<<<dim3((unsigned)(y.nseg * y.RC), D / G), CNT, cb, s>>>(A);
+            fc<<<dim3((unsigned)y.chunks, D / G), CNT, cb, s>>>(A);
         }
         if (std::is_same<CT, uint32_t>::value && y.T == C::Small::T)
             e = digits<XF, uint32_t, typename C::Small>(y, A, ws, grid_sms, s);
@@ -143,17 +159,15 @@ template <typename K> struct Radix {
             e = digits<XF, CT, typename C::Large>(y, A, ws, grid_sms, s);
         if (e != cudaSuccess) return e;
         if constexpr (D > 4) {
-            if (y.S) {
-                {
-                    auto ff = k_rx_fix<K, XF>;
-                    constexpr size_t fb = sizeof(K) * (FT + 2 * FL + 1) + 2 * (FT / 2 + 2);
-                    if ((e = smem_attr(ff, fb)) != cudaSuccess) return e;
-                    ProfScope ps_("radix_fix", s);
-                    ff<<<(unsigned)((A.in.n0 + FT - 1) / FT), FN, fb, s>>>(A);
-                }
-                ProfScope ps_("radix_long", s);
-                k_rx_long<K, XF><<<(unsigned)grid_sms, 512, 0, s>>>(A);
+            {
+                auto ff = k_rx_fix<K, XF>;
+                constexpr size_t fb = sizeof(K) * (FT + 2 * FL + 1) + 2 * (FT / 2 + 2);
+                if ((e = smem_attr(ff, fb)) != cudaSuccess) return e;
+                ProfScope ps_("radix_fix", s);
+                ff<<<(unsigned)y.fixes, FN, fb, s>>>(A);
             }
+            ProfScope ps_("radix_long", s);
+            k_rx_long<K, XF><<<(unsigned)grid_sms, 512, 0, s>>>(A);
         }
         return cudaGetLastError();
     }
@@ -176,18 +190,26 @@ template <typename K> struct Radix {
         A.in.n0 = a.n;
         A.n_B = 1;
         A.nseg = y.nseg;
-        A.R = y.R;
-        A.ntiles = y.ntiles;
         A.iptr = std::is_same<K, Rec>::value ? nullptr : (K* const*)a.inst_ptrs;
         A.hist = (unsigned long long*)(ws + y.o_hist);
         A.plan = (RxPlan*)(ws + y.o_plan);
         A.done = (unsigned*)(ws + y.o_done);
         A.ticket = (unsigned*)(ws + y.o_ticket);
+        A.T = y.T;
         A.chunk = y.chunk;
-        A.RC = y.RC;
-        A.sample = y.S;
+        A.sampled = D > 4;
+        A.one = RxSegAt{0, 0, 0, (int)y.S, rx_lead(a.inst_base ? a.n_max : a.n), 0};
+        A.ntiles1 = y.tiles;
+        A.at = (RxSegAt*)(ws + y.o_at);
+        A.tile_seg = (int*)(ws + y.o_tile);
+        A.chunk_seg = (int*)(ws + y.o_chunk);
+        A.fix_seg = (int*)(ws + y.o_fix);
+        A.maxpass = (int*)(ws + y.o_misc);
+        A.nflag = (unsigned*)(ws + y.o_misc + 4);
+        A.total = (int64_t*)(ws + y.o_misc + 8);
+        A.descents = (unsigned*)(ws + y.o_misc + 32);
         A.hits = (unsigned*)(ws + y.o_hits);
-        A.nflag = (unsigned*)(ws + y.o_nflag);
+        A.tab = (unsigned*)(ws + y.o_tab);
         A.flags = (uint8_t*)(ws + y.o_flags);
         A.keep = a.keep_order_keys;
         // a sort between two buffers, or one that leaves order keys, moves
@@ -196,12 +218,19 @@ template <typename K> struct Radix {
         return y.wide ? passes<XF, uint64_t>(a, y, A, ws, sms) : passes<XF, uint32_t>(a, y, A, ws, sms);
     }
 
-    static int run(const SortArgs& a)
+    // ws == nullptr: the workspace comes from the pool; otherwise cap bytes at
+    // ws are used and nothing is allocated (PS_ERR_INVALID_ARG if too few).
+    static int run(const SortArgs& a, char* ws = nullptr, size_t cap = 0)
     {
         const Layout y = layout(a);
-        char* ws = nullptr;
-        const int rc = ws_alloc((void**)&ws, y.total, a.stream);
-        if (rc != PS_OK) return rc;
+        char* own = nullptr;
+        if (ws) {
+            if (y.total > cap) return PS_ERR_INVALID_ARG;
+        } else {
+            const int rc = ws_alloc((void**)&own, y.total, a.stream);
+            if (rc != PS_OK) return rc;
+            ws = own;
+        }
         cudaError_t e;
         if constexpr (std::is_same<K, Rec>::value) {
             e = run_xf<0>(a, y, ws);
@@ -212,7 +241,7 @@ template <typename K> struct Radix {
             default: e = run_xf<0>(a, y, ws); break;
             }
         }
-        ws_free(ws, a.stream);
+        if (own) ws_free(own, a.stream);
         return e == cudaSuccess ? PS_OK : fail_cuda(e);
     }
 };

@@ -185,3 +185,69 @@ def test_record_runs_of_equal_leading_bytes(ps, sizes, top):
     k = clustered(n, sizes, top, seed=top)
     k[5::1000] = k[5]  # some equal keys, ordered by payload
     check_records(ps, k, (synth.splitmix64(9, n) >> np.uint64(40)).astype(np.uint32))
+
+
+def check_batch(ps, ora, lens, dtype, dist, how, seed=1):
+    """Every segment of a batch against the plain definition; `how`: the
+    batched call, a plan run twice, or the sort server (own buffers)."""
+    import torch
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    host = np.concatenate([synth.keys(int(n), dtype, dist, seed=synth.seed_for(seed, i)) for i, n in enumerate(lens)])
+    want = np.concatenate([ora.reference_sort(host[a:b]) for a, b in zip(off[:-1], off[1:])])
+    x = torch.from_numpy(host.copy()).cuda()
+    if how == "call":
+        ps.sort_batch(x, torch.from_numpy(off).cuda())
+    elif how == "plan":
+        plan = ps.BatchPlan(off, getattr(torch, dtype))
+        plan.run(x)
+        x.copy_(torch.from_numpy(host))
+        plan.run(x)
+        torch.cuda.synchronize()
+        plan.close()
+    else:
+        parts = [x[int(a):int(b)].clone() for a, b in zip(off[:-1], off[1:])]
+        torch.cuda.synchronize()
+        srv = ps.Server(budget_bytes=4 << 30)
+        left = {srv.submit(p) for p in parts}
+        while left:
+            for rid, status in srv.poll():
+                assert status == 0
+                left.discard(rid)
+        srv.close()
+        x = torch.cat(parts)
+    torch.cuda.synchronize()
+    assert x.cpu().numpy().tobytes() == want.tobytes()
+
+
+L32, L64 = 1 << 18, 1 << 17  # segments longer than this take the radix block sort
+
+
+@pytest.mark.parametrize("how", ["call", "plan", "server"])
+@pytest.mark.parametrize("dtype,edge", [("int32", L32), ("float32", L32), ("int64", L64), ("float64", L64)])
+@pytest.mark.parametrize("dist", ["uniform", "few_unique", "sorted"])
+def test_batch_segments(ps, ora, how, dtype, edge, dist):
+    """Segments on both sides of the shortest radix length, of one and several
+    tiles more, empty and tiny ones between; their digits (and the digits left
+    out of 64-bit keys) are chosen segment by segment."""
+    lens = [edge + 1, 0, edge, 3 * T32 * 8 + 5, 1, 700, edge + 4096 * 3, 5000, 2 * edge - 1]
+    check_batch(ps, ora, lens, dtype, dist, how)
+
+
+@pytest.mark.parametrize("dtype,n", [("int32", L32 + 5), ("int64", L64 + 5), ("int32", 20000)])
+@pytest.mark.parametrize("how", ["call", "plan"])
+def test_batch_of_one_long_segment(ps, ora, how, dtype, n):
+    """No short segments: the instance table starts with the long bin."""
+    check_batch(ps, ora, [n], dtype, "uniform", how)
+
+
+def test_batch_long_runs_per_segment(ps):
+    """64-bit segments with runs that leading bytes do not tell apart, longer
+    than the fix kernel ranks, in segments of their own buffers and shared ones."""
+    import torch
+    segs = [clustered(200003, (300, 70, 2), 5, 1), clustered(150001, (150001,), 4, 2), clustered(300000, (65, 64, 500), 6, 3)]
+    off = np.concatenate([[0], np.cumsum([s.size for s in segs])]).astype(np.int64)
+    want = np.concatenate([np.sort(s) for s in segs])
+    x = torch.from_numpy(np.concatenate(segs).view(np.int64)).cuda().view(torch.uint64)
+    ps.sort_batch(x, torch.from_numpy(off).cuda())
+    torch.cuda.synchronize()
+    assert x.view(torch.int64).cpu().numpy().view(np.uint64).tobytes() == want.tobytes()
