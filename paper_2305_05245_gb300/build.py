@@ -18,7 +18,7 @@ BUILD = os.path.join(HERE, "_build")
 
 SOURCES = ["psort_u32.cu", "psort_u64.cu", "psort_rec.cu", "psort_api.cu", "psort_noalloc.cu",
            "psort_server.cu", "psort_struct.cu", "psort_shapes.cu", "psort_radix32.cu", "psort_radix64.cu",
-           "psort_radixrec.cu"]
+           "psort_radixrec.cu", "psort_cluster32.cu", "psort_cluster64.cu", "psort_clusterrec.cu"]
 # Launch shapes (key bits, items per thread, threads per CTA) compiled besides
 # the automatic one, each from psort_shape.cu into an object of its own; the
 # 64-bit (32, 256) shape is the automatic one and is not repeated.

@@ -304,29 +304,32 @@ static int log_level()
     return lvl;
 }
 
-// Sorts whose blocks are the library's choice sort their input as
-// one block, by radix (the result is the same whatever the blocks are, and
-// nothing is left to partition or merge), from this many keys on.  Measured,
-// tiles and multiway merges against radix: 2^17 int32 keys 72 / 74 us (below,
-// the launches of the digit passes cost more than the merges), 3,000,001
-// float32 251 / 102 us, 2^26 int32 1.90 / 1.13 ms, 2^30 int64 54.7 / 47.4 ms
-// (a copy of the keys included in the last three).
-#ifndef PS_RADIX_MIN
-#define PS_RADIX_MIN 100000
-#endif
+// Sorts whose blocks are the library's choice sort their input as one block (the
+// result is the same whatever the blocks are, and nothing is left to partition
+// or merge): short ones by one thread-block cluster (cluster_takes), longer ones
+// by radix.  Measured, tiles and multiway merges against these:
+// 3,000,001 float32 251 / 97 us, 2^26 int32 1.90 / 1.01 ms, 2^30 int64 54.7 / 25.9
+// ms, 2^28 records 25.8 / 10.1 ms (a copy of the keys included).
 static bool free_params(const ps_params* p, const ps_trace* trace)
 {
     if (trace) return false;
     return !p || (p->n_blocks <= 0 && p->n_parts <= 0 && p->items_per_thread == 0 && p->block_threads == 0);
 }
+static bool one_block(const SortArgs& a)
+{
+    if (a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
+    const bool one = a.n_B == 1 && a.n_P == 1 && !a.trace && a.items == 0 && a.threads == 0;
+    return (a.free_blocks || one) && !a.inst_base;
+}
+static int64_t cluster_max(int dtype) { return dtype >= 0 && tune_family(dtype) == 0 ? CLUSTER_MAX32 : CLUSTER_MAX64; }
+static bool cluster_takes(const SortArgs& a)
+{
+    return one_block(a) && !a.keep_order_keys && a.n <= cluster_max(a.dtype);
+}
 static bool radix_takes(const SortArgs& a)
 {
     if (a.radix) return true;
-    if (a.merge_variant != PS_MERGE_TREE || a.presorted) return false;
-    const bool one = a.n_B == 1 && a.n_P == 1 && !a.trace && a.items == 0 && a.threads == 0;
-    if (!a.free_blocks && !one) return false;
-    if (a.n_inst != 1 || a.inst_ptrs || a.src_keys || a.dst_keys || a.inst_base) return false;
-    return a.n >= PS_RADIX_MIN;
+    return one_block(a) && !a.src_keys && !a.dst_keys && a.n > cluster_max(a.dtype);
 }
 
 static int dispatch(SortArgs& a)
@@ -338,6 +341,8 @@ static int dispatch(SortArgs& a)
     int rc = PS_OK;
     const ShapeEntry* sh = shape_of(a.dtype, a.items, a.threads, &rc);
     if (rc != PS_OK) return rc;
+    if (cluster_takes(a))
+        return a.dtype < 0 ? run_cluster_rec(a) : tune_family(a.dtype) == 0 ? run_cluster_u32(a) : run_cluster_u64(a);
     if (radix_takes(a))
         return a.dtype < 0 ? run_radix_rec(a) : tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
     if (sh) return sh->run(a);

@@ -1,0 +1,79 @@
+// psort_cluster_run.cuh -- host side of the one-launch sorts: shape by size.
+#pragma once
+
+#include "psort_cluster.cuh"
+#include "psort_pipeline.cuh"
+
+namespace ps {
+
+template <typename K> struct ClusterSort {
+    static constexpr int TW = Cfg<K>::TW;  // warp-shuffle levels of the tile sort
+    static constexpr int EMAX = sizeof(K) == 4 ? 16 : 8;
+    static constexpr int64_t MAX = int64_t(16) * 1024 * EMAX;  // longest instance
+
+    template <int NT, int E, int XF, int CS> static cudaError_t launch(const SortArgs& a, const Inst& in, int64_t nmax)
+    {
+        using SB = typename TileBuf<K, E>::type;
+        auto f = k_cluster_sort<NT, E, K, XF, TW, CS>;
+        const size_t sm = SB::bytes(NT * E) * (CS > 1 ? 2 : 1) + 64;
+        cudaError_t e = smem_attr(f, sm, CS > 8);
+        if (e != cudaSuccess) return e;
+        const int share = (int)(((nmax + CS - 1) / CS + E - 1) / E * E);
+        const GBuf<K> user = gbuf_user<K>(a);
+        const GBuf<K> src = gbuf_ext<K>(a.src_keys, user), dst = gbuf_ext<K>(a.dst_keys, user);
+        K* const* own = nullptr;
+        if constexpr (sizeof(K) <= 8) own = (K* const*)a.inst_ptrs;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(a.n_inst * CS));
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = a.stream;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = CS;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = CS > 1 ? 1 : 0;
+        ProfScope ps_("cluster_sort", a.stream);
+        return cudaLaunchKernelEx(&cfg, f, src, dst, in, share, own);
+    }
+
+    // Small shapes first: one CTA while a tile holds the keys, then clusters of 4
+    // and 16 (more, shorter shares sort sooner: 16384 keys in 4 x 4096, not 2 x 8192).
+    template <int XF> static cudaError_t run_xf(const SortArgs& a, const Inst& in, int64_t n)
+    {
+        if (n <= 1024) return launch<128, 8, XF, 1>(a, in, n);
+        if (n <= 2048) return launch<256, 8, XF, 1>(a, in, n);
+        if (n <= 4096) return launch<1024, 4, XF, 1>(a, in, n);
+        if (n <= 8192) return launch<1024, 8, XF, 1>(a, in, n);
+        if (n <= 16384) return launch<1024, 4, XF, 4>(a, in, n);
+        if (n <= 65536) return launch<1024, 4, XF, 16>(a, in, n);
+        if (n <= 131072) return launch<1024, 8, XF, 16>(a, in, n);
+        return launch<1024, EMAX, XF, 16>(a, in, n);
+    }
+
+    // One launch sorts every instance of a (at most MAX keys each).
+    static int run(const SortArgs& a)
+    {
+        Inst in;
+        in.base = a.inst_base;
+        in.n = a.inst_n;
+        in.count = a.n_inst;
+        in.n0 = a.n;
+        const int64_t n = a.inst_base ? a.n_max : a.n;
+        if (n > MAX) return PS_ERR_INVALID_ARG;
+        cudaError_t e;
+        if constexpr (sizeof(K) > 8) {
+            e = run_xf<0>(a, in, n);
+        } else {
+            switch (xf_of(a.dtype)) {
+            case 1: e = run_xf<1>(a, in, n); break;
+            case 2: e = run_xf<2>(a, in, n); break;
+            default: e = run_xf<0>(a, in, n); break;
+            }
+        }
+        return e == cudaSuccess ? PS_OK : fail_cuda(e);
+    }
+};
+
+}  // namespace ps

@@ -298,7 +298,8 @@ inline SmemAttrCache& smem_attr_cache()
     static SmemAttrCache c;
     return c;
 }
-template <typename KF> static cudaError_t smem_attr(KF* f, size_t bytes)
+// wide_cluster: the kernel is also launched in clusters of more than 8 CTAs.
+template <typename KF> static cudaError_t smem_attr(KF* f, size_t bytes, bool wide_cluster = false)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -313,6 +314,7 @@ template <typename KF> static cudaError_t smem_attr(KF* f, size_t bytes)
             return e;
         }
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && wide_cluster) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) c.set.push_back({(const void*)f, dev, bytes});
     return e;
 }

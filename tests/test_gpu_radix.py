@@ -13,7 +13,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 T32, T64 = 512 * 24, 384 * 24  # keys per tile of a digit pass (large sorts; smaller ones: 4096, 8192)
-MIN = 100000                   # smallest size the radix block sort takes
+MIN = 131073                   # smallest size the radix block sort takes (32-bit keys: 262145)
 
 
 @pytest.fixture(scope="module")
@@ -42,8 +42,8 @@ def check(ps, ora, host, mode="exact", offset=0, **kw):
     assert not buf[:offset].any() and not buf[offset + host.size:].any()
 
 
-SIZES = [MIN - 1, MIN, MIN + 1, 683 * T32 - 1, 683 * T32, 683 * T32 + 1, 43 * T64 - 1, 43 * T64,
-         43 * T64 + 1, 26 * 4096 + 1, 1 << 18, (1 << 18) + 1, 1 << 20, (1 << 23) + 1,
+SIZES = [MIN, MIN + 1, 683 * T32 - 1, 683 * T32, 683 * T32 + 1, 43 * T64 - 1, 43 * T64,
+         43 * T64 + 1, 38 * 4096 + 1, 1 << 18, (1 << 18) + 1, 1 << 20, (1 << 23) + 1,
          3000017]
 
 
@@ -66,7 +66,7 @@ def test_distributions(ps, ora, dtype, dist):
 def test_varying_bytes(ps, ora, dtype, bytes_):
     """Only the named bytes of the keys vary: none to three passes have work."""
     width = np.dtype(dtype).itemsize
-    z = synth.splitmix64(7, 250001)
+    z = synth.splitmix64(7, 270001)
     u = np.full(z.size, 0x0123456789ABCDEF, dtype=np.uint64)
     for b in bytes_:
         s = np.uint64(8 * (b % width))
@@ -77,7 +77,7 @@ def test_varying_bytes(ps, ora, dtype, bytes_):
 
 @pytest.mark.parametrize("dtype", ["float32", "float64"])
 def test_float_specials(ps, ora, dtype):
-    x = synth.keys(200001, dtype, "gaussian", seed=5)
+    x = synth.keys(270001, dtype, "gaussian", seed=5)
     info = np.finfo(dtype)
     sp = np.array([0.0, -0.0, np.inf, -np.inf, info.max, info.min, info.tiny, -info.tiny,
                    info.smallest_subnormal, -info.smallest_subnormal], dtype=dtype)
@@ -87,7 +87,7 @@ def test_float_specials(ps, ora, dtype):
 
 @pytest.mark.parametrize("dtype,offset", [("int32", 1), ("float32", 3), ("int64", 1), ("float64", 1)])
 def test_unaligned_buffers(ps, ora, dtype, offset):
-    check(ps, ora, synth.keys(150007, dtype, "uniform", seed=9), offset=offset)
+    check(ps, ora, synth.keys(270007, dtype, "uniform", seed=9), offset=offset)
 
 
 def test_one_block_given_by_the_caller(ps, ora):
@@ -141,7 +141,7 @@ def test_runs_of_equal_keys(ps, ora):
     check(ps, ora, u)
 
 
-@pytest.mark.parametrize("n", [110592 - 1, 110592, 110592 + 1, 110592 + 64, 110592 + 65])
+@pytest.mark.parametrize("n", [36 * 4096 - 1, 36 * 4096, 36 * 4096 + 1, 36 * 4096 + 64, 36 * 4096 + 65])
 def test_fix_tile_edges(ps, ora, n):
     """Keys of 24 leading bits that come in pairs and triples, sizes around the
     fix kernel's tiles of 4096 positions."""
@@ -161,7 +161,7 @@ def check_records(ps, k, p, mode="exact"):
     assert tp.cpu().numpy().view(np.uint32).tobytes() == p[o].tobytes()
 
 
-@pytest.mark.parametrize("n", [MIN - 1, MIN, MIN + 1, 43 * 6144 - 1, 43 * 6144, 43 * 6144 + 1, 1000003])
+@pytest.mark.parametrize("n", [MIN, MIN + 1, 43 * 6144 - 1, 43 * 6144, 43 * 6144 + 1, 1000003])
 @pytest.mark.parametrize("kind", ["uniform", "index", "few", "few_index", "one_key", "all_equal"])
 def test_records(ps, n, kind):
     """Payloads that are the input position, or random, or few; keys distinct,
