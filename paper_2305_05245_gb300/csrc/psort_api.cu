@@ -428,8 +428,8 @@ size_t sort_ws_bytes(int64_t n, int dtype)
 // and fixes each bin's parameters and its part of the instance table (per
 // bin: all starts, then all lengths); launching a plan queues one persistent
 // launch for the segments of at most one tile (both short bins together), one
-// multi-instance pipeline per longer bin and one radix sort of all segments
-// beyond those.
+// multi-instance pipeline (or one launch of clusters) per longer bin and one
+// radix sort of all segments beyond those.
 struct BatchBin {
     size_t at;                // offset of the bin's starts in the instance table
     int64_t cnt, nmax, nsum;  // instances, longest, total keys
@@ -437,7 +437,8 @@ struct BatchBin {
     int items, threads;       // launch shape (0, 0: automatic)
     bool small;               // at most SMALL_SEG keys each (one warp each)
     bool front;               // at most one tile each: sorted by the persistent front kernel
-    bool radix;               // longer than batch_radix_min: every segment one block, sorted by radix
+    bool cluster;             // few segments of at most cluster_max keys: a cluster each
+    bool radix;               // longer than batch_radix_min, or few keys: every segment one block, by radix
 };
 struct BatchPlan {
     int dtype = 0, mode = 0;
@@ -461,6 +462,15 @@ struct BatchPlan {
 #define PS_BATCH_RADIX64 131072
 #endif
 static int64_t batch_radix_min(int dtype) { return tune_family(dtype) == 0 ? PS_BATCH_RADIX32 : PS_BATCH_RADIX64; }
+// Size bins of few keys below that cost their launches (75-110 us each).  They
+// join the radix run when there is one (2^23 keys add 0.17 ms to it) or when three
+// or more of them would run one by one; else a bin whose clusters fit the GPU at
+// once is one launch of those: 2^18 int32 keys in segments of 11,000 / 46,000 /
+// 183,000, merges 51 / 82 / 93 us, radix 67, clusters 28 / 53 / 58 (2^20 keys: 53 / 89
+// / 96, 84, 68 / 115 / 105).
+static constexpr int64_t BATCH_FEW = int64_t(1) << 23, BATCH_FEW_ALONE = int64_t(1) << 22;
+static constexpr int64_t BATCH_CLUSTER_CTAS = 176;
+static int64_t cluster_ctas(int64_t n) { return n <= 8192 ? 1 : n <= 16384 ? 4 : 16; }
 
 // own (optional): one device pointer per segment; segment i then lives in its
 // own buffer, and off only lays the segments out for the workspace.
@@ -493,6 +503,20 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         if (!force && len > rmin) b = (int)bins.size() - 1;
         bins[b].push_back(i);
     }
+    std::vector<int64_t> sum(bins.size(), 0);
+    for (size_t b = 0; b < bins.size(); b++)
+        for (int64_t i : bins[b]) sum[b] += off[i + 1] - off[i];
+    if (!force) {
+        const size_t last = bins.size() - 1;
+        int few = 0;
+        for (size_t b = 2; b < last; b++) few += sum[b] > 0 && sum[b] <= BATCH_FEW_ALONE;
+        const int64_t cap = !bins[last].empty() ? BATCH_FEW : few >= 3 ? BATCH_FEW_ALONE : 0;
+        for (size_t b = 2; b < last; b++)
+            if (sum[b] > 0 && sum[b] <= cap) {
+                bins[last].insert(bins[last].end(), bins[b].begin(), bins[b].end());
+                bins[b].clear();
+            }
+    }
     for (size_t b = 0; b < bins.size(); b++) {
         if (bins[b].empty()) continue;
         BatchBin bb;
@@ -511,7 +535,9 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         ps_params r;
         memset(&r, 0, sizeof(r));
         bb.radix = b + 1 == bins.size();
-        if (b <= 1 || bb.radix) {
+        bb.cluster = b > 1 && !bb.radix && !force && bb.nmax <= cluster_max(dtype) &&
+                     bb.cnt * cluster_ctas(bb.nmax) <= BATCH_CLUSTER_CTAS;
+        if (b <= 1 || bb.radix || bb.cluster) {
             r.n_blocks = r.n_parts = 1;  // the block sort is the whole sort
         } else if (force) {
             r = *force;
@@ -595,7 +621,9 @@ static int batch_launch(const BatchPlan& bp, const int64_t* dev_table, void* key
     for (size_t i = 0; i < bp.bins.size() && rc == PS_OK; i++) {
         if (bp.bins[i].front) continue;
         SortArgs a = batch_bin_args(bp, bp.bins[i], dev_table, keys, s);
-        if (ws && a.radix) {
+        if (bp.bins[i].cluster) {
+            rc = narrow ? run_cluster_u32(a) : run_cluster_u64(a);
+        } else if (ws && a.radix) {
             rc = narrow ? run_radix_u32(a, ws, cap) : run_radix_u64(a, ws, cap);
         } else if (ws) {
             const ShapeEntry* sh = shape_of(a.dtype, a.items, a.threads, &rc);
@@ -990,7 +1018,7 @@ int ps_batch_plan_create(const int64_t* host_seg_offsets, int64_t n_segs, int dt
     int rc = batch_make_plan(off, dtype, pivot_mode, nullptr, &p->plan);
     size_t ws = 0;
     for (const BatchBin& bb : p->plan.bins) {
-        if (bb.front) continue;
+        if (bb.front || bb.cluster) continue;
         SortArgs a = batch_bin_args(p->plan, bb, nullptr, nullptr, nullptr);
         int src = PS_OK;
         if (bb.radix) {

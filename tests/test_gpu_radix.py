@@ -251,3 +251,16 @@ def test_batch_long_runs_per_segment(ps):
     ps.sort_batch(x, torch.from_numpy(off).cuda())
     torch.cuda.synchronize()
     assert x.view(torch.int64).cpu().numpy().view(np.uint64).tobytes() == want.tobytes()
+
+
+@pytest.mark.parametrize("how", ["call", "plan", "server"])
+@pytest.mark.parametrize("dtype", ["int32", "float64"])
+@pytest.mark.parametrize("lens", [
+    [8193, 16384, 9000],                                # one small bin: a cluster per segment
+    [16385, 65536, 30000, 8193, 131072],                # three and more small bins: one radix run
+    [8193, 20000, 12289, 9216, 9217, 300000, 40000],    # a long segment takes the small bins along
+    [8193 + 7 * i for i in range(300)],                 # one bin too large for clusters
+    [70000, 500, 1025],
+])
+def test_batch_small_bins(ps, ora, how, dtype, lens):
+    check_batch(ps, ora, lens, dtype, "uniform", how)
