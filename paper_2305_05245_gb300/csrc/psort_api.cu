@@ -494,6 +494,7 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
     // batch_radix_min keys; the last bin = all longer ones
     const int64_t tile = 8192, rmin = std::max(tile, batch_radix_min(dtype));
     std::vector<std::vector<int64_t>> bins(49);
+    std::vector<int64_t> sum(bins.size(), 0);  // keys per bin
     for (int64_t i = 0; i < n_segs; i++) {
         const int64_t len = off[i + 1] - off[i];
         if (len <= 1) continue;
@@ -502,10 +503,8 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         while (len > (tile << (b - 1)) && b > 0) b++;
         if (!force && len > rmin) b = (int)bins.size() - 1;
         bins[b].push_back(i);
+        sum[b] += len;
     }
-    std::vector<int64_t> sum(bins.size(), 0);
-    for (size_t b = 0; b < bins.size(); b++)
-        for (int64_t i : bins[b]) sum[b] += off[i + 1] - off[i];
     if (!force) {
         const size_t last = bins.size() - 1;
         int few = 0;
@@ -848,8 +847,26 @@ static constexpr int64_t HOST_PIPE_MIN = int64_t(1) << 24;
 #define PS_HOST_RANGES 8   // partition ranges copied out while later ones merge
 #endif
 
+//
+// Blocks that are the library's choice (free) are as few as the transfers want:
+// one block per copy group, sorted by radix, and as many partitions, so that the
+// final merge has a small fan-in; both pivot modes then split exactly (the result
+// is the same).  More groups leave less sorting after the last copy but cost
+// launches: 4, 8 and 16 of them take 3.27 / 3.34 / 4.45 ms for 2^26 int32 and 23.5 /
+// 22.7 / 22.3 ms for 2^28 int64 (n_B = 128 and 16 blocks in 8 groups before: 3.95
+// and 23.8 ms).  Below HOST_FREE_MIN bytes copies before and after the radix sort
+// are faster: 2^24 int64 1.82 against 2.01 ms.
+static constexpr size_t HOST_FREE_MIN = (size_t)3 << 26;
+static ps_params host_free_blocks(size_t bytes)
+{
+    ps_params r;
+    memset(&r, 0, sizeof(r));
+    r.n_blocks = r.n_parts = std::min<int64_t>(16, std::max<int64_t>(4, (int64_t)(bytes >> 26)));
+    return r;
+}
+
 static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t n, int dtype, int mode,
-                          const ps_params& r, cudaStream_t s)
+                          const ps_params& r, bool free_blocks, cudaStream_t s)
 {
     const int64_t nb = r.n_blocks, L = (n + nb - 1) / nb;
     const size_t kb = dtype_size(dtype);
@@ -857,7 +874,7 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
     std::vector<int64_t> tab(2 * (size_t)nb);
     for (int64_t b = 0; b < nb; b++) {
         const int64_t bs = std::min(b * L, n), be = std::min(bs + L, n);
-        tab[(size_t)b] = bs;
+        tab[(size_t)b] = free_blocks ? 0 : bs;  // (free: every block in a call of its own)
         tab[(size_t)(nb + b)] = be - bs;
     }
     int64_t* dtab = nullptr;
@@ -865,7 +882,7 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
     if (rc != PS_OK) return rc;
     cudaError_t e = cudaMemcpyAsync(dtab, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, s);
     cudaStream_t sc = nullptr;
-    const int64_t G = std::max<int64_t>(1, (nb + PS_HOST_GROUPS - 1) / PS_HOST_GROUPS);  // blocks per group
+    const int64_t G = free_blocks ? 1 : std::max<int64_t>(1, (nb + PS_HOST_GROUPS - 1) / PS_HOST_GROUPS);  // blocks per group
     const int64_t ng = (nb + G - 1) / G;
     std::vector<cudaEvent_t> ev((size_t)ng + 1, nullptr);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&sc, cudaStreamNonBlocking);
@@ -901,11 +918,17 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
         a.n_sum = k1 - k0;
         a.extent = n;
         a.keep_order_keys = true;
+        if (free_blocks) {
+            a.keys = (char*)d + k0 * kb;
+            a.extent = L;
+            a.radix = true;
+        }
         rc = dispatch(a);
     }
     void* d2 = nullptr;  // the final merge's device output (exact splitting)
     if (e == cudaSuccess && rc == PS_OK && mode == PS_PIVOT_EXACT && PS_HOST_RANGES > 1)
         rc = ws_alloc(&d2, (size_t)n * kb, s);
+    if (rc == PS_ERR_NO_MEMORY && free_blocks) rc = PS_OK;  // merge into the host buffer instead
     if (e == cudaSuccess && rc == PS_OK) {
         SortArgs a;  // steps 2 to 4 on the sorted blocks, result into the host buffer
         a.keys = d;
@@ -923,7 +946,7 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
         a.dst_keys = d2 ? d2 : mapped;
         a.host_out = d2 ? const_cast<void*>(host_keys) : nullptr;
         a.copy_stream = d2 ? sc : nullptr;
-        a.out_ranges = PS_HOST_RANGES;
+        a.out_ranges = free_blocks ? (int)r.n_parts : PS_HOST_RANGES;
         a.presorted = true;
         rc = dispatch(a);
     }
@@ -1092,9 +1115,12 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode, const ps
     cudaError_t e = cudaSuccess;
     ps_params r;
     resolve(n, dtype, params, &r);
-    if (mapped && r.n_blocks > 1 && n >= HOST_PIPE_MIN) {
-        rc = host_pipelined(host_keys, mapped, d, n, dtype, pivot_mode, r, s);
-    } else if (mapped) {
+    const bool free_blocks = free_params(params, nullptr) && r.merge_variant == PS_MERGE_TREE;
+    if (mapped && free_blocks && bytes >= HOST_FREE_MIN) {
+        rc = host_pipelined(host_keys, mapped, d, n, dtype, PS_PIVOT_EXACT, host_free_blocks(bytes), true, s);
+    } else if (mapped && !free_blocks && r.n_blocks > 1 && n >= HOST_PIPE_MIN) {
+        rc = host_pipelined(host_keys, mapped, d, n, dtype, pivot_mode, r, false, s);
+    } else if (mapped && !(free_blocks && n > cluster_max(dtype))) {
         SortArgs a;
         a.keys = d;
         a.payload = nullptr;
@@ -1110,6 +1136,7 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode, const ps
         a.stream = s;
         a.src_keys = mapped;
         a.dst_keys = mapped;
+        a.free_blocks = free_blocks;
         rc = dispatch(a);
     } else {
         e = cudaMemcpyAsync(d, host_keys, bytes, cudaMemcpyHostToDevice, s);

@@ -264,3 +264,20 @@ def test_batch_long_runs_per_segment(ps):
 ])
 def test_batch_small_bins(ps, ora, how, dtype, lens):
     check_batch(ps, ora, lens, dtype, "uniform", how)
+
+
+@pytest.mark.parametrize("dtype,n", [("int32", 300000), ("float64", 200001), ("int32", (3 << 24) - 1), ("float32", 3 << 24),
+                                     ("int64", (3 << 23) + 5), ("float64", (1 << 26) + 1)])
+@pytest.mark.parametrize("mode", ["exact", "regular"])
+def test_pinned_host_keys(ps, ora, dtype, n, mode):
+    """Automatic sorts of pinned host keys around the smallest size that is
+    copied in groups, with a short last block."""
+    import torch
+    if n >= (1 << 26) and mode == "regular":
+        pytest.skip("one large case")
+    src = synth.keys_torch(n, dtype, "uniform", seed=n)
+    h = torch.empty_like(src, device="cpu", pin_memory=True)
+    h.copy_(src)
+    ps.sort_host(h, mode)
+    want = torch.sort(src)[0]
+    assert torch.equal(h.cuda(), want)
