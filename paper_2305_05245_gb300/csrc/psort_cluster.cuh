@@ -45,10 +45,11 @@ template <int W> __device__ __forceinline__ SBuf<Rec, W> cl_buf(const SBuf<Rec, 
     return q;
 }
 
-// Sorts instance blockIdx.x / CS of `in`; share: keys per CTA, a multiple of E,
-// at most NT*E, with CS * share no less than the longest instance.  src and dst
-// may be the same buffer (every key is read before the first barrier and written
-// after the last).  iptr (keys only): instances in buffers of their own.
+// Sorts block blockIdx.x / CS of the instances' n_B blocks each; share: keys per
+// CTA, a multiple of E, at most NT*E, with CS * share no less than the longest
+// block.  src and dst may be the same buffer (every key is read before the first
+// barrier and written after the last).  iptr (keys only, n_B = 1): instances in
+// buffers of their own.  keep: the result stays order keys.
 //
 // Latency bound: one cluster, a CTA of up to 32 warps per SM.  Shares of 1024 x 4
 // keys take half the merge work per thread of 1024 x 8 and are used while they
@@ -56,7 +57,7 @@ template <int W> __device__ __forceinline__ SBuf<Rec, W> cl_buf(const SBuf<Rec, 
 // / this kernel: 2^15 int32 85 / 31 us, 2^16 89 / 40 us, 40961 int64 (with a copy of
 // the keys) 84.7 / 34.8 us; 2^17 int32 by radix 60, here 55 us.
 template <int NT, int E, typename K, int XF, int WLEV, int CS>
-__global__ void __launch_bounds__(NT, 1) k_cluster_sort(GBuf<K> src, GBuf<K> dst, Inst in, int share, K* const* iptr)
+__global__ void __launch_bounds__(NT, 1) k_cluster_sort(GBuf<K> src, GBuf<K> dst, Inst in, int64_t n_B, int share, K* const* iptr, bool keep)
 {
     constexpr int T = NT * E;
     using SB = typename TileBuf<K, E>::type;
@@ -64,10 +65,12 @@ __global__ void __launch_bounds__(NT, 1) k_cluster_sort(GBuf<K> src, GBuf<K> dst
     extern __shared__ __align__(16) char smem[];
     char* sp = smem;
     const SB sb = SB::carve(sp, T);
-    const int64_t inst = blockIdx.x / CS;
+    const int64_t inst = n_B == 1 ? blockIdx.x / CS : blockIdx.x / CS / n_B;
     const unsigned c = CS > 1 ? cl_rank() : 0;
-    const int64_t N = in.len(inst);
-    const int64_t o = in.off(inst) + (int64_t)c * share;
+    int64_t bs = 0, be = in.len(inst);
+    if (n_B > 1) block_bounds(in.len(inst), n_B, blockIdx.x / CS - inst * n_B, bs, be);
+    const int64_t N = be - bs;
+    const int64_t o = in.off(inst) + bs + (int64_t)c * share;
     const int64_t left = N - (int64_t)c * share;
     const int n = left <= 0 ? 0 : (int)(left < share ? left : share);  // this CTA's keys
     const int tid = threadIdx.x;
@@ -151,7 +154,10 @@ __global__ void __launch_bounds__(NT, 1) k_cluster_sort(GBuf<K> src, GBuf<K> dst
             return;
         }
     }
-    for (int i = tid; i < n; i += NT) dst.template stx<XF>(o + i, sb.ld(i));
+    if (keep)
+        for (int i = tid; i < n; i += NT) dst.st(o + i, sb.ld(i));
+    else
+        for (int i = tid; i < n; i += NT) dst.template stx<XF>(o + i, sb.ld(i));
 }
 
 }  // namespace ps

@@ -1699,11 +1699,28 @@ __global__ void k_psrs_samples(GBuf<K> blk, GBuf<K> samples, Inst in, int64_t n_
     samples.st(idx, blk.ld(in.off(inst) + bs + pos));
 }
 
+// Copies n samples into shared memory at sp (16-byte aligned); the returned view
+// starts at its first sample.
+template <int NT, typename K> __device__ GBuf<K> pool_to_shared(const GBuf<K>& g, int64_t at, int n, char* sp)
+{
+    const GBuf<K> s{(K*)sp, n};
+    for (int i = threadIdx.x; i < n; i += NT) s.st(i, g.ld(at + i));
+    return s;
+}
+template <int NT> __device__ GBuf<Rec> pool_to_shared(const GBuf<Rec>& g, int64_t at, int n, char* sp)
+{
+    const GBuf<Rec> s{(uint64_t*)sp, (uint32_t*)(sp + 8 * (size_t)n), n};
+    for (int i = threadIdx.x; i < n; i += NT) s.st(i, g.ld(at + i));
+    return s;
+}
+
 // PSRS pivot k of an instance = element of rank (k-1)*nb1 + floor((nb1-1)/2)
 // of its sorted pool of samples; the pool is nb1 sorted lists, so the rank is
 // found by the same value bisection as exact splitting, without sorting the
 // pool.  One CTA per (instance, pivot).
-template <int NT, typename K>
+// MAXPER = 1 (at most NT blocks): the pool fits shared memory after the windows and
+// is searched there (64 x 63 samples: 34 -> 15 us; every probe was an L2 round trip).
+template <int NT, typename K, int MAXPER = (MAX_RUNS + NT - 1) / NT>
 __global__ void __launch_bounds__(NT) k_psrs_select(GBuf<K> samples, Inst in, int64_t n_B, int64_t n_P, K* piv)
 {
     extern __shared__ __align__(16) char smem[];
@@ -1718,13 +1735,15 @@ __global__ void __launch_bounds__(NT) k_psrs_select(GBuf<K> samples, Inst in, in
     const int64_t L = (N + n_B - 1) / n_B;
     const int64_t nb1 = (N + L - 1) / L;
     const int64_t per = n_P - 1;
+    const int64_t row0 = MAXPER == 1 ? 0 : inst * n_B;
     for (int64_t r = threadIdx.x; r < nb1; r += NT) {
-        a[r] = (inst * n_B + r) * per;
+        a[r] = (row0 + r) * per;
         b[r] = a[r] + per;
     }
+    if constexpr (MAXPER == 1) samples = pool_to_shared<NT>(samples, inst * n_B * per, (int)(nb1 * per), (char*)(b + n_B));
     __syncthreads();
     const int64_t q = (k - 1) * nb1 + (nb1 - 1) / 2;
-    const K v = select_value<NT, K>(samples, a, b, (int)nb1, q + 1);
+    const K v = select_value<NT, K, MAXPER>(samples, a, b, (int)nb1, q + 1);
     if (threadIdx.x == 0) piv[blockIdx.x] = v;
 }
 
@@ -1746,7 +1765,7 @@ __global__ void k_psrs_splits(GBuf<K> blk, const K* piv, Inst in, int64_t n_B, i
 // max(r_k, 1) (Eq. 1); c_k = r_k - #{x < P_k} (Eq. 2); split of block b =
 // #{x < P_k in b} plus the copies of P_k it contributes, taken greedily in
 // block order until c_k copies are placed.  One CTA per (instance, pivot).
-template <int NT, typename K>
+template <int NT, typename K, int MAXPER = (MAX_RUNS + NT - 1) / NT>
 __global__ void __launch_bounds__(NT) k_pses(GBuf<K> blk, Inst in, int64_t n_B, int64_t n_P, K* piv,
                                              int64_t* cvec, int64_t* splits)
 {
@@ -1801,7 +1820,7 @@ __global__ void __launch_bounds__(NT) k_pses(GBuf<K> blk, Inst in, int64_t n_B, 
             hi0 = (U)s_hi;
         }
     }
-    const K v = select_value<NT, K>(blk, a, b, (int)n_B, t, lo0, hi0);
+    const K v = select_value<NT, K, MAXPER>(blk, a, b, (int)n_B, t, lo0, hi0);
     const int per = (int)((n_B + NT - 1) / NT);
     const int r0 = threadIdx.x * per;
     int64_t lbs = 0, eqs = 0;
@@ -1852,6 +1871,7 @@ __global__ void k_offsets(const int64_t* splits, Inst in, int64_t n_B, int64_t n
     if (idx >= in.count * (n_P + 1)) return;
     const int64_t inst = idx / (n_P + 1), k = idx - inst * (n_P + 1);
     int64_t s = in.off(inst);
+#pragma unroll 8
     for (int64_t b = 0; b < n_B; b++) s += splits[(inst * n_B + b) * (n_P + 1) + k];
     offsets[idx] = s;
 }

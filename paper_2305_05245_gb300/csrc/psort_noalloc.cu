@@ -114,6 +114,12 @@ extern "C" int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode,
     a.n_P = r.n_parts;
     a.trace = nullptr;
     a.stream = (cudaStream_t)stream;
+    // short: one cluster, no workspace; else by radix where its workspace fits
+    // (it does up to PS_NOALLOC_MAX_KEYS)
+    if (n <= (narrow ? CLUSTER_MAX32 : CLUSTER_MAX64)) return narrow ? run_cluster_u32(a) : run_cluster_u64(a);
+    if ((narrow ? radix_bytes_u32(a) : radix_bytes_u64(a)) <= PS_NOALLOC_SCRATCH_BYTES)
+        return narrow ? run_radix_u32(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES)
+                      : run_radix_u64(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);
     return narrow ? run_sort_u32_on(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES)
                   : run_sort_u64_on(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);
 }

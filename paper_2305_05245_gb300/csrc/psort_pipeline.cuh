@@ -60,6 +60,7 @@ template <> struct Cfg<Rec> {
 
 constexpr int64_t FMAX = 256;  // largest fan-in of one in-block merge pass
 constexpr int MAXLEV = 6;     // refinement levels of one merge job
+constexpr size_t PSRS_POOL = 64 << 10;  // largest sample pool searched in shared memory (bytes)
 
 template <typename K> struct GStore {
     static constexpr size_t bytes = sizeof(K);
@@ -337,6 +338,29 @@ template <> inline GBuf<Rec> trace_gbuf<Rec>(const ps_trace* t)
     return GBuf<Rec>{(uint64_t*)t->pivots, t->pivot_payload, INT64_MAX};
 }
 
+// Step 1 of a few short blocks, as order keys, one thread-block cluster per block
+// (psort_cluster*.cu): one launch in place of the tile sort and the in-block merge
+// passes (8 launches each).  Taken while two rounds of CTAs at most hold all
+// blocks (one round of blocks that fit a tile, where only the tile sort is saved);
+// beyond, the tile sort's smaller CTAs use the GPU better.  64 blocks of 16384
+// uint32: 91 -> 27 us; 300 blocks of 3496: the tile sort is 8 us faster.
+template <typename K>
+cudaError_t cluster_blocks(int xf, const GBuf<K>& src, const GBuf<K>& dst, const Inst& in, int64_t n_B, int64_t L,
+                           cudaStream_t s);
+template <> cudaError_t cluster_blocks<uint32_t>(int, const GBuf<uint32_t>&, const GBuf<uint32_t>&, const Inst&, int64_t,
+                                                 int64_t, cudaStream_t);
+template <> cudaError_t cluster_blocks<uint64_t>(int, const GBuf<uint64_t>&, const GBuf<uint64_t>&, const Inst&, int64_t,
+                                                 int64_t, cudaStream_t);
+template <> cudaError_t cluster_blocks<Rec>(int, const GBuf<Rec>&, const GBuf<Rec>&, const Inst&, int64_t, int64_t,
+                                            cudaStream_t);
+static inline bool cluster_fits(int64_t blocks, int64_t L)
+{
+    if (L > CLUSTER_MAX64) return false;
+    int64_t cs = 1;
+    while (cs * 8192 < L) cs *= 2;
+    return blocks * cs <= (cs == 1 ? 152 : 2 * 152);
+}
+
 template <typename K, typename CF = Cfg<K>> struct Pipeline {
     using C = CF;
     using PlanK = Plan<K, CF>;
@@ -499,10 +523,18 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         const bool end_in_user = pl.direct;
         GBuf<K> cur = ((pl.npass % 2 == 0) != end_in_user) ? wsb : user;
         if (end_in_user && pl.npass == 0) cur = last;
-        if (a.presorted) cur = user;
-        else if ((e = tile_sort<XF>(first, cur, pl, a, s)) != cudaSuccess) return e;
+        bool sorted = a.presorted;
+        if (a.presorted) {
+            cur = user;
+        } else if (std::is_same<CF, Cfg<K>>::value && !pl.direct && !a.inst_ptrs && cluster_fits(pl.n_inst * pl.n_B, pl.L)) {
+            cur = wsb;
+            if ((e = cluster_blocks<K>(XF, first, cur, in, pl.n_B, pl.L, s)) != cudaSuccess) return e;
+            sorted = true;
+        } else if ((e = tile_sort<XF>(first, cur, pl, a, s)) != cudaSuccess) {
+            return e;
+        }
         int64_t W = T;
-        for (int p = 0; p < pl.npass && !a.presorted; p++) {
+        for (int p = 0; p < pl.npass && !sorted; p++) {
             MergeJob job{};  // in-block pass p
             job.kind = 0;
             job.K = (int)pl.F[p];
@@ -538,11 +570,12 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         if (pl.n_P > 1) {
             const int64_t npiv = pl.n_inst * (pl.n_P - 1);
             if (a.mode == PS_PIVOT_EXACT) {
-                auto f = k_pses<512, K>;
+                const bool few = pl.n_B <= 128;  // a thread per block: four warps wait less at the barriers
+                auto f = few ? k_pses<128, K, 1> : k_pses<512, K>;
                 size_t sm = 16 * (size_t)pl.n_B + 64;
                 if ((e = smem_attr(f, sm)) != cudaSuccess) return e;
                 ProfScope ps_("pses", s);
-                f<<<(unsigned)npiv, 512, sm, s>>>(cur, in, pl.n_B, pl.n_P, piv, cvec, splits);
+                f<<<(unsigned)npiv, few ? 128 : 512, sm, s>>>(cur, in, pl.n_B, pl.n_P, piv, cvec, splits);
             } else {
                 GBuf<K> samp = gbuf_at<K>(ws + pl.o_samp, nrows * (pl.n_P - 1));
                 const int64_t ns = nrows * (pl.n_P - 1);
@@ -550,12 +583,15 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
                     ProfScope ps_("psrs_samples", s);
                     k_psrs_samples<K><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(cur, samp, in, pl.n_B, pl.n_P);
                 }
-                auto f = k_psrs_select<512, K>;
-                size_t sm = 16 * (size_t)pl.n_B + 64;
+                // a sample pool of few blocks is searched in shared memory
+                const size_t pool = (size_t)pl.n_B * (pl.n_P - 1) * GStore<K>::bytes + 32;
+                const bool few = pl.n_B <= 128 && pool <= PSRS_POOL;
+                auto f = few ? k_psrs_select<128, K, 1> : k_psrs_select<512, K>;
+                size_t sm = 16 * (size_t)pl.n_B + 64 + (few ? pool : 0);
                 if ((e = smem_attr(f, sm)) != cudaSuccess) return e;
                 {
                     ProfScope ps_("psrs_select", s);
-                    f<<<(unsigned)npiv, 512, sm, s>>>(samp, in, pl.n_B, pl.n_P, piv);
+                    f<<<(unsigned)npiv, few ? 128 : 512, sm, s>>>(samp, in, pl.n_B, pl.n_P, piv);
                 }
                 ProfScope ps_("psrs_splits", s);
                 k_psrs_splits<K><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(cur, piv, in, pl.n_B, pl.n_P, splits);

@@ -114,3 +114,51 @@ def test_streams_and_capture(ps, ora):
         g.replay()
         torch.cuda.synchronize()
         assert x.cpu().numpy().tobytes() == ora.reference_sort(h[:x.numel()]).tobytes()
+
+
+@pytest.mark.parametrize("n,nb,np_", [(64 * 8192, 64, 16), (64 * 8192 + 1, 64, 64), (100 * 16384 - 7, 100, 7), (16385 * 32, 32, 5),
+                                      (65537 * 8, 8, 8), (131072 * 4, 4, 3), (131073 * 4, 4, 3), (70001, 129, 200), (50, 64, 64),
+                                      (300007, 128, 129)])
+@pytest.mark.parametrize("dtype", ["int32", "float64"])
+@pytest.mark.parametrize("mode", ["exact", "regular"])
+def test_blocks_given_by_the_caller(ps, ora, dtype, mode, n, nb, np_):
+    """Blocks sorted by clusters (up to 131072 keys each) and the sample pool in
+    shared memory (up to 128 blocks): output and intermediates of the four steps."""
+    import torch
+    host = synth.keys(n, dtype, "few_unique" if nb == 100 else "uniform", seed=n + nb)
+    x = torch.from_numpy(host.copy()).cuda()
+    tr = ps.sort(x, mode, n_blocks=nb, n_parts=np_, trace=True)
+    torch.cuda.synchronize()
+    ref = ora.sort(host, ora.EXACT if mode == "exact" else ora.REGULAR, nb, np_)
+    assert x.cpu().numpy().tobytes() == ref.out.tobytes()
+    assert tr.pivots.cpu().numpy()[:np_ - 1].tobytes() == ref.pivots.tobytes()
+    assert np.array_equal(tr.splits.cpu().numpy(), ref.splits)
+    assert np.array_equal(tr.offsets.cpu().numpy(), ref.offsets)
+
+
+@pytest.mark.parametrize("n,nb,np_", [(64 * 8192 + 5, 64, 16), (40000, 3, 9), (20000, 128, 60)])
+@pytest.mark.parametrize("mode", ["exact", "regular"])
+def test_record_blocks_given_by_the_caller(ps, n, nb, np_, mode):
+    import torch
+    z = synth.splitmix64(n, 2 * n)
+    k, p = z[:n] & np.uint64(0xFFFF), (z[n:] >> np.uint64(32)).astype(np.uint32)
+    tk, tp = torch.from_numpy(k.view(np.int64).copy()).cuda(), torch.from_numpy(p.view(np.int32).copy()).cuda()
+    ps.sort_pairs(tk, tp, mode, nb, np_)
+    torch.cuda.synchronize()
+    o = np.lexsort((p, k))
+    assert tk.cpu().numpy().view(np.uint64).tobytes() == k[o].tobytes()
+    assert tp.cpu().numpy().view(np.uint32).tobytes() == p[o].tobytes()
+
+
+@pytest.mark.parametrize("dtype,n", [("int32", 262144), ("int32", 262145), ("float32", 1 << 20), ("int64", 131072),
+                                     ("int64", 131073), ("float64", 1 << 20), ("uint64", 999999)])
+def test_noalloc(ps, ora, dtype, n):
+    import torch
+    host = synth.keys(n, dtype, "uniform", seed=n)
+    st = {"uint64": np.int64}.get(dtype, host.dtype)
+    x = torch.from_numpy(host.view(st).copy()).cuda()
+    for _ in range(2):
+        x.copy_(torch.from_numpy(host.view(st)))
+        ps.sort_noalloc(x.view(getattr(torch, dtype)))
+        torch.cuda.synchronize()
+        assert x.cpu().numpy().tobytes() == ora.reference_sort(host).tobytes()
