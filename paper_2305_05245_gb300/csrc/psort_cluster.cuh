@@ -55,10 +55,11 @@ template <int W> __device__ __forceinline__ SBuf<Rec, W> cl_buf(const SBuf<Rec, 
 // keys take half the merge work per thread of 1024 x 8 and are used while they
 // fit.  Measured per call, a tile sort, planning kernels and a chunk merge before
 // / this kernel: 2^15 int32 85 / 31 us, 2^16 89 / 40 us, 40961 int64 (with a copy of
-// the keys) 84.7 / 34.8 us; 2^17 int32 by radix 60, here 55 us.
+// the keys) 84.7 / 34.8 us.
 template <int NT, int E, typename K, int XF, int WLEV, int CS>
 __global__ void __launch_bounds__(NT, 1) k_cluster_sort(GBuf<K> src, GBuf<K> dst, Inst in, int64_t n_B, int share, K* const* iptr, bool keep)
 {
+    kernel_entry();
     constexpr int T = NT * E;
     using SB = typename TileBuf<K, E>::type;
     using SV = typename ViewOf<SB>::type;

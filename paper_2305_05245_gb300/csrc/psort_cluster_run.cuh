@@ -8,8 +8,6 @@ namespace ps {
 
 template <typename K> struct ClusterSort {
     static constexpr int TW = Cfg<K>::TW;  // warp-shuffle levels of the tile sort
-    static constexpr int EMAX = sizeof(K) == 4 ? 16 : 8;
-    static constexpr int64_t MAX = int64_t(16) * 1024 * EMAX;  // longest instance
 
     struct Job {
         GBuf<K> src, dst;
@@ -32,12 +30,14 @@ template <typename K> struct ClusterSort {
         cfg.blockDim = dim3(NT);
         cfg.dynamicSmemBytes = sm;
         cfg.stream = j.stream;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = CS;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = CS > 1 ? 1 : 0;
+        cudaLaunchAttribute at[2] = {};
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (see launch_next)
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = CS;
+        at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = CS > 1 ? 2 : 1;
         ProfScope ps_("cluster_sort", j.stream);
         return cudaLaunchKernelEx(&cfg, f, j.src, j.dst, j.in, j.n_B, share, j.own, j.keep);
     }
@@ -52,8 +52,7 @@ template <typename K> struct ClusterSort {
         if (n <= 8192) return launch<1024, 8, XF, 1>(j, n);
         if (n <= 16384) return launch<1024, 4, XF, 4>(j, n);
         if (n <= 65536) return launch<1024, 4, XF, 16>(j, n);
-        if (n <= 131072) return launch<1024, 8, XF, 16>(j, n);
-        return launch<1024, EMAX, XF, 16>(j, n);
+        return launch<1024, 8, XF, 16>(j, n);
     }
 
     // Many blocks (step 1 of a sort whose blocks were given): the fewest CTAs each.
@@ -74,7 +73,7 @@ template <typename K> struct ClusterSort {
         else return xf == 1 ? blocks_xf<1>(j, L) : xf == 2 ? blocks_xf<2>(j, L) : blocks_xf<0>(j, L);
     }
 
-    // One launch sorts every instance of a (at most MAX keys each).
+    // One launch sorts every instance of a (at most CLUSTER_MAX keys each).
     static int run(const SortArgs& a)
     {
         Inst in;
@@ -83,7 +82,7 @@ template <typename K> struct ClusterSort {
         in.count = a.n_inst;
         in.n0 = a.n;
         const int64_t n = a.inst_base ? a.n_max : a.n;
-        if (n > MAX) return PS_ERR_INVALID_ARG;
+        if (n > CLUSTER_MAX) return PS_ERR_INVALID_ARG;
         const GBuf<K> user = gbuf_user<K>(a);
         Job j{gbuf_ext<K>(a.src_keys, user), gbuf_ext<K>(a.dst_keys, user), in, 1, nullptr, false, a.stream};
         if constexpr (sizeof(K) <= 8) j.own = (K* const*)a.inst_ptrs;

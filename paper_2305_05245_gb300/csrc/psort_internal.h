@@ -140,9 +140,8 @@ size_t radix_bytes_rec(const SortArgs& a);
 size_t radix_bytes_u32(const SortArgs& a);
 size_t radix_bytes_u64(const SortArgs& a);
 // Short instances, each sorted by one thread-block cluster (psort_cluster.cuh),
-// all in one launch without workspace: at most CLUSTER_MAX32 (32-bit keys) or
-// CLUSTER_MAX64 keys each.
-constexpr int64_t CLUSTER_MAX32 = 262144, CLUSTER_MAX64 = 131072;
+// all in one launch without workspace: at most CLUSTER_MAX keys each.
+constexpr int64_t CLUSTER_MAX = 131072;
 int run_cluster_u32(const SortArgs& a);
 int run_cluster_u64(const SortArgs& a);
 int run_cluster_rec(const SortArgs& a);

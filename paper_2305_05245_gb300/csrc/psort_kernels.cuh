@@ -51,6 +51,17 @@ static __device__ __noinline__ void ps_violation(int site, long long idx, long l
 #define PS_IN(i, n, site) true
 #endif
 
+// ---------------------------------------------------------------- launches
+// First statement of every kernel: the library's kernels are launched with
+// programmatic stream serialization (launch_next), so a kernel's CTAs may be
+// scheduled while the kernel before them ends; they wait here until all its work
+// is done and visible, and let the kernel after them be scheduled in turn.  Hides
+// launch latency between the many short kernels of a sort.
+__device__ __forceinline__ void kernel_entry()
+{
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- key types
 
 // A record: 64-bit key and 32-bit payload, ordered by (key, payload).
@@ -870,6 +881,7 @@ template <int NT, int E, typename K, int XF, bool FINAL, int WLEV = 0>
 __global__ void __launch_bounds__(NT, (data_ctas<K, NT, E>()))
     k_tile_sort(GBuf<K> src, GBuf<K> dst, Inst in, int64_t n_B, int64_t R0, K* const* iptr)
 {
+    kernel_entry();
     constexpr int T = NT * E;
     constexpr bool PLAIN = sizeof(K) == 4 || sizeof(K) == 8;
     using SB = typename TileBuf<K, E>::type;
@@ -913,6 +925,7 @@ template <int NT, int E, typename K, int XF, int WLEV>
 __global__ void __launch_bounds__(NT, (data_ctas<K, NT, E>()))
     k_batch_front(GBuf<K> keys, Inst tiles, K* const* tptr, Inst small, K* const* sptr, unsigned long long* next)
 {
+    kernel_entry();
     static_assert(E == 32 && NT * E >= (NT / 32) * 1024, "one 1024-key run per warp in the tile buffer");
     constexpr int T = NT * E;
     constexpr int WARPS = NT / 32;
@@ -1044,10 +1057,12 @@ struct Level {
     int64_t* ng;
 };
 
-// Level 0 of a merge job: its groups' runs, output bases and sizes.
+// Level 0 of a merge job: its groups' runs, output bases and sizes; no oversized
+// groups yet.
 template <int DUMMY = 0>
-__global__ void k_root_windows(MergeJob job, int64_t G, Level L)
+__global__ void k_root_windows(MergeJob job, int64_t G, Level L, unsigned long long* nbig)
 {
+    kernel_entry();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= G * job.K) return;
     const int64_t g = idx / job.K;
@@ -1062,7 +1077,10 @@ __global__ void k_root_windows(MergeJob job, int64_t G, Level L)
         L.base[g] = job.out_base(g);
         L.size[g] = job.size(g);
     }
-    if (idx == 0) *L.ng = G;
+    if (idx == 0) {
+        *L.ng = G;
+        *nbig = 0;
+    }
 }
 
 // Children per group: ceil(M / cnom), at most jcap (so that the sample pool
@@ -1079,6 +1097,7 @@ __device__ __forceinline__ int64_t chunks_for(int64_t M, int64_t cnom, int64_t j
 template <int NT>
 __global__ void __launch_bounds__(NT) k_chunk_plan(Level L, int64_t cnom, int64_t jcap, int64_t* choff)
 {
+    kernel_entry();
     const int64_t G = *L.ng < L.cap ? *L.ng : L.cap;
     (void)PS_IN(*L.ng, L.cap + 1, 21);
     int64_t carry = 0;
@@ -1124,6 +1143,7 @@ template <int NT, int E, typename K, int SPC>
 __global__ void __launch_bounds__(NT) k_pool(Level L, GBuf<K> src, const int64_t* choff, int* chgrp,
                                              Splitter<K>* spl, int64_t ccap, Level C)
 {
+    kernel_entry();
     constexpr int POOL = NT * E;
     extern __shared__ __align__(16) char smem[];
     const int64_t g = blockIdx.x;
@@ -1295,6 +1315,7 @@ template <typename K>
 __global__ void k_corank(Level L, GBuf<K> src, const Splitter<K>* spl, const int64_t* choff, const int* chgrp,
                          Level C)
 {
+    kernel_entry();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int Kr = L.K;
     const int64_t c = idx / Kr;
@@ -1328,6 +1349,7 @@ __global__ void k_corank(Level L, GBuf<K> src, const Splitter<K>* spl, const int
 template <int NT>
 __global__ void __launch_bounds__(NT) k_child_stats(Level L, const int64_t* choff, const int* chgrp, Level C)
 {
+    kernel_entry();
     const int lane = threadIdx.x & 31;
     const int64_t c = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
     const int64_t ng = *L.ng < L.cap ? *L.ng : L.cap;
@@ -1480,6 +1502,7 @@ template <int NT, int E, typename K, int XF, bool BIG, bool ALIGNED, bool SORTCH
 __global__ void __launch_bounds__(NT, (BIG ? 1 : data_ctas<K, NT, E>())) k_merge(Level C, GBuf<K> src, GBuf<K> dst, int64_t nout, int64_t* big,
                                               unsigned long long* nbig, K* const* iptr, Inst in)
 {
+    kernel_entry();
     static_assert(!(BIG && ALIGNED), "the oversized-group path merges unpadded pieces");
     static_assert(!(SORTCHUNK && (BIG || ALIGNED)), "copy-and-sort chunks are unpadded and fit the capacity");
     constexpr int CAP = NT * E;
@@ -1605,6 +1628,7 @@ __global__ void __launch_bounds__(NT, (BIG ? 1 : data_ctas<K, NT, E>())) k_merge
 template <typename K, int XF>
 __global__ void k_merge_select(Level C, GBuf<K> src, GBuf<K> dst, int64_t nout, int KP, int TPB)
 {
+    kernel_entry();
     extern __shared__ __align__(16) char smem[];
     const int Kr = C.K;
     int64_t ng = *C.ng;
@@ -1685,6 +1709,7 @@ __global__ void k_merge_select(Level C, GBuf<K> src, GBuf<K> dst, int64_t nout, 
 template <typename K>
 __global__ void k_psrs_samples(GBuf<K> blk, GBuf<K> samples, Inst in, int64_t n_B, int64_t n_P)
 {
+    kernel_entry();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t per = n_P - 1;
     if (idx >= in.count * n_B * per) return;
@@ -1723,6 +1748,7 @@ template <int NT> __device__ GBuf<Rec> pool_to_shared(const GBuf<Rec>& g, int64_
 template <int NT, typename K, int MAXPER = (MAX_RUNS + NT - 1) / NT>
 __global__ void __launch_bounds__(NT) k_psrs_select(GBuf<K> samples, Inst in, int64_t n_B, int64_t n_P, K* piv)
 {
+    kernel_entry();
     extern __shared__ __align__(16) char smem[];
     int64_t* a = (int64_t*)smem;
     int64_t* b = a + n_B;
@@ -1751,6 +1777,7 @@ __global__ void __launch_bounds__(NT) k_psrs_select(GBuf<K> samples, Inst in, in
 template <typename K>
 __global__ void k_psrs_splits(GBuf<K> blk, const K* piv, Inst in, int64_t n_B, int64_t n_P, int64_t* splits)
 {
+    kernel_entry();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= in.count * n_B * (n_P - 1)) return;
     const int64_t row = idx / (n_P - 1), k = idx - row * (n_P - 1) + 1;
@@ -1769,6 +1796,7 @@ template <int NT, typename K, int MAXPER = (MAX_RUNS + NT - 1) / NT>
 __global__ void __launch_bounds__(NT) k_pses(GBuf<K> blk, Inst in, int64_t n_B, int64_t n_P, K* piv,
                                              int64_t* cvec, int64_t* splits)
 {
+    kernel_entry();
     extern __shared__ __align__(16) char smem[];
     int64_t* a = (int64_t*)smem;
     int64_t* b = a + n_B;
@@ -1852,6 +1880,7 @@ __global__ void __launch_bounds__(NT) k_pses(GBuf<K> blk, Inst in, int64_t n_B, 
 template <int DUMMY = 0>
 __global__ void k_split_borders(Inst in, int64_t n_B, int64_t n_P, int64_t* splits)
 {
+    kernel_entry();
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= in.count * n_B) return;
     const int64_t inst = row / n_B, b = row - inst * n_B;
@@ -1867,6 +1896,7 @@ __global__ void k_split_borders(Inst in, int64_t n_B, int64_t n_P, int64_t* spli
 template <int DUMMY = 0>
 __global__ void k_offsets(const int64_t* splits, Inst in, int64_t n_B, int64_t n_P, int64_t* offsets)
 {
+    kernel_entry();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= in.count * (n_P + 1)) return;
     const int64_t inst = idx / (n_P + 1), k = idx - inst * (n_P + 1);
@@ -1880,6 +1910,7 @@ __global__ void k_offsets(const int64_t* splits, Inst in, int64_t n_B, int64_t n
 template <typename K, int XF>
 __global__ void k_trace_pivots(const K* piv, int64_t n, GBuf<K> out)
 {
+    kernel_entry();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out.template stx<XF>(i, piv[i]);
 }

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <mutex>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "psort_internal.h"
@@ -320,6 +321,24 @@ template <typename KF> static cudaError_t smem_attr(KF* f, size_t bytes, bool wi
     return e;
 }
 
+// Launches f so that it may be scheduled while the kernel before it on the stream
+// ends (f starts with kernel_entry, which waits for that kernel).
+template <typename... P, typename... A>
+static inline cudaError_t launch_next(void (*f)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, std::forward<A>(args)...);
+}
+
 static inline int xf_of(int dtype)
 {
     switch (dtype) {
@@ -355,7 +374,7 @@ template <> cudaError_t cluster_blocks<Rec>(int, const GBuf<Rec>&, const GBuf<Re
                                             cudaStream_t);
 static inline bool cluster_fits(int64_t blocks, int64_t L)
 {
-    if (L > CLUSTER_MAX64) return false;
+    if (L > CLUSTER_MAX) return false;
     int64_t cs = 1;
     while (cs * 8192 < L) cs *= 2;
     return blocks * cs <= (cs == 1 ? 152 : 2 * 152);
@@ -410,7 +429,7 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         if (e != cudaSuccess) return e;
         const int64_t grid = pl.n_inst * pl.n_B * pl.R0;
         ProfScope ps_("tile_sort", s);
-        f<<<(unsigned)grid, TNT, tile_smem(), s>>>(src, dst, inst_of(pl, a_), pl.n_B, pl.R0, iptrs(a_));
+        launch_next(f, (unsigned)grid, TNT, tile_smem(), s, src, dst, inst_of(pl, a_), pl.n_B, pl.R0, iptrs(a_));
         return cudaGetLastError();
     }
 
@@ -439,11 +458,13 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
             Lv[l].size = (int64_t*)(m + sh.o_size[l]);
             Lv[l].ng = (int64_t*)(m + sh.o_ng[l]);
         }
+        int64_t* big = (int64_t*)(m + sh.o_big);  // number of oversized groups (zeroed with the windows), then the groups
+        unsigned long long* nbig = (unsigned long long*)big;
         cudaError_t e;
         {
             ProfScope ps_(fin ? "windows_final" : "windows_inblock", s);
             const int64_t nt = G0 * Kr;
-            k_root_windows<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(job, G0, Lv[0]);
+            launch_next(k_root_windows<0>, (unsigned)((nt + 255) / 256), 256, 0, s, job, G0, Lv[0], nbig);
         }
         auto fp = k_pool<PNT, PE, K, PS_POOL_SPC>;
         if ((e = smem_attr(fp, pool_smem(Kr))) != cudaSuccess) return e;
@@ -453,26 +474,22 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
             Splitter<K>* spl = (Splitter<K>*)(m + sh.o_spl[l]);
             {
                 ProfScope ps_(level_label(fin, 0, l), s);
-                k_chunk_plan<1024><<<1, 1024, 0, s>>>(Lv[l], sh.cnom[l], sh.jcap, choff);
+                launch_next(k_chunk_plan<1024>, 1, 1024, 0, s, Lv[l], sh.cnom[l], sh.jcap, choff);
             }
             {
                 ProfScope ps_(level_label(fin, 1, l), s);
-                fp<<<(unsigned)sh.G[l], PNT, pool_smem(Kr), s>>>(Lv[l], src, choff, chgrp, spl, sh.G[l + 1],
-                                                                 Lv[l + 1]);
+                launch_next(fp, (unsigned)sh.G[l], PNT, pool_smem(Kr), s, Lv[l], src, choff, chgrp, spl, sh.G[l + 1], Lv[l + 1]);
             }
             {
                 ProfScope ps_(level_label(fin, 2, l), s);
                 const int64_t nt = sh.G[l + 1] * Kr;
-                k_corank<K><<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(Lv[l], src, spl, choff, chgrp, Lv[l + 1]);
+                launch_next(k_corank<K>, (unsigned)((nt + 255) / 256), 256, 0, s, Lv[l], src, spl, choff, chgrp, Lv[l + 1]);
             }
             {
                 ProfScope ps_(level_label(fin, 3, l), s);
-                k_child_stats<256><<<(unsigned)((sh.G[l + 1] + 7) / 8), 256, 0, s>>>(Lv[l], choff, chgrp, Lv[l + 1]);
+                launch_next(k_child_stats<256>, (unsigned)((sh.G[l + 1] + 7) / 8), 256, 0, s, Lv[l], choff, chgrp, Lv[l + 1]);
             }
         }
-        int64_t* big = (int64_t*)(m + sh.o_big);
-        unsigned long long* nbig = (unsigned long long*)big;
-        if ((e = cudaMemsetAsync(nbig, 0, 8, s)) != cudaSuccess) return e;
         const Level& Lf = Lv[sh.nlev];
         const int64_t gf = sh.G[sh.nlev];
         if (variant == PS_MERGE_SELECT) {
@@ -485,7 +502,7 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
             auto fs = k_merge_select<K, XF>;
             if ((e = smem_attr(fs, (size_t)tpb * per)) != cudaSuccess) return e;
             ProfScope ps_(fin ? "merge_final" : "merge_inblock", s);
-            fs<<<(unsigned)((gf + tpb - 1) / tpb), 32, (size_t)tpb * per, s>>>(Lf, src, dst, pl.N, KP, tpb);
+            launch_next(fs, (unsigned)((gf + tpb - 1) / tpb), 32, (size_t)tpb * per, s, Lf, src, dst, pl.N, KP, tpb);
             return cudaGetLastError();
         }
         auto fm = variant == PS_MERGE_SORT ? k_merge<MNT, ME, K, XF, false, false, true>
@@ -494,14 +511,13 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         if ((e = smem_attr(fm, merge_smem(Kr))) != cudaSuccess) return e;
         {
             ProfScope ps_(fin ? "merge_final" : "merge_inblock", s);
-            fm<<<(unsigned)gf, MNT, merge_smem(Kr), s>>>(Lf, src, dst, pl.N, big + 1, nbig, own, job.in);
+            launch_next(fm, (unsigned)gf, MNT, merge_smem(Kr), s, Lf, src, dst, pl.N, big + 1, nbig, own, job.in);
         }
         auto fb = k_merge<MNT, BE, K, XF, true, false>;
         if ((e = smem_attr(fb, big_smem(Kr))) != cudaSuccess) return e;
         {
             ProfScope ps_(fin ? "merge_big_final" : "merge_big_inblock", s);
-            fb<<<(unsigned)std::min<int64_t>(gf, 2 * 152), MNT, big_smem(Kr), s>>>(Lf, src, dst, pl.N, big + 1,
-                                                                                    nbig, own, job.in);
+            launch_next(fb, (unsigned)std::min<int64_t>(gf, 2 * 152), MNT, big_smem(Kr), s, Lf, src, dst, pl.N, big + 1, nbig, own, job.in);
         }
         return cudaGetLastError();
     }
@@ -565,7 +581,7 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         const int64_t nrows = pl.n_inst * pl.n_B;
         {
             ProfScope ps_("split_borders", s);
-            k_split_borders<<<(unsigned)((nrows + 255) / 256), 256, 0, s>>>(in, pl.n_B, pl.n_P, splits);
+            launch_next(k_split_borders<0>, (unsigned)((nrows + 255) / 256), 256, 0, s, in, pl.n_B, pl.n_P, splits);
         }
         if (pl.n_P > 1) {
             const int64_t npiv = pl.n_inst * (pl.n_P - 1);
@@ -575,13 +591,13 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
                 size_t sm = 16 * (size_t)pl.n_B + 64;
                 if ((e = smem_attr(f, sm)) != cudaSuccess) return e;
                 ProfScope ps_("pses", s);
-                f<<<(unsigned)npiv, few ? 128 : 512, sm, s>>>(cur, in, pl.n_B, pl.n_P, piv, cvec, splits);
+                launch_next(f, (unsigned)npiv, few ? 128 : 512, sm, s, cur, in, pl.n_B, pl.n_P, piv, cvec, splits);
             } else {
                 GBuf<K> samp = gbuf_at<K>(ws + pl.o_samp, nrows * (pl.n_P - 1));
                 const int64_t ns = nrows * (pl.n_P - 1);
                 {
                     ProfScope ps_("psrs_samples", s);
-                    k_psrs_samples<K><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(cur, samp, in, pl.n_B, pl.n_P);
+                    launch_next(k_psrs_samples<K>, (unsigned)((ns + 255) / 256), 256, 0, s, cur, samp, in, pl.n_B, pl.n_P);
                 }
                 // a sample pool of few blocks is searched in shared memory
                 const size_t pool = (size_t)pl.n_B * (pl.n_P - 1) * GStore<K>::bytes + 32;
@@ -591,16 +607,16 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
                 if ((e = smem_attr(f, sm)) != cudaSuccess) return e;
                 {
                     ProfScope ps_("psrs_select", s);
-                    f<<<(unsigned)npiv, few ? 128 : 512, sm, s>>>(samp, in, pl.n_B, pl.n_P, piv);
+                    launch_next(f, (unsigned)npiv, few ? 128 : 512, sm, s, samp, in, pl.n_B, pl.n_P, piv);
                 }
                 ProfScope ps_("psrs_splits", s);
-                k_psrs_splits<K><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(cur, piv, in, pl.n_B, pl.n_P, splits);
+                launch_next(k_psrs_splits<K>, (unsigned)((ns + 255) / 256), 256, 0, s, cur, piv, in, pl.n_B, pl.n_P, splits);
             }
         }
         {
             ProfScope ps_("offsets", s);
             const int64_t no = pl.n_inst * (pl.n_P + 1);
-            k_offsets<<<(unsigned)((no + 255) / 256), 256, 0, s>>>(splits, in, pl.n_B, pl.n_P, offs);
+            launch_next(k_offsets<0>, (unsigned)((no + 255) / 256), 256, 0, s, splits, in, pl.n_B, pl.n_P, offs);
         }
         // Step 4: merge the k-th partitions of all blocks into the caller's
         // buffer (nothing to merge when the block sort was the whole sort).
@@ -651,7 +667,7 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
             if (t->pivots && pl.n_P > 1) {
                 GBuf<K> tp = trace_buf(t);
                 ProfScope ps_("trace_pivots", s);
-                k_trace_pivots<K, XF><<<(unsigned)((pl.n_P - 1 + 255) / 256), 256, 0, s>>>(piv, pl.n_P - 1, tp);
+                launch_next(k_trace_pivots<K, XF>, (unsigned)((pl.n_P - 1 + 255) / 256), 256, 0, s, piv, pl.n_P - 1, tp);
             }
             if (t->c && pl.n_P > 1) {
                 if (a.mode == PS_PIVOT_EXACT)
@@ -729,8 +745,7 @@ template <typename K, typename CF = Cfg<K>> struct Pipeline {
         if (e != cudaSuccess) return e;
         GBuf<K> user = gbuf_user<K>(a);
         ProfScope ps_("batch_front", a.stream);
-        f<<<(unsigned)grid, NT, smb, a.stream>>>(user, ti, t ? iptrs(*t) : nullptr, si, sm ? iptrs(*sm) : nullptr,
-                                                 next);
+        launch_next(f, (unsigned)grid, NT, smb, a.stream, user, ti, t ? iptrs(*t) : nullptr, si, sm ? iptrs(*sm) : nullptr, next);
         return cudaGetLastError();
     }
 

@@ -262,6 +262,7 @@ template <> __device__ __forceinline__ bool rx_differ(const Rec& x, const Rec& y
 // other CTAs then stop looking).
 template <int NT> __global__ void __launch_bounds__(NT) k_rx_descents(const uint32_t* p, int64_t n, unsigned* descents)
 {
+    kernel_entry();
     constexpr int U = 8;
     for (int64_t i0 = (int64_t)blockIdx.x * NT * U; i0 < n; i0 += (int64_t)gridDim.x * NT * U) {
         if (__syncthreads_or(*(volatile unsigned*)descents != 0)) return;
@@ -282,6 +283,7 @@ template <int NT> __global__ void __launch_bounds__(NT) k_rx_descents(const uint
 template <typename K, int XF>
 __global__ void __launch_bounds__(128) k_rx_sample(RxArgs<K> A)
 {
+    kernel_entry();
     constexpr int D = Rx<K>::D;
     const int64_t seg = blockIdx.x;
     const RxSegAt at = rx_at(A, seg);
@@ -332,6 +334,7 @@ template <typename K> __device__ __forceinline__ int rx_choose_lo(const RxArgs<K
 // (one CTA), then lists the segment of each (a warp per segment).
 template <int NT, typename K> __global__ void __launch_bounds__(NT) k_rx_at(RxArgs<K> A)
 {
+    kernel_entry();
     const int64_t per = (A.nseg + NT - 1) / NT, s0 = threadIdx.x * per, s1 = s0 + per < A.nseg ? s0 + per : A.nseg;
     int64_t c[4] = {0, 0, 0, 0};
     auto sizes = [&](int64_t seg, int64_t (&v)[4]) {
@@ -363,6 +366,7 @@ template <int NT, typename K> __global__ void __launch_bounds__(NT) k_rx_at(RxAr
 }
 template <typename K> __global__ void __launch_bounds__(256) k_rx_lists(RxArgs<K> A)
 {
+    kernel_entry();
     const int64_t seg = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (seg >= A.nseg) return;
     const RxSegAt at = A.at[seg];
@@ -386,6 +390,7 @@ template <typename K> __global__ void __launch_bounds__(256) k_rx_lists(RxArgs<K
 template <int NT, int G, typename K, int XF>
 __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
 {
+    kernel_entry();
     constexpr int D = Rx<K>::D;
     extern __shared__ __align__(16) char smem[];
     uint32_t* cnt = (uint32_t*)smem;  // [G][128][32]
@@ -618,6 +623,7 @@ constexpr unsigned RX_SPINS = 1u << 24;  // looks at one predecessor before a wa
 template <typename K, int XF, typename CT, int NT, int E, int CTAS>
 __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT* lb, CT* lb_next)
 {
+    kernel_entry();
     constexpr int T = NT * E, W = NT / 32, LB = 8;
     static_assert(NT >= 256, "one thread per digit value");
     extern __shared__ __align__(16) char smem[];
@@ -883,6 +889,7 @@ constexpr int FN = 256, FL = 64;
 template <typename K, int XF>
 __global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
 {
+    kernel_entry();
     if (A.nseg > 1 && blockIdx.x >= A.total[2]) return;
     const int64_t seg = A.nseg == 1 ? 0 : A.fix_seg[blockIdx.x];
     const RxPlan& pl = A.plan[seg];
@@ -1084,6 +1091,7 @@ __device__ void rx_sort_run(const GBuf<K>& x, const GBuf<K>& y, int64_t s, int64
 template <typename K, int XF>
 __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
 {
+    kernel_entry();
     constexpr int NT = 512;
     if (*A.nflag == 0) return;
     __shared__ uint32_t wt[(NT / 32) * 256];

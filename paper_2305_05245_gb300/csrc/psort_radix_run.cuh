@@ -119,7 +119,7 @@ template <typename K> struct Radix {
         CT* l1 = (CT*)(ws + y.o_lb1);
         for (int i = 0; i < D; i++) {
             ProfScope ps_("radix_pass", s);
-            fp<<<grid, SH::NT, sb, s>>>(A, i, (i & 1) ? l1 : l0, (i & 1) ? l0 : l1);
+            launch_next(fp, grid, SH::NT, sb, s, A, i, (i & 1) ? l1 : l0, (i & 1) ? l0 : l1);
         }
         return cudaGetLastError();
     }
@@ -131,25 +131,25 @@ template <typename K> struct Radix {
         cudaError_t e;
         if (y.nseg > 1) {
             ProfScope ps_("radix_segments", s);
-            k_rx_at<1024, K><<<1, 1024, 0, s>>>(A);
-            k_rx_lists<K><<<(unsigned)((y.nseg + 7) / 8), 256, 0, s>>>(A);
+            launch_next(k_rx_at<1024, K>, 1, 1024, 0, s, A);
+            launch_next(k_rx_lists<K>, (unsigned)((y.nseg + 7) / 8), 256, 0, s, A);
         }
         if constexpr (std::is_same<K, Rec>::value) {
             ProfScope ps_("radix_descents", s);
             const int64_t g = (A.in.n0 + 4095) / 4096;
-            k_rx_descents<512><<<(unsigned)std::min<int64_t>(g, grid_sms * 4), 512, 0, s>>>(A.first.p, A.in.n0, A.descents);
+            launch_next(k_rx_descents<512>, (unsigned)std::min<int64_t>(g, grid_sms * 4), 512, 0, s, A.first.p, A.in.n0, A.descents);
         }
         if constexpr (D > 4) {
             ProfScope ps_("radix_sample", s);
             const unsigned z = (unsigned)std::min<int64_t>((y.S + 127) / 128, y.nseg == 1 ? 512 : 16);
-            k_rx_sample<K, XF><<<dim3((unsigned)y.nseg, RX_TRY, z), 128, 0, s>>>(A);
+            launch_next(k_rx_sample<K, XF>, dim3((unsigned)y.nseg, RX_TRY, z), 128, 0, s, A);
         }
         auto fc = k_rx_count<CNT, G, K, XF>;
         const size_t cb = (size_t)G * 4096 * 4;
         if ((e = smem_attr(fc, cb)) != cudaSuccess) return e;
         {
             ProfScope ps_("radix_count", s);
-            fc<<<dim3((unsigned)y.chunks, D / G), CNT, cb, s>>>(A);
+            launch_next(fc, dim3((unsigned)y.chunks, D / G), CNT, cb, s, A);
         }
         if (std::is_same<CT, uint32_t>::value && y.T == C::Small::T)
             e = digits<XF, uint32_t, typename C::Small>(y, A, ws, grid_sms, s);
@@ -164,10 +164,10 @@ template <typename K> struct Radix {
                 constexpr size_t fb = sizeof(K) * (FT + 2 * FL + 1) + 2 * (FT / 2 + 2);
                 if ((e = smem_attr(ff, fb)) != cudaSuccess) return e;
                 ProfScope ps_("radix_fix", s);
-                ff<<<(unsigned)y.fixes, FN, fb, s>>>(A);
+                launch_next(ff, (unsigned)y.fixes, FN, fb, s, A);
             }
             ProfScope ps_("radix_long", s);
-            k_rx_long<K, XF><<<(unsigned)grid_sms, 512, 0, s>>>(A);
+            launch_next(k_rx_long<K, XF>, (unsigned)grid_sms, 512, 0, s, A);
         }
         return cudaGetLastError();
     }

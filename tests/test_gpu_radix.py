@@ -13,7 +13,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 T32, T64 = 512 * 24, 384 * 24  # keys per tile of a digit pass (large sorts; smaller ones: 4096, 8192)
-MIN = 131073                   # smallest size the radix block sort takes (32-bit keys: 262145)
+MIN = 131073                   # smallest size the radix block sort takes
 
 
 @pytest.fixture(scope="module")
