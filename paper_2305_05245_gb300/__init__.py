@@ -25,16 +25,21 @@ _MODES = {"regular": _lib.PS_PIVOT_REGULAR, "psrs": _lib.PS_PIVOT_REGULAR, 0: 0,
           "exact": _lib.PS_PIVOT_EXACT, "pses": _lib.PS_PIVOT_EXACT, 1: 1}
 
 
+_DTYPES = {}  # torch dtype -> code, filled on first use (the package imports without torch)
+
+
 def _dtype_code(dt) -> int:
-    import torch
-    m = {torch.int32: _lib.PS_I32, torch.int64: _lib.PS_I64, torch.float32: _lib.PS_F32,
-         torch.float64: _lib.PS_F64}
-    if hasattr(torch, "uint32"):
-        m[torch.uint32] = _lib.PS_U32
-        m[torch.uint64] = _lib.PS_U64
-    if dt not in m:
-        raise TypeError("unsupported key dtype %s" % dt)
-    return m[dt]
+    code = _DTYPES.get(dt)
+    if code is None:
+        import torch
+        _DTYPES.update({torch.int32: _lib.PS_I32, torch.int64: _lib.PS_I64, torch.float32: _lib.PS_F32,
+                        torch.float64: _lib.PS_F64})
+        if hasattr(torch, "uint32"):
+            _DTYPES.update({torch.uint32: _lib.PS_U32, torch.uint64: _lib.PS_U64})
+        if dt not in _DTYPES:
+            raise TypeError("unsupported key dtype %s" % dt)
+        code = _DTYPES[dt]
+    return code
 
 
 def _np_dtype_code(dt) -> int:
@@ -66,6 +71,14 @@ def _params(n_blocks: int, n_parts: int, merge_variant="tree", items_per_thread:
     p.items_per_thread = items_per_thread
     p.block_threads = block_threads
     return p
+
+
+def _params_arg(*args):
+    """The parameter block as a call argument; none when every field is
+    automatic (the library takes the two for the same)."""
+    if args == (0, 0, "tree", 0, 0):
+        return None
+    return ctypes.byref(_params(*args))
 
 
 def _stream_handle(stream) -> int | None:
@@ -143,8 +156,7 @@ def sort(keys, pivot_mode="exact", n_blocks: int = 0, n_parts: int = 0, trace: b
     if trace:
         tr, ct = _make_trace(n, code, n_blocks, n_parts, keys.dtype, keys.device, False)
     rc = lib.ps_sort_ex(keys.data_ptr() if n else None, n, code, _mode(pivot_mode),
-                        ctypes.byref(_params(n_blocks, n_parts, merge_variant, items_per_thread,
-                                             block_threads)),
+                        _params_arg(n_blocks, n_parts, merge_variant, items_per_thread, block_threads),
                         ctypes.byref(ct) if ct is not None else None, _stream_handle(stream))
     _lib.check(lib, "ps_sort_ex", rc)
     return tr
@@ -165,7 +177,7 @@ def sort_pairs(keys, payload, pivot_mode="exact", n_blocks: int = 0, n_parts: in
     if trace:
         tr, ct = _make_trace(n, -1, n_blocks, n_parts, keys.dtype, keys.device, True)
     rc = lib.ps_sort_pairs(keys.data_ptr() if n else None, payload.data_ptr() if n else None, n,
-                           _mode(pivot_mode), ctypes.byref(_params(n_blocks, n_parts, merge_variant)),
+                           _mode(pivot_mode), _params_arg(n_blocks, n_parts, merge_variant, 0, 0),
                            ctypes.byref(ct) if ct is not None else None, _stream_handle(stream))
     _lib.check(lib, "ps_sort_pairs", rc)
     return tr
@@ -189,7 +201,7 @@ def sort_struct(records, record_bytes: int | None = None, key_offset: int = 0, p
         raise ValueError("the tensor is not a whole number of records")
     n = nbytes // record_bytes
     rc = lib.ps_sort_struct(records.data_ptr() if n else None, n, record_bytes, key_offset, _mode(pivot_mode),
-                            ctypes.byref(_params(n_blocks, n_parts)), _stream_handle(stream))
+                            _params_arg(n_blocks, n_parts, "tree", 0, 0), _stream_handle(stream))
     _lib.check(lib, "ps_sort_struct", rc)
 
 
@@ -255,7 +267,7 @@ def sort_host(arr, pivot_mode="exact", n_blocks: int = 0, n_parts: int = 0, stre
             raise ValueError("host tensor must be a contiguous CPU tensor")
         code, ptr, n = _dtype_code(arr.dtype), arr.data_ptr(), arr.numel()
     rc = lib.ps_sort_host(ptr if n else None, n, code, _mode(pivot_mode),
-                          ctypes.byref(_params(n_blocks, n_parts)), _stream_handle(stream))
+                          _params_arg(n_blocks, n_parts, "tree", 0, 0), _stream_handle(stream))
     _lib.check(lib, "ps_sort_host", rc)
 
 
