@@ -307,9 +307,7 @@ static int log_level()
 // Sorts whose blocks are the library's choice sort their input as one block (the
 // result is the same whatever the blocks are, and nothing is left to partition
 // or merge): short ones by one thread-block cluster (cluster_takes), longer ones
-// by radix (2^17 int32 50 / 55 us, 2^18 71 / 62).  Measured, tiles and multiway merges
-// against these:
-// 3,000,001 float32 251 / 97 us, 2^26 int32 1.90 / 1.01 ms, 2^30 int64 54.7 / 25.9
+// by radix.  Measured, tiles and multiway merges against these: 3,000,001 float32 251 / 97 us, 2^26 int32 1.90 / 1.01 ms, 2^30 int64 54.7 / 25.9
 // ms, 2^28 records 25.8 / 10.1 ms (a copy of the keys included).
 static bool free_params(const ps_params* p, const ps_trace* trace)
 {
@@ -324,12 +322,12 @@ static bool one_block(const SortArgs& a)
 }
 static bool cluster_takes(const SortArgs& a)
 {
-    return one_block(a) && !a.keep_order_keys && a.n <= CLUSTER_MAX;
+    return one_block(a) && !a.keep_order_keys && a.n <= cluster_max(a.dtype);
 }
 static bool radix_takes(const SortArgs& a)
 {
     if (a.radix) return true;
-    return one_block(a) && !a.src_keys && !a.dst_keys && a.n > CLUSTER_MAX;
+    return one_block(a) && !a.src_keys && !a.dst_keys && a.n > cluster_max(a.dtype);
 }
 
 static int dispatch(SortArgs& a)
@@ -437,7 +435,7 @@ struct BatchBin {
     int items, threads;       // launch shape (0, 0: automatic)
     bool small;               // at most SMALL_SEG keys each (one warp each)
     bool front;               // at most one tile each: sorted by the persistent front kernel
-    bool cluster;             // few segments of at most CLUSTER_MAX keys: a cluster each
+    bool cluster;             // few segments of at most cluster_max keys: a cluster each
     bool radix;               // longer than batch_radix_min, or few keys: every segment one block, by radix
 };
 struct BatchPlan {
@@ -534,7 +532,7 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         ps_params r;
         memset(&r, 0, sizeof(r));
         bb.radix = b + 1 == bins.size();
-        bb.cluster = b > 1 && !bb.radix && !force && bb.nmax <= CLUSTER_MAX &&
+        bb.cluster = b > 1 && !bb.radix && !force && bb.nmax <= cluster_max(dtype) &&
                      bb.cnt * cluster_ctas(bb.nmax) <= BATCH_CLUSTER_CTAS;
         if (b <= 1 || bb.radix || bb.cluster) {
             r.n_blocks = r.n_parts = 1;  // the block sort is the whole sort
@@ -1120,7 +1118,7 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode, const ps
         rc = host_pipelined(host_keys, mapped, d, n, dtype, PS_PIVOT_EXACT, host_free_blocks(bytes), true, s);
     } else if (mapped && !free_blocks && r.n_blocks > 1 && n >= HOST_PIPE_MIN) {
         rc = host_pipelined(host_keys, mapped, d, n, dtype, pivot_mode, r, false, s);
-    } else if (mapped && !(free_blocks && n > CLUSTER_MAX)) {
+    } else if (mapped && !(free_blocks && n > cluster_max(dtype))) {
         SortArgs a;
         a.keys = d;
         a.payload = nullptr;

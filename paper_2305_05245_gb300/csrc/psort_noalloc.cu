@@ -116,7 +116,7 @@ extern "C" int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode,
     a.stream = (cudaStream_t)stream;
     // short: one cluster, no workspace; else by radix where its workspace fits
     // (it does up to PS_NOALLOC_MAX_KEYS)
-    if (n <= CLUSTER_MAX) return narrow ? run_cluster_u32(a) : run_cluster_u64(a);
+    if (n <= cluster_max(dtype)) return narrow ? run_cluster_u32(a) : run_cluster_u64(a);
     if ((narrow ? radix_bytes_u32(a) : radix_bytes_u64(a)) <= PS_NOALLOC_SCRATCH_BYTES)
         return narrow ? run_radix_u32(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES)
                       : run_radix_u64(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);

@@ -228,7 +228,7 @@ static __device__ unsigned long long rx_stall;
 #ifndef PS_RX_RUN
 #define PS_RX_RUN 1
 #endif
-constexpr int RX_SAMPLE_MAX = 1 << 16, RX_TRY = 4;
+constexpr int RX_SAMPLE_MAX = 1 << 16, RX_TRY = 4, RX_SLOTS = 4;  // (table slots per sampled key)
 // sqrt(8 n) sampled keys: runs with one other key each then give four hits.
 __host__ __device__ inline int rx_samples(int64_t n)
 {
@@ -278,8 +278,12 @@ template <int NT> __global__ void __launch_bounds__(NT) k_rx_descents(const uint
         }
     }
 }
-// CTA (segment, choice, part of the sample); tab: [RX_TRY][2 * S] entries
-// (sample + 1) per segment.
+// CTA (segment, choice, part of the sample); tab: [RX_TRY][RX_SLOTS * S] entries per
+// segment, sample + 1 in 17 bits and 15 further bits of the hash above them, so that
+// a probe reads another sample only when it is likely the same prefix.  Bound by the
+// longest chain of probes in a warp, an L2 round trip each (2^20 keys: 20 -> 5 us of kernel;
+// two slots per key and no hash bits took twice the probes, each with a read of the
+// other key).
 template <typename K, int XF>
 __global__ void __launch_bounds__(128) k_rx_sample(RxArgs<K> A)
 {
@@ -295,22 +299,26 @@ __global__ void __launch_bounds__(128) k_rx_sample(RxArgs<K> A)
     auto pos = [&](int j) { return (int64_t)__umul64hi(rx_mix((uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull), (uint64_t)n); };
     const typename Rx<K>::M m = Rx<K>::mask(lo, D - 1);
     const bool asc = *A.descents == 0;
-    unsigned* t = A.tab + at.tab0 + (size_t)blockIdx.y * 2 * S;
+    const unsigned slots = RX_SLOTS * (unsigned)S;
+    unsigned* t = A.tab + at.tab0 + (size_t)blockIdx.y * slots;
     unsigned c = 0;
     for (int i = blockIdx.z * 128 + threadIdx.x; i < S; i += gridDim.z * 128) {
         const int64_t pi = pos(i);
         const K x = src.template ldx<XF>(pi);
-        unsigned q = (unsigned)rx_mix(Rx<K>::word(x, m)) & (unsigned)(2 * S - 1);
-        for (int probe = 0; probe < 2 * S; probe++) {
-            const unsigned cur = atomicCAS(&t[q], 0u, (unsigned)(i + 1));
+        const uint64_t h = rx_mix(Rx<K>::word(x, m));
+        const unsigned tag = (unsigned)(h >> 49);
+        unsigned q = (unsigned)h & (slots - 1);
+        for (unsigned probe = 0; probe < slots; probe++) {
+            const unsigned cur = atomicCAS(&t[q], 0u, (tag << 17) | (unsigned)(i + 1));
             if (cur == 0) break;
-            const int64_t pj = pos((int)cur - 1);
-            const K y = src.template ldx<XF>(pj);
-            if (Rx<K>::same(x, y, m)) {
-                c += rx_differ(x, y, asc);
-                break;
+            if ((cur >> 17) == tag) {
+                const K y = src.template ldx<XF>(pos((int)(cur & 0x1FFFFu) - 1));
+                if (Rx<K>::same(x, y, m)) {
+                    c += rx_differ(x, y, asc);
+                    break;
+                }
             }
-            q = (q + 1) & (unsigned)(2 * S - 1);
+            q = (q + 1) & (slots - 1);
         }
     }
     c = __reduce_add_sync(0xFFFFFFFFu, c);
@@ -344,7 +352,7 @@ template <int NT, typename K> __global__ void __launch_bounds__(NT) k_rx_at(RxAr
         v[0] = (n + A.T - 1) / A.T;
         v[1] = (n + A.chunk - 1) / A.chunk;
         v[2] = A.sampled ? (n + FT - 1) / FT : 0;
-        v[3] = A.sampled ? RX_TRY * 2 * (int64_t)rx_samples(n) : 0;
+        v[3] = A.sampled ? RX_TRY * RX_SLOTS * (int64_t)rx_samples(n) : 0;
         return n;
     };
     for (int64_t seg = s0; seg < s1; seg++) {

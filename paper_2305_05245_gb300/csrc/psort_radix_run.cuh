@@ -83,7 +83,7 @@ template <typename K> struct Radix {
         y.o_hits = o;
         o += align256(sampled ? (size_t)y.nseg * RX_TRY * 4 : 0);
         y.o_tab = o;
-        o += align256(sampled ? (size_t)many * RX_TRY * 2 * 4 : 0);
+        o += align256(sampled ? (size_t)many * RX_TRY * RX_SLOTS * 4 : 0);
         y.o_flags = o;
         o += align256((size_t)y.fixes);
         y.o_lb0 = o;

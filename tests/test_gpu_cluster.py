@@ -35,7 +35,7 @@ def check(ps, ora, host, mode="exact", offset=0):
     assert not buf[:offset].any() and not buf[offset + host.size:].any()
 
 
-EDGES = [1024, 2048, 4096, 8192, 16384, 65536, 131072, 262144]
+EDGES = [1024, 2048, 4096, 8192, 16384, 65536, 98304, 131072, 262144]
 SIZES = sorted({2, 3, 31, 33, 100, 1000, 4 * 4096 - 3, 40961, 16 * 1028, 16 * 1028 + 1, 100003, 200001} |
                {e + d for e in EDGES for d in (-1, 0, 1)})
 
