@@ -139,26 +139,36 @@ def peaks():
 def kernel_source_hash() -> str:
     import hashlib
     csrc = os.path.join(ROOT, "paper_2305_05245_gb300", "csrc")
-    src = "".join(open(os.path.join(csrc, f)).read() for f in ("psort_kernels.cuh", "psort_pipeline.cuh"))
+    src = "".join(open(os.path.join(csrc, f)).read() for f in ("psort_kernels.cuh", "psort_pipeline.cuh", "psort_radix.cuh",
+                                                                  "psort_radix_run.cuh"))
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
-def ncu_traffic(kernel: str, workload: str):
-    """dram bytes per launch recorded in profiles/ncu_traffic.json for this
-    kernel and workload; null when absent, or when the kernel sources changed
-    since the counters were taken."""
+def ncu_traffic(kernel: str, workload: str, field: str = "dram_bytes_per_launch"):
+    """dram bytes per launch (or another field) recorded in
+    profiles/ncu_traffic.json for this kernel and workload; null when absent, or
+    when the kernel sources changed since the counters were taken."""
     try:
         with open(os.path.join(ROOT, "profiles", "ncu_traffic.json")) as f:
             d = json.load(f)
         if d.get("kernel_source_sha256_16") != kernel_source_hash():
             return None
         e = d.get(workload, {}).get(kernel)
-        return None if e is None else e.get("dram_bytes_per_launch")
+        return None if e is None else e.get(field)
     except Exception:
         return None
 
 
 # ------------------------------------------------------------ reference arm
+def radix_passes(prof, workload: str):
+    """Digit passes that moved keys, per sort, of a radix sort (None: not one).  A sort
+    queues one launch per byte of the key and the device decides which have work;
+    the number is the one recorded with the counters for this workload."""
+    if "radix_pass" not in prof:
+        return None
+    return ncu_traffic("radix_pass", workload, "active_launches_per_sort")
+
+
 def host_cpu():
     """nproc and the CPU model of this host (x86 "model name"; on Arm, lscpu's
     model name, else the implementer/part codes of /proc/cpuinfo)."""
@@ -607,6 +617,7 @@ def run_records(a):
                 "peak_source": src_peak, "traffic": None, "algorithmic_bytes_per_launch": per_launch}
     nb, np_ = ps.resolve_params(n, -1, a.n_blocks, a.n_parts)
     inblock = prof.get("merge_inblock", (0, 0))[0] // max(a.steps, 1)
+    passes = None if "radix_pass" in prof else 2 + inblock
     line = {
         "metric": METRIC, "value": n / ms / 1e6, "unit": "Gkeys/s", "n_gpus": 1, "steps": a.steps,
         "warmup": a.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -616,9 +627,9 @@ def run_records(a):
                    "l2": "inputs larger than L2 (no flush needed)", "in_block_merge_passes": inblock},
         "roofline": roof,
         "sort_roofline": {"algorithmic_bytes_per_key": 48, "achieved_gbs": 48 * n / (ms / 1e3) / 1e9,
-                          "frac": 48 * n / (ms / 1e3) / 1e9 / hbm, "passes_made": 2 + inblock,
-                          "passes_gbs": (2 + inblock) * 24 * n / (ms / 1e3) / 1e9,
-                          "passes_frac": (2 + inblock) * 24 * n / (ms / 1e3) / 1e9 / hbm},
+                          "frac": 48 * n / (ms / 1e3) / 1e9 / hbm, "passes_made": passes,
+                          "passes_gbs": passes and passes * 24 * n / (ms / 1e3) / 1e9,
+                          "passes_frac": passes and passes * 24 * n / (ms / 1e3) / 1e9 / hbm},
         "kernels": {kk: {"launches": v[0], "ms_per_step": v[1] / a.steps} for kk, v in prof.items()},
         "gpu_launches": sum(v[0] for v in prof.values()), "clocks": clk.summary(),
         "check": "ok" if ok else "FAILED",
@@ -906,6 +917,14 @@ def main():
     per_launch_bytes = 2 * n * s if dname in data_pass else None
     inblock_passes = prof.get("merge_inblock", (0, 0))[0] // max(a.steps, 1)
     wl = workload_name(a)
+    passes = 2 + inblock_passes
+    active = radix_passes(prof, wl)
+    if "radix_pass" in prof:
+        # every digit pass reads and writes the keys; counting and the ordering of
+        # runs read them once each, a pass between them
+        passes = None if active is None else active + 1
+        if dname == "radix_pass" and active:
+            per_launch_bytes, dl = 2 * n * s, active * a.steps
     roof = None
     if per_launch_bytes:
         ach = per_launch_bytes / (dms / dl / 1e3) / 1e9
@@ -932,10 +951,10 @@ def main():
         "roofline": roof,
         "sort_roofline": {"algorithmic_bytes_per_key": 4 * s, "achieved_gbs": 4 * s * n / (sort_ms / 1e3) / 1e9,
                           "frac": 4 * s * n / (sort_ms / 1e3) / 1e9 / hbm,
-                          "passes_made": 2 + inblock_passes,
+                          "passes_made": passes,
                           # the passes actually made, each a read and a write of every key
-                          "passes_gbs": (2 + inblock_passes) * 2 * s * n / (sort_ms / 1e3) / 1e9,
-                          "passes_frac": (2 + inblock_passes) * 2 * s * n / (sort_ms / 1e3) / 1e9 / hbm},
+                          "passes_gbs": passes and passes * 2 * s * n / (sort_ms / 1e3) / 1e9,
+                          "passes_frac": passes and passes * 2 * s * n / (sort_ms / 1e3) / 1e9 / hbm},
         "kernels": {k: {"launches": v[0], "ms_per_step": v[1] / a.steps} for k, v in prof.items()},
         "cpu_baseline": cpu,
         "e2e": e2e,

@@ -171,7 +171,8 @@ int ps_sort_struct(void* records, int64_t n, int64_t record_bytes, int64_t key_o
  * most one shared-memory tile (8192 keys) is sorted by one persistent launch
  * (a grid sized to the GPU whose CTAs take work items from a device counter:
  * a CTA per segment above 1024 keys, a warp per segment up to 1024 keys);
- * every longer bin runs the four-step method on all of its segments at once.
+ * longer segments run in size bins (all segments of a bin at once) or, the
+ * longest ones and bins of few keys, in one radix run of all of them.
  * So the number of kernel launches depends on the number of size bins, not
  * on the number of segments.  Each segment's result equals ps_sort on it alone.
  * The call reads seg_offsets back to the host (it waits for `stream` once,
@@ -214,7 +215,8 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode,
  * uniform keys of `dtype`'s width for every power-of-two size 2^b in
  * [max(n_min, 2^14), n_max], and records the fastest pair per (key width, b)
  * in a process-wide table that automatic parameters then use for sorts of
- * round(log2 n) = b.  batched = 0 tunes single sorts; batched = 1 tunes the
+ * round(log2 n) = b wherever n_B and n_P matter (see ps_params: not in plain
+ * sorts, nor in batches' radix runs).  batched = 0 tunes single sorts; batched = 1 tunes the
  * size bins of ps_sort_batch (batches of about 2^26 keys in segments of
  * (2^(b-1), 2^b] keys) and fills a separate table.  Each size then also
  * times every launch shape (items_per_thread x block_threads) the dtype
@@ -294,10 +296,7 @@ int ps_server_debug_fail(ps_server* server, int what, int count);
  * runtime.  ps_sort_noalloc sorts like ps_sort (same dtypes and pivot modes,
  * result bit-identical) but takes all of its workspace from one static device
  * array of PS_NOALLOC_SCRATCH_BYTES that the library reserves on every GPU it
- * is loaded on, for the life of the process.  Its n_B and n_P always come from
- * the size heuristic (not from tuned or measured table entries, which
- * ps_sort prefers): the array is sized for the heuristic's shapes, so the
- * speed may differ from ps_sort's, the result does not.
+ * is loaded on, for the life of the process (short sorts need none of it).
  *   - n above PS_NOALLOC_MAX_KEYS (or a shape whose workspace would not fit
  *     the array) is rejected with PS_ERR_INVALID_ARG before any work is queued.
  *   - It calls no cudaMalloc, cudaFree or pool allocation.  (Keep profiling

@@ -307,8 +307,9 @@ static int log_level()
 // Sorts whose blocks are the library's choice sort their input as one block (the
 // result is the same whatever the blocks are, and nothing is left to partition
 // or merge): short ones by one thread-block cluster (cluster_takes), longer ones
-// by radix.  Measured, tiles and multiway merges against these: 3,000,001 float32 251 / 97 us, 2^26 int32 1.90 / 1.01 ms, 2^30 int64 54.7 / 25.9
-// ms, 2^28 records 25.8 / 10.1 ms (a copy of the keys included).
+// by radix.  Measured, tiles and multiway merges against these: 3,000,001 float32
+// 252 / 89 us, 2^26 int32 1.90 / 1.02 ms, 2^30 int64 54.7 / 25.3 ms, 2^28 records
+// 25.7 / 10.2 ms (a copy of the keys included).
 static bool free_params(const ps_params* p, const ps_trace* trace)
 {
     if (trace) return false;

@@ -1106,8 +1106,9 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
     __shared__ uint32_t wt[(NT / 32) * 256];
     __shared__ unsigned long long cnt[256];
     __shared__ unsigned long long s_min;
-    const int64_t nt = A.nseg == 1 ? (A.in.n0 + FT - 1) / FT : A.total[2];
     int64_t off = 0, len = 0;
+    if (A.nseg == 1) rx_seg(A, 0, off, len);  // (its length, not the longest it might have had)
+    const int64_t nt = A.nseg == 1 ? (len + FT - 1) / FT : A.total[2];
     RxPlan pl{};
     RxSegAt at{};
     typename Rx<K>::M m{};

@@ -281,3 +281,20 @@ def test_pinned_host_keys(ps, ora, dtype, n, mode):
     ps.sort_host(h, mode)
     want = torch.sort(src)[0]
     assert torch.equal(h.cuda(), want)
+
+
+def test_pinned_host_keys_short_last_block(ps, ora):
+    """Copy groups whose last block ends a fix tile before the others, with runs
+    longer than a thread orders in every block."""
+    import torch
+    L = 6144 * 1024 + 1                     # 4 blocks of L keys; the last has L - 3
+    n = 4 * L - 3
+    u = synth.splitmix64(77, n)
+    top = u & ~np.uint64(0xFFFFFFFF)
+    for b in range(4):                      # 90 keys of one leading half in every block
+        at = b * L + 1000 * np.arange(90)
+        top[at] = top[b * L]
+    u = (top | (u & np.uint64(0xFFFFFFFF))).view(np.int64)
+    h = torch.from_numpy(u.copy()).pin_memory()
+    ps.sort_host(h)
+    assert torch.equal(h.cuda(), torch.sort(torch.from_numpy(u).cuda())[0])
