@@ -1,14 +1,14 @@
 // psort_radix.cuh -- step 1 (sort each block) as a least-significant-digit
 // radix sort of the order keys, for blocks of many tiles.
 //
-// A segment is one block of one instance (a single sort with one block is one
-// segment).  One kernel counts every digit of every segment; then one kernel
-// per digit reads the keys tile by tile, groups each tile by the digit in
-// shared memory and writes the groups to their places (one read and one write
-// of the data per digit, counting included in neither).  A tile learns where
-// its groups go by decoupled look-back (Merrill & Garland, "Single-pass
-// Parallel Prefix Scan with Decoupled Look-back", 2016): it publishes its
-// digit counts, sums the counts of the tiles before it and publishes the sum.
+// A segment is one instance, sorted as one block (a single sort is one segment).
+// One kernel counts every digit of every segment; then one kernel per digit reads
+// the keys tile by tile, groups each tile by the digit in shared memory and writes
+// the groups to their places (one read and one write of the data per digit,
+// counting included in neither).  A tile learns where its groups go by decoupled
+// look-back (Merrill & Garland, "Single-pass Parallel Prefix Scan with Decoupled
+// Look-back", 2016): it publishes its digit counts, sums the counts of the tiles
+// before it and publishes the sum.
 #pragma once
 
 #include <type_traits>
@@ -124,8 +124,7 @@ struct RxSegAt {
 template <typename K> struct RxArgs {
     GBuf<K> first, a, b, last;
     Inst in;
-    int64_t n_B;
-    int64_t nseg;            // segments (instances x blocks)
+    int64_t nseg;            // segments (instances)
     K* const* iptr;          // instances in buffers of their own (first, a and last)
     unsigned long long* hist;  // [nseg][D][256]: digit counts, then their exclusive sums
     RxPlan* plan;            // [nseg]
@@ -153,16 +152,8 @@ constexpr int FT = 4096;  // positions of a fix tile (k_rx_fix)
 
 template <typename K> __device__ __forceinline__ void rx_seg(const RxArgs<K>& A, int64_t seg, int64_t& off, int64_t& len)
 {
-    if (A.n_B == 1) {
-        off = A.in.off(seg);
-        len = A.in.len(seg);
-        return;
-    }
-    const int64_t inst = seg / A.n_B, b = seg - inst * A.n_B;
-    int64_t bs, be;
-    block_bounds(A.in.len(inst), A.n_B, b, bs, be);
-    off = A.in.off(inst) + bs;
-    len = be - bs;
+    off = A.in.off(seg);
+    len = A.in.len(seg);
 }
 // The segment's part of a buffer.
 template <typename K> __device__ __forceinline__ GBuf<K> rx_sub(const GBuf<K>& g, int64_t off, int64_t len)

@@ -188,7 +188,6 @@ template <typename K> struct Radix {
         A.in.n = a.inst_n;
         A.in.count = a.n_inst;
         A.in.n0 = a.n;
-        A.n_B = 1;
         A.nseg = y.nseg;
         A.iptr = std::is_same<K, Rec>::value ? nullptr : (K* const*)a.inst_ptrs;
         A.hist = (unsigned long long*)(ws + y.o_hist);
