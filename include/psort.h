@@ -318,6 +318,8 @@ int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode, ps_stream_
  * allocations of the library fail with PS_ERR_NO_MEMORY before any CUDA call
  * (0 turns it off).  Sorts then return PS_ERR_NO_MEMORY with nothing queued. */
 int ps_debug_fail_alloc(int count);
+/* The same for `count` allocations after the next `skip` of them. */
+int ps_debug_fail_alloc_after(int skip, int count);
 
 /* ---- checked builds -------------------------------------------------------
  * A build compiled with -DPS_CHECKED (libpsort_checked.so) validates every

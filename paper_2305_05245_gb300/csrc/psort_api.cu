@@ -54,14 +54,20 @@ static int get_pool(cudaMemPool_t* out)
     return PS_OK;
 }
 
-// Host-side failure injection (ps_debug_fail_alloc): the next n workspace
-// allocations fail with PS_ERR_NO_MEMORY before any CUDA call.
-static std::atomic<int> g_fail_alloc{0};
+// Host-side failure injection (ps_debug_fail_alloc, ps_debug_fail_alloc_after):
+// after g_skip_alloc more workspace allocations the next g_fail_alloc of them
+// fail with PS_ERR_NO_MEMORY before any CUDA call.
+static std::atomic<int> g_skip_alloc{0}, g_fail_alloc{0};
+static bool take_one(std::atomic<int>& c)
+{
+    for (int k = c.load(); k > 0;)
+        if (c.compare_exchange_weak(k, k - 1)) return true;
+    return false;
+}
 
 int ws_alloc(void** p, size_t bytes, cudaStream_t s)
 {
-    for (int k = g_fail_alloc.load(); k > 0;)
-        if (g_fail_alloc.compare_exchange_weak(k, k - 1)) return PS_ERR_NO_MEMORY;
+    if (g_fail_alloc.load() > 0 && !take_one(g_skip_alloc) && take_one(g_fail_alloc)) return PS_ERR_NO_MEMORY;
     cudaMemPool_t pool;
     int rc = get_pool(&pool);
     if (rc != PS_OK) return rc;
@@ -925,9 +931,10 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
         rc = dispatch(a);
     }
     void* d2 = nullptr;  // the final merge's device output (exact splitting)
-    if (e == cudaSuccess && rc == PS_OK && mode == PS_PIVOT_EXACT && PS_HOST_RANGES > 1)
+    if (e == cudaSuccess && rc == PS_OK && mode == PS_PIVOT_EXACT && PS_HOST_RANGES > 1) {
         rc = ws_alloc(&d2, (size_t)n * kb, s);
-    if (rc == PS_ERR_NO_MEMORY && free_blocks) rc = PS_OK;  // merge into the host buffer instead
+        if (rc == PS_ERR_NO_MEMORY && free_blocks) rc = PS_OK;  // merge into the host buffer instead
+    }
     if (e == cudaSuccess && rc == PS_OK) {
         SortArgs a;  // steps 2 to 4 on the sorted blocks, result into the host buffer
         a.keys = d;
@@ -1262,9 +1269,13 @@ const char* ps_status_string(int status)
 
 int ps_last_cuda_error(void) { return g_last_cuda; }
 
-int ps_debug_fail_alloc(int count)
+int ps_debug_fail_alloc(int count) { return ps_debug_fail_alloc_after(0, count); }
+
+int ps_debug_fail_alloc_after(int skip, int count)
 {
-    if (count < 0) return PS_ERR_INVALID_ARG;
+    if (skip < 0 || count < 0) return PS_ERR_INVALID_ARG;
+    g_fail_alloc.store(0);
+    g_skip_alloc.store(skip);
     g_fail_alloc.store(count);
     return PS_OK;
 }
