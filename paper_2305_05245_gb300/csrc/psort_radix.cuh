@@ -109,10 +109,6 @@ struct RxPlan {
     uint8_t dig[16];
 };
 
-// Device tables and buffers of one radix sort.  Pass 0 reads `first`, pass i
-// writes b (i even) or a (i odd); a last pass of odd index writes `last`
-// instead of a.  (A last pass of even index leaves the keys in b: only when
-// low digits were left out, k_rx_fix then moves them to `last`.)
 // Where a segment's work lies: its first tile, counting chunk and fix tile
 // among those of all segments, and its sample.
 struct RxSegAt {
@@ -121,6 +117,20 @@ struct RxSegAt {
     int b0;        // leading bytes of the sample's first choice
     int64_t tab0;  // its hash tables
 };
+// Work of k_rx_long: positions [s, e) of a segment.
+struct RxBad {
+    int64_t s, e;
+    int seg;
+    int tile;                 // 1: the runs inside one fix tile, 0: one run that spans tiles
+    unsigned slot;            // its first row of the digit table (runs longer than LONG_ONE)
+    unsigned ticket, done;    // tasks taken and finished (the same)
+    unsigned dp;              // bits that differ among its payloads and keys (the same)
+    unsigned long long dk;
+};
+// Device tables and buffers of one radix sort.  Pass 0 reads `first`, pass i
+// writes b (i even) or a (i odd); a last pass of odd index writes `last`
+// instead of a.  (A last pass of even index leaves the keys in b: only when
+// low digits were left out, k_rx_fix then moves them to `last`.)
 template <typename K> struct RxArgs {
     GBuf<K> first, a, b, last;
     Inst in;
@@ -145,6 +155,11 @@ template <typename K> struct RxArgs {
     unsigned* tab;           // hash tables
     uint8_t* flags;          // [fix tiles], see k_rx_fix
     unsigned* nflag;         // number of flagged tiles
+    // k_rx_long
+    unsigned* started;       // [fix tiles]: the long run that starts there is listed
+    RxBad* bad;              // [2 * fix tiles]: the list
+    unsigned* bads;          // [4]: its entries, rows of dtab given out; listing tasks taken and finished
+    void* dtab;              // digit table, 256 counts a row (CT)
     int min_pass;            // least number of passes (a sort between two buffers needs some)
     bool keep;               // the last pass leaves order keys
 };
@@ -207,8 +222,10 @@ static __device__ unsigned long long rx_stall;
 // bytes counts as a hit.  S keys have S^2/2 pairs, so a key has about
 // 2 * hits * n / S^2 different ones in its run; the smallest number of leading
 // bytes that keeps this at PS_RX_RUN or less wins.  Hits count whatever order
-// the two keys come in: nearly sorted input has long runs too.  A wrong guess
-// costs time, never order.  Measured: 2^30 int64 uniform 47.4 -> 27.3 ms, 2^26
+// the two keys come in: nearly sorted input has long runs too.  A guess can be
+// wrong (one value makes up a large share of the input and few of its
+// neighbours share its leading bytes: the sample sees none of them); it then
+// costs the passes of k_rx_long, never order.  Measured: 2^30 int64 uniform 47.4 -> 27.3 ms, 2^26
 // float64 Gaussian 3.03 -> 2.3 ms (five leading bytes), a copy of the keys
 // included.
 // Records of equal keys differ in their payload.  Where the payloads ascend
@@ -999,182 +1016,424 @@ __global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
     }
 }
 
-// Stable radix sort of x[s, e) by the bytes below lo, by one CTA, with y[s, e)
-// as scratch; both hold keys as the user sees them when inv.
-template <int NT, typename K, int XF>
-__device__ void rx_sort_run(const GBuf<K>& x, const GBuf<K>& y, int64_t s, int64_t e, int lo, bool inv, uint32_t* wt,
-                            unsigned long long* cnt)
+// --------------------------------------------------------------- long runs
+// Keys of one task of k_rx_long, and the longest run that one CTA sorts alone.
+constexpr int LONG_T = 16384, LONG_ONE = 2 * LONG_T;
+// The first position of [a, b) for which pred fails (it holds for those before),
+// by one warp, 32 probes a round.
+template <typename F> __device__ __forceinline__ int64_t rx_search(int64_t a, int64_t b, F pred)
 {
-    constexpr int W = NT / 32, E = 4;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    auto ld = [&](const GBuf<K>& b, int64_t i) { return inv ? b.template ldx<XF>(i) : b.ld(i); };
-    bool swapped = false;
-    for (int d = 0; d < lo; d++) {
-        const GBuf<K> src = swapped ? y : x, dst = swapped ? x : y;
-        for (int i = tid; i < 256; i += NT) cnt[i] = 0;
-        __syncthreads();
-        for (int64_t i = s + tid; i < e; i += NT) atomicAdd(&cnt[Rx<K>::dig(ld(src, i), d)], 1ull);
-        __syncthreads();
-        bool all = false;
-        for (int i = tid; i < 256; i += NT) all |= cnt[i] == (unsigned long long)(e - s);
-        if (__syncthreads_or(all)) continue;  // one value: nothing to do
-        if (tid < 32) {  // exclusive sums
-            unsigned long long v[8], t = 0;
-            for (int q = 0; q < 8; q++) t += v[q] = cnt[lane * 8 + q];
-            unsigned long long z = t;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long u = __shfl_up_sync(0xFFFFFFFFu, z, o);
-                if (lane >= o) z += u;
-            }
-            z -= t;
-            for (int q = 0; q < 8; q++) {
-                cnt[lane * 8 + q] = z;
-                z += v[q];
-            }
-        }
-        for (int64_t c = s; c < e; c += NT * E) {
-            for (int i = tid; i < W * 256; i += NT) wt[i] = 0;
-            __syncthreads();
-            K k[E];
-            uint32_t rk[E];
-            for (int j = 0; j < E; j++) {
-                const int64_t i = c + w * 32 * E + j * 32 + lane;
-                const bool in = i < e;
-                k[j] = ld(src, in ? i : s);
-                const unsigned v = Rx<K>::dig(k[j], d);
-                unsigned mt = __ballot_sync(0xFFFFFFFFu, in);
-                for (int b = 0; b < 8; b++) {
-                    const bool bit = (v >> b) & 1;
-                    const unsigned u = __ballot_sync(0xFFFFFFFFu, bit);
-                    mt &= bit ? u : ~u;
-                }
-                const unsigned r = __popc(mt & ((1u << lane) - 1));
-                const uint32_t old = wt[w * 256 + v];
-                __syncwarp();
-                if (in && r == 0) wt[w * 256 + v] = old + __popc(mt);
-                __syncwarp();
-                rk[j] = old + r;
-            }
-            __syncthreads();
-            uint32_t tot = 0;
-            if (tid < 256)
-                for (int q = 0; q < W; q++) {
-                    const uint32_t t = wt[q * 256 + tid];
-                    wt[q * 256 + tid] = tot;
-                    tot += t;
-                }
-            __syncthreads();
-            for (int j = 0; j < E; j++) {
-                if (c + w * 32 * E + j * 32 + lane >= e) continue;
-                const unsigned v = Rx<K>::dig(k[j], d);
-                const int64_t p = s + (int64_t)cnt[v] + wt[w * 256 + v] + rk[j];
-                if (p >= e) continue;
-                if (inv) dst.template stx<XF>(p, k[j]);
-                else dst.st(p, k[j]);
-            }
-            __syncthreads();
-            if (tid < 256) cnt[tid] += tot;
-            __syncthreads();
-        }
-        swapped = !swapped;
+    const int lane = threadIdx.x & 31;
+    while (a < b) {
+        const int64_t step = (b - a + 31) / 32, mid = a + (lane + 1) * step - 1;
+        const int k = __popc(__ballot_sync(0xFFFFFFFFu, mid < b && pred(mid)));
+        const int64_t top = a + (k + 1) * step - 1;
+        a += k * step;
+        if (a > b) a = b;
+        if (top < b) b = top;
     }
-    if (swapped)
-        for (int64_t i = s + tid; i < e; i += NT) x.st(i, y.ld(i));
+    return a;
+}
+// Lists the runs of the fix tile at t0 that are out of order (one warp; flag: the
+// tile's): those inside it as one range, one that goes beyond it once, whichever of
+// its tiles comes first.
+template <typename K, typename LD>
+__device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, unsigned flag, int seg, unsigned* started,
+                                        RxBad* bad, unsigned* nbad, unsigned* nslot)
+{
+    const typename Rx<K>::M m = Rx<K>::mask(lo, Rx<K>::D - 1);
+    const int64_t t1 = t0 + FT < len ? t0 + FT : len;
+    const bool one = (threadIdx.x & 31) == 0;
+    auto below = [&](const K& v) { return [&](int64_t i) { return Rx<K>::lt(ld(i), v, m); }; };
+    auto upto = [&](const K& v) { return [&](int64_t i) { return !Rx<K>::lt(v, ld(i), m); }; };
+    auto list = [&](int64_t s, int64_t e, int inside) {
+        if (!one) return;
+        const unsigned rows = e - s > LONG_ONE ? (unsigned)((e - s + LONG_T - 1) / LONG_T) : 0;
+        bad[atomicAdd(nbad, 1u)] = RxBad{s, e, seg, inside, rows ? atomicAdd(nslot, rows) : 0u, 0, 0, 0, 0};
+    };
+    auto spans = [&](int64_t s, int64_t e) {
+        const unsigned was = one ? atomicExch(&started[s / FT], 1u) : 0;
+        if (__shfl_sync(0xFFFFFFFFu, was, 0) == 0) list(s, e, 0);
+    };
+    // [in, out): the runs inside the tile
+    const K head = ld(t0), tail = ld(t1 - 1);
+    const int64_t in = t0 > 0 && Rx<K>::same(ld(t0 - 1), head, m) ? rx_search(t0, t1, upto(head)) : t0;
+    if (flag & 1) spans(rx_search(0, t0, below(head)), in < t1 ? in : rx_search(t1, len, upto(head)));
+    const int64_t out = t1 < len && Rx<K>::same(ld(t1), tail, m) ? rx_search(in, t1, below(tail)) : t1;
+    if (flag & 2) spans(out, rx_search(t1, len, upto(tail)));
+    if (flag & 4) list(in, out, 1);
+}
+// The bits in which a key differs from another, and the same as a key.
+__device__ __forceinline__ void rx_diff(uint64_t x, uint64_t y, unsigned long long& dk, unsigned&) { dk |= x ^ y; }
+__device__ __forceinline__ void rx_diff(const Rec& x, const Rec& y, unsigned long long& dk, unsigned& dp)
+{
+    dk |= x.k ^ y.k;
+    dp |= x.p ^ y.p;
+}
+template <typename K> __device__ __forceinline__ K rx_bits(unsigned long long dk, unsigned) { return dk; }
+template <> __device__ __forceinline__ Rec rx_bits<Rec>(unsigned long long dk, unsigned dp) { return Rec{dk, dp}; }
+// The bits in which the keys of [a, b) differ from ref, added to *dk and *dp (one
+// CTA; in shared or device memory).
+template <int NT, typename K, typename LD>
+__device__ __forceinline__ void rx_range_bits(LD ld, int64_t a, int64_t b, const K& ref, unsigned long long* dk, unsigned* dp)
+{
+    unsigned long long vk = 0;
+    unsigned vp = 0;
+#pragma unroll 8
+    for (int64_t i = a + threadIdx.x; i < b; i += NT) rx_diff(ld(i), ref, vk, vp);
+    const unsigned lo = __reduce_or_sync(0xFFFFFFFFu, (unsigned)vk), hi = __reduce_or_sync(0xFFFFFFFFu, (unsigned)(vk >> 32));
+    vp = __reduce_or_sync(0xFFFFFFFFu, vp);
+    if ((threadIdx.x & 31) == 0) {
+        if (lo | hi) atomicOr(dk, ((unsigned long long)hi << 32) | lo);
+        if (vp) atomicOr(dp, vp);
+    }
+}
+// How often each value of digit d occurs in [a, b), into cnt[256] (one CTA; wt: a
+// table per warp).  Mostly one value, so a warp adds its lanes' equal digits as one.
+template <int NT, typename K, typename LD>
+__device__ __forceinline__ void rx_range_count(LD ld, int64_t a, int64_t b, int d, uint32_t* wt, uint32_t* cnt)
+{
+    constexpr int W = NT / 32, U = 8;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint32_t* my = wt + (tid >> 5) * 256;
+    for (int i = tid; i < W * 256; i += NT) wt[i] = 0;
+    __syncthreads();
+    for (int64_t c = a; c < b; c += NT * U) {
+        unsigned v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = c + u * NT + tid;
+            v[u] = Rx<K>::dig(ld(i < b ? i : a), d);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const bool in = c + u * NT + tid < b;
+            const unsigned act = __ballot_sync(0xFFFFFFFFu, in), v0 = __shfl_sync(0xFFFFFFFFu, v[u], 0);
+            int one;
+            __match_all_sync(0xFFFFFFFFu, in ? v[u] : v0, &one);  // (lane 0 is in if any lane is)
+            if (one && act) {
+                if (lane == 0) atomicAdd(&my[v[u]], (uint32_t)__popc(act));
+            } else if (in) {
+                atomicAdd(&my[v[u]], 1u);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid < 256) {
+        uint32_t t = 0;
+#pragma unroll
+        for (int q = 0; q < W; q++) t += wt[q * 256 + tid];
+        cnt[tid] = t;
+    }
+    __syncthreads();
+}
+// Exclusive sums over the first 256 threads (red: 8 words of scratch).
+__device__ __forceinline__ unsigned long long rx_exsum256(unsigned long long t, unsigned long long* red)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long x = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (w < 8 && lane == 31) red[w] = x;
+    __syncthreads();
+    x -= t;
+    for (int q = 0; q < 8; q++)
+        if (q < w) x += red[q];
+    __syncthreads();
+    return x;
+}
+// Moves the keys of [a, b) to the places that pos[256] gives for digit d, in order
+// (one CTA; keys before `lim` only), and advances pos.
+template <int NT, typename K, typename LD, typename ST>
+__device__ __forceinline__ void rx_range_scatter(LD ld, ST st, int64_t a, int64_t b, int64_t lim, int d, uint32_t* wt,
+                                                 unsigned long long* pos)
+{
+    constexpr int W = NT / 32, E = 8;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    uint32_t* my = wt + w * 256;
+    for (int64_t c = a; c < b; c += NT * E) {
+        const int64_t p0 = c + w * 32 * E + lane;
+        for (int i = lane; i < 256; i += 32) my[i] = 0;
+        __syncwarp();
+        K k[E];
+        uint32_t rk[E];
+#pragma unroll
+        for (int j = 0; j < E; j++) k[j] = ld(p0 + j * 32 < b ? p0 + j * 32 : a);
+#pragma unroll
+        for (int j = 0; j < E; j++) {
+            const bool in = p0 + j * 32 < b;
+            const unsigned v = Rx<K>::dig(k[j], d);
+            unsigned mt = __ballot_sync(0xFFFFFFFFu, in);
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const bool bit = (v >> q) & 1;
+                const unsigned u = __ballot_sync(0xFFFFFFFFu, bit);
+                mt &= bit ? u : ~u;
+            }
+            const unsigned r = __popc(mt & ((1u << lane) - 1));
+            const uint32_t old = my[v];
+            __syncwarp();
+            if (in && r == 0) my[v] = old + __popc(mt);
+            __syncwarp();
+            rk[j] = old + r;
+        }
+        __syncthreads();
+        uint32_t tot = 0;
+        if (tid < 256) {
+#pragma unroll
+            for (int q = 0; q < W; q++) {
+                const uint32_t t = wt[q * 256 + tid];
+                wt[q * 256 + tid] = tot;
+                tot += t;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < E; j++) {
+            if (p0 + j * 32 >= b) continue;
+            const unsigned v = Rx<K>::dig(k[j], d);
+            const int64_t p = (int64_t)pos[v] + my[v] + rk[j];
+            if (p < lim) st(p, k[j]);
+        }
+        __syncthreads();
+        if (tid < 256) pos[tid] += tot;
+    }
     __syncthreads();
 }
 
-// The long runs that k_rx_fix left out of order, one CTA each (the sample
-// makes them rare).  Who sorts a run that spans tiles: the tile where it
-// starts if that tile saw it out of order, else the first later tile that did.
-// The flags and the leading bytes do not change here, so every CTA decides
-// alike.
-template <typename K, int XF>
+// Waits until *done reaches `need` (thread 0; bounded).
+__device__ __forceinline__ bool rx_reached(const unsigned* done, unsigned need, unsigned long long what)
+{
+    for (unsigned spins = 0; spins <= RX_SPINS; spins++) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+        if (v >= need) return true;
+        __nanosleep(100);
+    }
+    atomicExch(&rx_stall, what + 1);
+    return false;
+}
+
+// What k_rx_fix flagged.  All CTAs first list it (a task per LIST fix tiles, taken
+// in order from a counter) and wait until the list is whole.  The runs inside a tile are sorted together in shared
+// memory, by one CTA (they lie in order of their leading bytes already).  A run
+// that spans tiles is sorted by the bytes left out of the passes that vary in it,
+// lowest first, one CTA alone for up to LONG_ONE keys, all CTAs together for more:
+// its work is cut into tasks, taken in order from a counter:
+//   differing bits (a task per LONG_T keys); then for each varying byte: counts
+//   (the same), running sums of them (16), moves (the same); if the moves are odd
+//   in number, the way back.
+// A task waits until all tasks of the kinds before it are finished; those were
+// taken by CTAs that are running, so the waits end whatever share of the grid is
+// on the GPU.  (Listing in k_rx_fix costs that kernel 3% where there is nothing to list.)  So a sample that misjudged the input costs at most the passes it
+// saved, each at a grid's full width, and a counting pass each.  Measured, a whole
+// sort (one CTA per run before / this kernel; uniform keys in brackets): 2^20 float64
+// of which 30% are the mean 34.9 / 0.23 ms (0.11), 2^24 uint64 of which half are zero
+// 1171 / 1.05 ms (0.42), 2^26 int64 zeros with 1e-4 small values 7288 / 2.1 ms (1.44),
+// 2^26 records of such keys 8622 / 3.0 ms (2.4).
+// Records whose payloads ascend keep that order in a run: equal keys need no
+// payload digits.
+template <typename K, int XF, typename CT>
 __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
 {
     kernel_entry();
-    constexpr int NT = 512;
+    constexpr int NT = 512, E = 8, W = NT / 32;
+    static_assert(NT * E == FT, "a fix tile is one shared-memory sort");
+    constexpr int LIST = 64;
     if (*A.nflag == 0) return;
-    __shared__ uint32_t wt[(NT / 32) * 256];
-    __shared__ unsigned long long cnt[256];
-    __shared__ unsigned long long s_min;
-    int64_t off = 0, len = 0;
-    if (A.nseg == 1) rx_seg(A, 0, off, len);  // (its length, not the longest it might have had)
-    const int64_t nt = A.nseg == 1 ? (len + FT - 1) / FT : A.total[2];
-    RxPlan pl{};
-    RxSegAt at{};
-    typename Rx<K>::M m{};
-    GBuf<K> x, y;
+    using SB = typename TileBuf<K, E>::type;
+    extern __shared__ __align__(16) char smem[];
+    uint32_t* wt = (uint32_t*)smem;                              // [W][256]
+    unsigned long long* pos = (unsigned long long*)(wt + W * 256);  // [256]
+    uint32_t* cnt = (uint32_t*)(pos + 256);                      // [256]
+    unsigned long long* red = (unsigned long long*)(cnt + 256);  // [8]
+    __shared__ unsigned long long s_dk;
+    __shared__ unsigned s_dp, s_t;
+    __shared__ bool s_ok;
+    const int tid = threadIdx.x;
     const bool inv = !A.keep;
-    auto ld = [&](int64_t i) { return inv ? x.template ldx<XF>(i) : x.ld(i); };
-    // first position of [a, b) whose leading bytes are not below (not above) v's
-    auto lower = [&](int64_t a, int64_t b, const K& v) {
-        while (a < b) {
-            const int64_t q = a + ((b - a) >> 1);
-            if (Rx<K>::lt(ld(q), v, m)) a = q + 1;
-            else b = q;
-        }
-        return a;
+    const bool ascending = sizeof(K) > 8 && *A.descents == 0;
+    GBuf<K> x, y;
+    int64_t off, len;
+    int lo = 0, first = 0;  // the bytes to sort: [first, lo)
+    auto open = [&](const RxBad& q) {
+        rx_seg(A, (int64_t)q.seg, off, len);
+        lo = A.plan[q.seg].lo;
+        first = ascending && lo >= 4 ? 4 : 0;
+        x = rx_global(A.iptr ? rx_own(A.iptr, (int64_t)q.seg, 0, len) : rx_sub(A.last, off, len));
+        y = rx_global(rx_sub(A.b, off, len));
     };
-    auto upper = [&](int64_t a, int64_t b, const K& v) {
-        while (a < b) {
-            const int64_t q = a + ((b - a) >> 1);
-            if (!Rx<K>::lt(v, ld(q), m)) a = q + 1;
-            else b = q;
-        }
-        return a;
+    // keys of x, or of y once they are swapped
+    auto from = [&](bool swapped) {
+        return [&, swapped](int64_t i) {
+            const GBuf<K>& b = swapped ? y : x;
+            return inv ? b.template ldx<XF>(i) : b.ld(i);
+        };
     };
-    for (int64_t f0 = (int64_t)blockIdx.x * 32; f0 < nt; f0 += (int64_t)gridDim.x * 32) {
-        const int fl = threadIdx.x < 32 && f0 + threadIdx.x < nt ? A.flags[f0 + threadIdx.x] : 0;
-        if (!__syncthreads_or(fl)) continue;
-        for (int64_t f = f0; f < f0 + 32 && f < nt; f++) {
-            const int g = A.flags[f];
-            if (g == 0) continue;
-            const int64_t seg = A.nseg == 1 ? 0 : A.fix_seg[f];
-            rx_seg(A, seg, off, len);
-            pl = A.plan[seg];
-            at = rx_at(A, seg);
-            m = Rx<K>::mask(pl.lo, Rx<K>::D - 1);
-            x = A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.last, off, len);
-            y = rx_sub(A.b, off, len);
-            const int64_t t0 = (f - at.fix0) * FT, t1 = t0 + FT < len ? t0 + FT : len;
-            if (g & 4) {
-                for (int64_t from = t0 + 1;;) {
-                    if (threadIdx.x == 0) s_min = ~0ull;
-                    __syncthreads();
-                    for (int64_t i = from + threadIdx.x; i < t1; i += NT) {
-                        const K v = ld(i), u = ld(i - 1);
-                        if (!Rx<K>::same(u, v, m) || !key_lt(v, u)) continue;
-                        if (t0 > 0 && Rx<K>::same(ld(t0 - 1), v, m)) continue;
-                        if (t1 < len && Rx<K>::same(ld(t1), v, m)) continue;
-                        atomicMin(&s_min, (unsigned long long)i);
-                    }
-                    __syncthreads();
-                    const unsigned long long at = s_min;
-                    __syncthreads();
-                    if (at == ~0ull) break;
-                    const K v = ld((int64_t)at);
-                    const int64_t s = lower(t0, (int64_t)at, v), e = upper((int64_t)at, t1, v);
-                    __syncthreads();
-                    rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
-                    from = e;
-                }
+    auto into = [&](bool swapped) {
+        return [&, swapped](int64_t i, const K& v) {
+            const GBuf<K>& b = swapped ? x : y;
+            if (inv) b.template stx<XF>(i, v);
+            else b.st(i, v);
+        };
+    };
+    {
+        if (A.nseg == 1) rx_seg(A, 0, off, len);  // (its length, not the longest it might have had)
+        const int64_t tiles = A.nseg == 1 ? (len + FT - 1) / FT : A.total[2];
+        const unsigned tasks = (unsigned)((tiles + LIST - 1) / LIST);
+        for (;;) {
+            __syncthreads();
+            if (tid == 0) s_t = atomicAdd(&A.bads[2], 1u);
+            __syncthreads();
+            const unsigned t = s_t;
+            if (t >= tasks) break;
+            const int64_t f0 = (int64_t)t * LIST + (tid >> 5) * (LIST / W);  // a few tiles per warp
+            for (int64_t f = f0; f < f0 + LIST / W && f < tiles; f++) {
+                const unsigned flag = A.flags[f];
+                if (flag == 0) continue;
+                RxBad q{};
+                q.seg = A.nseg == 1 ? 0 : A.fix_seg[f];
+                const int fix0 = rx_at(A, q.seg).fix0;
+                open(q);
+                rx_list<K>(from(false), len, (f - fix0) * FT, lo, flag, q.seg, A.started + fix0, A.bad, A.bads, A.bads + 1);
             }
-            if (g & 2) {
-                const K v = ld(t1 - 1);
-                const int64_t s = lower(t0, t1 - 1, v), e = upper(t1, len, v);
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) atomicAdd(&A.bads[3], 1u);
+        }
+        if (tid == 0) s_ok = rx_reached(&A.bads[3], tasks, ~0ull - 1);
+        __syncthreads();
+        if (!s_ok) return;
+    }
+    const unsigned nbad = __ldcg(A.bads);
+    for (unsigned r = blockIdx.x; r < nbad; r += gridDim.x) {
+        const RxBad q = A.bad[r];
+        if (!q.tile && q.e - q.s > LONG_ONE) continue;
+        open(q);
+        __syncthreads();
+        if (q.tile) {
+            char* sp = smem;
+            const SB sb = SB::carve(sp, FT);
+            const int n = (int)(q.e - q.s);
+            if (inv) tile_sort_body<NT, E, K, XF, true, 0>(sb, x, q.s, x, q.s, n);
+            else tile_sort_body<NT, E, K, 0, true, 0>(sb, x, q.s, x, q.s, n);
+            continue;
+        }
+        if (tid == 0) s_dk = s_dp = 0;
+        __syncthreads();
+        const auto ld = from(false);
+        rx_range_bits<NT, K>(ld, q.s, q.e, ld(q.s), &s_dk, &s_dp);
+        __syncthreads();
+        const K bits = rx_bits<K>(s_dk, s_dp);
+        bool swapped = false;
+        for (int d = first; d < lo; d++) {
+            if (Rx<K>::dig(bits, d) == 0) continue;
+            rx_range_count<NT, K>(from(swapped), q.s, q.e, d, wt, cnt);
+            const unsigned long long ex = rx_exsum256(tid < 256 ? cnt[tid] : 0, red);
+            if (tid < 256) pos[tid] = (unsigned long long)q.s + ex;
+            __syncthreads();
+            rx_range_scatter<NT, K>(from(swapped), into(swapped), q.s, q.e, q.e, d, wt, pos);
+            swapped = !swapped;
+        }
+        if (swapped)
+            for (int64_t i = q.s + tid; i < q.e; i += NT) x.st(i, y.ld(i));
+    }
+    // the longest runs, each CTA from a place of its own on, then the others'
+    const unsigned start = (unsigned)((unsigned long long)blockIdx.x * nbad / gridDim.x);
+    for (unsigned k0 = 0; k0 < nbad; k0 += NT) {
+        for (unsigned next = k0;;) {
+            __syncthreads();
+            if (tid == 0) s_t = ~0u;
+            __syncthreads();
+            const unsigned k = k0 + tid;
+            if (k >= next && k < nbad) {
+                const RxBad* q = A.bad + (start + k) % nbad;
+                if (!q->tile && q->e - q->s > LONG_ONE) atomicMin(&s_t, k);
+            }
+            __syncthreads();
+            const unsigned pick = s_t;
+            if (pick == ~0u) break;
+            next = pick + 1;
+            RxBad* bad = A.bad + (start + pick) % nbad;
+            open(*bad);
+            const int64_t s = bad->s, e = bad->e;
+            const unsigned nt = (unsigned)((e - s + LONG_T - 1) / LONG_T);
+            CT* table = (CT*)A.dtab + (size_t)bad->slot * 256;  // [256][nt]: counts, then their running sums
+            K bits{};
+            int digits = -1;  // varying bytes, once known
+            for (;;) {
                 __syncthreads();
-                rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
-            }
-            if (g & 1) {
-                const K v = ld(t0);
-                const int64_t s = lower(0, t0, v), fs = at.fix0 + s / FT;
-                bool other = threadIdx.x == 0 && (A.flags[fs] & 2);
-                for (int64_t q = fs + 1 + threadIdx.x; q < f; q += NT) other |= (A.flags[q] & 1) != 0;
-                if (!__syncthreads_or(other)) {
-                    const int64_t e = upper(t0, len, v);
+                if (tid == 0) s_t = atomicAdd(&bad->ticket, 1u);
+                __syncthreads();
+                const unsigned t = s_t;
+                if (t < nt) {
+                    const auto ld = from(false);
+                    const int64_t a = s + (int64_t)t * LONG_T, b = a + LONG_T < e ? a + LONG_T : e;
+                    rx_range_bits<NT, K>(ld, a, b, ld(s), &bad->dk, &bad->dp);
+                } else {
+                    if (digits < 0) {
+                        if (tid == 0) s_ok = rx_reached(&bad->done, nt, bad->slot);
+                        __syncthreads();
+                        if (!s_ok) return;
+                        bits = rx_bits<K>(__ldcg(&bad->dk), __ldcg(&bad->dp));
+                        digits = 0;
+                        for (int d = first; d < lo; d++) digits += Rx<K>::dig(bits, d) != 0;
+                    }
+                    const unsigned per = 2 * nt + 16;  // tasks of one byte
+                    const unsigned di = (t - nt) / per, sub = (t - nt) - di * per;
+                    const bool back = (int)di == digits;
+                    if ((int)di > digits || (back && (!(digits & 1) || sub >= nt))) break;
+                    const unsigned kind = back || sub < nt ? 0 : sub < nt + 16 ? 1 : 2;
+                    const unsigned before = nt + di * per + (kind == 0 ? 0 : kind == 1 ? nt : nt + 16);
+                    if (tid == 0) s_ok = rx_reached(&bad->done, before, bad->slot);
                     __syncthreads();
-                    rx_sort_run<NT, K, XF>(x, y, s, e, pl.lo, inv, wt, cnt);
+                    if (!s_ok) return;
+                    int d = first;  // the byte
+                    for (unsigned c = 0; d < lo; d++)
+                        if (Rx<K>::dig(bits, d) != 0 && c++ == di) break;
+                    const bool swapped = di & 1;
+                    const unsigned tile = kind == 2 ? sub - nt - 16 : sub;
+                    const int64_t a = s + (int64_t)tile * LONG_T, b = a + LONG_T < e ? a + LONG_T : e;
+                    if (back) {
+                        for (int64_t i = a + tid; i < b; i += NT) x.st(i, y.ld(i));
+                    } else if (kind == 0) {
+                        rx_range_count<NT, K>(from(swapped), a, b, d, wt, cnt);
+                        if (tid < 256) table[(size_t)tid * nt + tile] = cnt[tid];
+                    } else if (kind == 1) {
+                        // a warp per value: inclusive sums of its tiles' counts
+                        CT* row = table + (size_t)((sub - nt) * W + (tid >> 5)) * nt;
+                        CT sum = 0;
+                        for (unsigned i0 = 0; i0 < nt; i0 += 32) {
+                            const unsigned i = i0 + (tid & 31);
+                            CT v = i < nt ? __ldcg(row + i) : (CT)0;
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const CT u = __shfl_up_sync(0xFFFFFFFFu, v, o);
+                                if ((tid & 31) >= o) v += u;
+                            }
+                            v += sum;
+                            if (i < nt) row[i] = v;
+                            sum = __shfl_sync(0xFFFFFFFFu, v, 31);
+                        }
+                    } else {
+                        unsigned long long mine = 0, all = 0;
+                        if (tid < 256) {
+                            const CT* row = table + (size_t)tid * nt;
+                            mine = tile ? (unsigned long long)__ldcg(row + tile - 1) : 0;
+                            all = (unsigned long long)__ldcg(row + nt - 1);
+                        }
+                        const unsigned long long ex = rx_exsum256(all, red);
+                        if (tid < 256) pos[tid] = (unsigned long long)s + ex + mine;
+                        __syncthreads();
+                        rx_range_scatter<NT, K>(from(swapped), into(swapped), a, b, e, d, wt, pos);
+                    }
                 }
+                __threadfence();
+                __syncthreads();
+                if (tid == 0) atomicAdd(&bad->done, 1u);
             }
         }
     }

@@ -47,7 +47,7 @@ template <typename K> struct Radix {
         int T;  // keys per tile
         int64_t nseg, tiles, chunk, chunks, fixes, S;  // (several segments: upper bounds)
         bool wide;     // 64-bit look-back words
-        size_t o_hist, o_done, o_ticket, o_misc, o_hits, o_tab, o_flags, o_lb0, zero_bytes, o_lb1, o_plan, o_at, o_tile,
+        size_t o_hist, o_done, o_ticket, o_misc, o_hits, o_tab, o_flags, o_started, o_lb0, zero_bytes, o_lb1, o_plan, o_at, o_tile,
             o_chunk, o_fix, o_data, total;
     };
     static Layout layout(const SortArgs& a)
@@ -78,7 +78,7 @@ template <typename K> struct Radix {
         o += align256((size_t)y.nseg * 4);
         y.o_ticket = o;
         o += 256;
-        y.o_misc = o;  // most passes, flagged tiles, totals
+        y.o_misc = o;  // most passes, counters, totals
         o += 256;
         y.o_hits = o;
         o += align256(sampled ? (size_t)y.nseg * RX_TRY * 4 : 0);
@@ -86,6 +86,8 @@ template <typename K> struct Radix {
         o += align256(sampled ? (size_t)many * RX_TRY * RX_SLOTS * 4 : 0);
         y.o_flags = o;
         o += align256((size_t)y.fixes);
+        y.o_started = o;
+        o += align256((size_t)y.fixes * 4);
         y.o_lb0 = o;
         o += lb;
         y.zero_bytes = o;  // everything up to here starts as zeros
@@ -166,8 +168,15 @@ template <typename K> struct Radix {
                 ProfScope ps_("radix_fix", s);
                 launch_next(ff, (unsigned)y.fixes, FN, fb, s, A);
             }
+            auto fl = k_rx_long<K, XF, CT>;
+            const size_t lb = std::max(TileBuf<K, 8>::type::bytes(FT), (size_t)(16 * 256 * 4 + 256 * 8 + 256 * 4 + 64));
+            // at most 1.5 rows per LONG_T keys, in the look-back tables of 1 row per tile
+            static_assert(3 * C::Large::T <= 2 * LONG_T && 3 * C::Mid::T <= 2 * LONG_T && 3 * C::Small::T <= 2 * LONG_T,
+                          "the digit table fits the look-back tables");
+            static_assert(sizeof(RxBad) * 2 * C::Large::T <= 1024 * FT, "and so does the list");
+            if ((e = smem_attr(fl, lb)) != cudaSuccess) return e;
             ProfScope ps_("radix_long", s);
-            launch_next(k_rx_long<K, XF>, (unsigned)grid_sms, 512, 0, s, A);
+            launch_next(fl, (unsigned)grid_sms, 512, lb, s, A);
         }
         return cudaGetLastError();
     }
@@ -207,9 +216,14 @@ template <typename K> struct Radix {
         A.nflag = (unsigned*)(ws + y.o_misc + 4);
         A.total = (int64_t*)(ws + y.o_misc + 8);
         A.descents = (unsigned*)(ws + y.o_misc + 32);
+        A.bads = (unsigned*)(ws + y.o_misc + 64);
         A.hits = (unsigned*)(ws + y.o_hits);
         A.tab = (unsigned*)(ws + y.o_tab);
         A.flags = (uint8_t*)(ws + y.o_flags);
+        A.started = (unsigned*)(ws + y.o_started);
+        // the look-back tables serve k_rx_long once the passes are over
+        A.dtab = ws + y.o_lb0;
+        A.bad = (RxBad*)(ws + y.o_lb1);
         A.keep = a.keep_order_keys;
         // a sort between two buffers, or one that leaves order keys, moves
         // (and transforms) the keys even when they are all equal
