@@ -257,7 +257,8 @@ int ps_last_cuda_error(void);
  * queue in arrival order; a worker thread admits the queue's head whenever a
  * stream slot is free, fewer than max_inflight requests are on the GPU and the
  * memory budget holds the request's cost (scratch for a copy of its keys plus
- * the sort's workspace).  Each admission round runs as one batched sort per
+ * the sort's workspace); requests admitted together are charged what their
+ * batched sorts take where that is more.  Each admission round runs as one batched sort per
  * (dtype, pivot mode) that reads every request from its own buffer and writes
  * the result back there (no gather or scatter copies), on one of several
  * server streams, so rounds admitted while others run overlap on the GPU.
@@ -320,6 +321,10 @@ int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode, ps_stream_
 int ps_debug_fail_alloc(int count);
 /* The same for `count` allocations after the next `skip` of them. */
 int ps_debug_fail_alloc_after(int skip, int count);
+/* As if the device had `bytes` for workspaces: an allocation fails with
+ * PS_ERR_NO_MEMORY when those taken since this call and not given back would
+ * exceed it (0 turns it off).  Call it while no sort is under way. */
+int ps_debug_limit_alloc(size_t bytes);
 
 /* ---- checked builds -------------------------------------------------------
  * A build compiled with -DPS_CHECKED (libpsort_checked.so) validates every

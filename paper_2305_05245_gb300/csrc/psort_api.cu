@@ -8,6 +8,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "psort_internal.h"
@@ -65,9 +66,21 @@ static bool take_one(std::atomic<int>& c)
     return false;
 }
 
+// Host-side limit (ps_debug_limit_alloc): allocations that would take the bytes
+// held beyond it fail.  What is held is only counted while a limit is set.
+static std::atomic<size_t> g_limit_alloc{0};
+static std::mutex g_held_mu;
+static std::unordered_map<void*, size_t> g_held;
+static size_t g_held_bytes = 0;
+
 int ws_alloc(void** p, size_t bytes, cudaStream_t s)
 {
     if (g_fail_alloc.load() > 0 && !take_one(g_skip_alloc) && take_one(g_fail_alloc)) return PS_ERR_NO_MEMORY;
+    const size_t limit = g_limit_alloc.load();
+    if (limit) {
+        std::lock_guard<std::mutex> lk(g_held_mu);
+        if (g_held_bytes + bytes > limit) return PS_ERR_NO_MEMORY;
+    }
     cudaMemPool_t pool;
     int rc = get_pool(&pool);
     if (rc != PS_OK) return rc;
@@ -76,12 +89,26 @@ int ws_alloc(void** p, size_t bytes, cudaStream_t s)
         cudaGetLastError();
         return fail_cuda(e);
     }
+    if (limit) {
+        std::lock_guard<std::mutex> lk(g_held_mu);
+        g_held[*p] = bytes;
+        g_held_bytes += bytes;
+    }
     return PS_OK;
 }
 
 void ws_free(void* p, cudaStream_t s)
 {
-    if (p) cudaFreeAsync(p, s);
+    if (!p) return;
+    if (g_limit_alloc.load()) {
+        std::lock_guard<std::mutex> lk(g_held_mu);
+        const auto it = g_held.find(p);
+        if (it != g_held.end()) {
+            g_held_bytes -= it->second;
+            g_held.erase(it);
+        }
+    }
+    cudaFreeAsync(p, s);
 }
 
 // ---- profiling records
@@ -640,6 +667,34 @@ static int batch_launch(const BatchPlan& bp, const int64_t* dev_table, void* key
     return rc;
 }
 
+// Workspace of a plan's launches, which follow one another: the largest bin's.
+static size_t plan_ws_bytes(const BatchPlan& bp, int* rc)
+{
+    const bool narrow = narrow_dtype(bp.dtype);
+    size_t ws = 0;
+    for (const BatchBin& bb : bp.bins) {
+        if (bb.front || bb.cluster) continue;
+        const SortArgs a = batch_bin_args(bp, bb, nullptr, nullptr, nullptr);
+        if (bb.radix) {
+            ws = std::max(ws, narrow ? radix_bytes_u32(a) : radix_bytes_u64(a));
+            continue;
+        }
+        int src = PS_OK;
+        const ShapeEntry* sh = shape_of(bp.dtype, a.items, a.threads, &src);
+        if (src != PS_OK && *rc == PS_OK) *rc = src;
+        ws = std::max(ws, sh ? sh->ws(a) : narrow ? ws_bytes_args_u32(a) : ws_bytes_args_u64(a));
+    }
+    return ws;
+}
+
+size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const std::vector<void*>* own)
+{
+    BatchPlan bp;
+    int rc = batch_make_plan(off, dtype, mode, nullptr, &bp, own);
+    if (rc != PS_OK) return 0;
+    return bp.table.size() * 8 + plan_ws_bytes(bp, &rc);
+}
+
 // Batched sort of the segments [off[i], off[i+1]) of `keys` (host offsets):
 // bins by length, one multi-instance pipeline per bin, queued on s.
 int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
@@ -1045,19 +1100,7 @@ int ps_batch_plan_create(const int64_t* host_seg_offsets, int64_t n_segs, int dt
     ps_batch_plan* p = new (std::nothrow) ps_batch_plan();
     if (!p) return PS_ERR_NO_MEMORY;
     int rc = batch_make_plan(off, dtype, pivot_mode, nullptr, &p->plan);
-    size_t ws = 0;
-    for (const BatchBin& bb : p->plan.bins) {
-        if (bb.front || bb.cluster) continue;
-        SortArgs a = batch_bin_args(p->plan, bb, nullptr, nullptr, nullptr);
-        int src = PS_OK;
-        if (bb.radix) {
-            ws = std::max(ws, narrow_dtype(dtype) ? radix_bytes_u32(a) : radix_bytes_u64(a));
-            continue;
-        }
-        const ShapeEntry* sh = shape_of(dtype, a.items, a.threads, &src);
-        if (src != PS_OK && rc == PS_OK) rc = src;
-        ws = std::max(ws, sh ? sh->ws(a) : narrow_dtype(dtype) ? ws_bytes_args_u32(a) : ws_bytes_args_u64(a));
-    }
+    const size_t ws = plan_ws_bytes(p->plan, &rc);
     cudaError_t e = cudaSuccess;
     if (rc == PS_OK && !p->plan.table.empty()) {
         e = cudaMalloc((void**)&p->table, p->plan.table.size() * 8);
@@ -1277,6 +1320,15 @@ int ps_debug_fail_alloc_after(int skip, int count)
     g_fail_alloc.store(0);
     g_skip_alloc.store(skip);
     g_fail_alloc.store(count);
+    return PS_OK;
+}
+
+int ps_debug_limit_alloc(size_t bytes)
+{
+    std::lock_guard<std::mutex> lk(g_held_mu);
+    g_held.clear();
+    g_held_bytes = 0;
+    g_limit_alloc.store(bytes);
     return PS_OK;
 }
 

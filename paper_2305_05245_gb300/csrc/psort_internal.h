@@ -113,6 +113,8 @@ int viol_read_radix_rec(unsigned long long* out);
 int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
                int64_t* pinned, size_t pinned_cap, const ps_params* force = nullptr,
                const std::vector<void*>* own = nullptr);
+// Device bytes that batch_sort takes for such a call (instance table and workspace).
+size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const std::vector<void*>* own);
 // The size heuristic alone (no tuned entries), with every field automatic.
 void resolve_default(int64_t n, int dtype, ps_params* out);
 // Records (uint64 key, uint32 payload) through the validated record path.

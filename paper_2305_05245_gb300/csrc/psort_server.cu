@@ -112,6 +112,33 @@ struct Server {
         retire_with(r, r->status);
     }
 
+    // A round's requests of one (dtype, mode): one batched sort.
+    struct Group {
+        int dtype, mode;
+        std::vector<int64_t> off;
+        std::vector<void*> own;
+        size_t stage() const { return (size_t)off.back() * key_bytes(dtype); }
+    };
+    static std::vector<Group> groups(const std::vector<Req>& reqs)
+    {
+        std::vector<Group> gs;
+        for (const Req& q : reqs) {
+            size_t g = 0;
+            while (g < gs.size() && (gs[g].dtype != q.dtype || gs[g].mode != q.mode)) g++;
+            if (g == gs.size()) gs.push_back(Group{q.dtype, q.mode, {0}, {}});
+            gs[g].off.push_back(gs[g].off.back() + q.n);
+            gs[g].own.push_back(q.keys);
+        }
+        return gs;
+    }
+    // Device bytes a round takes: its groups follow one another on one stream.
+    static size_t round_bytes(const std::vector<Req>& reqs)
+    {
+        size_t most = 0;
+        for (const Group& g : groups(reqs)) most = std::max(most, g.stage() + batch_bytes(g.off, g.dtype, g.mode, &g.own));
+        return most;
+    }
+
     // Queue one round on its slot's stream: gather, batched sort, scatter.
     int launch(Round* r)
     {
@@ -140,30 +167,15 @@ struct Server {
         }
         size_t pin_at = 0;
         if (inject) rc = PS_ERR_CUDA;  // as if a launch had failed: nothing is queued
-        // group by (dtype, mode): each group is one batched sort
-        std::vector<bool> taken(r->reqs.size(), false);
-        for (size_t i = 0; i < r->reqs.size() && rc == PS_OK; i++) {
-            if (taken[i]) continue;
-            std::vector<size_t> grp;
-            for (size_t j = i; j < r->reqs.size(); j++)
-                if (!taken[j] && r->reqs[j].dtype == r->reqs[i].dtype && r->reqs[j].mode == r->reqs[i].mode) {
-                    grp.push_back(j);
-                    taken[j] = true;
-                }
-            const int dtype = r->reqs[i].dtype, mode = r->reqs[i].mode;
-            const size_t kb = key_bytes(dtype);
-            std::vector<int64_t> off(grp.size() + 1, 0);
-            for (size_t k = 0; k < grp.size(); k++) off[k + 1] = off[k] + r->reqs[grp[k]].n;
-            const int64_t total = off.back();
-            int64_t* pin = sl.pinned ? sl.pinned + pin_at : nullptr;
-            const size_t pin_cap = sl.pinned ? 3 * grp.size() + 1 : 0;
-            pin_at += 3 * grp.size() + 1;
-            std::vector<void*> own(grp.size());
-            for (size_t k = 0; k < grp.size(); k++) own[k] = r->reqs[grp[k]].keys;
-            void* stage = nullptr;  // the passes between the first and the last
-            rc = ws_alloc(&stage, (size_t)total * kb, st);
+        for (const Group& g : groups(r->reqs)) {
             if (rc != PS_OK) break;
-            rc = batch_sort(off, stage, dtype, mode, st, pin, pin_cap, nullptr, &own);
+            int64_t* pin = sl.pinned ? sl.pinned + pin_at : nullptr;
+            const size_t pin_cap = sl.pinned ? 3 * g.own.size() + 1 : 0;
+            pin_at += 3 * g.own.size() + 1;
+            void* stage = nullptr;  // the passes between the first and the last
+            rc = ws_alloc(&stage, g.stage(), st);
+            if (rc != PS_OK) break;
+            rc = batch_sort(g.off, stage, g.dtype, g.mode, st, pin, pin_cap, nullptr, &g.own);
             ws_free(stage, st);
         }
         r->status = rc;
@@ -254,6 +266,24 @@ struct Server {
                 r->cost += pending.front().cost;
                 r->reqs.push_back(pending.front());
                 pending.pop_front();
+            }
+            // Requests sorted together can take more than each alone (their share of
+            // a radix run's tables): the round is charged what it takes, and gives
+            // its last requests back to the queue until that fits the budget.
+            while (r->reqs.size() > 1) {
+                lk.unlock();
+                const size_t need = round_bytes(r->reqs);
+                lk.lock();
+                if (used + std::max(r->cost, need) <= budget) {
+                    r->cost = std::max(r->cost, need);
+                    break;
+                }
+                for (size_t k = (r->reqs.size() + 7) / 8; k > 0 && r->reqs.size() > 1; k--) {
+                    r->cost -= r->reqs.back().cost;
+                    pending_keys += r->reqs.back().n;
+                    pending.push_front(r->reqs.back());
+                    r->reqs.pop_back();
+                }
             }
             used += r->cost;
             inflight += (int)r->reqs.size();
