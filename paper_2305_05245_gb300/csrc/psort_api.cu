@@ -20,6 +20,7 @@ static thread_local int g_last_cuda = 0;
 int fail_cuda(cudaError_t e)
 {
     g_last_cuda = (int)e;
+    cudaGetLastError();  // the failure is reported here: later calls must not see it again
     if (e == cudaErrorMemoryAllocation) return PS_ERR_NO_MEMORY;
     return PS_ERR_CUDA;
 }
@@ -85,10 +86,7 @@ int ws_alloc(void** p, size_t bytes, cudaStream_t s)
     int rc = get_pool(&pool);
     if (rc != PS_OK) return rc;
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes ? bytes : 256, pool, s);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail_cuda(e);
-    }
+    if (e != cudaSuccess) return fail_cuda(e);
     if (limit) {
         std::lock_guard<std::mutex> lk(g_held_mu);
         g_held[*p] = bytes;
