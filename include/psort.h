@@ -326,6 +326,10 @@ int ps_debug_fail_alloc_after(int skip, int count);
  * exceed it (0 turns it off).  Call it while no sort is under way. */
 int ps_debug_limit_alloc(size_t bytes);
 
+/* As if the device could place thread-block clusters of at most `ctas` blocks
+ * (0 turns it off): sorts that need larger ones take another way. */
+int ps_debug_max_cluster(int ctas);
+
 /* ---- checked builds -------------------------------------------------------
  * A build compiled with -DPS_CHECKED (libpsort_checked.so) validates every
  * global and shared-memory index in its kernels; the first out-of-range

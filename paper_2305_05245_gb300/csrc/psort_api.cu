@@ -354,7 +354,7 @@ static bool one_block(const SortArgs& a)
 }
 static bool cluster_takes(const SortArgs& a)
 {
-    return one_block(a) && !a.keep_order_keys && a.n <= cluster_max(a.dtype);
+    return one_block(a) && !a.keep_order_keys && (a.n <= 8192 || a.n <= cluster_max(a.dtype));
 }
 static bool radix_takes(const SortArgs& a)
 {
@@ -1327,6 +1327,13 @@ int ps_debug_limit_alloc(size_t bytes)
     g_held.clear();
     g_held_bytes = 0;
     g_limit_alloc.store(bytes);
+    return PS_OK;
+}
+
+int ps_debug_max_cluster(int ctas)
+{
+    if (ctas < 0 || ctas > 16) return PS_ERR_INVALID_ARG;
+    cluster_debug_cap(ctas);
     return PS_OK;
 }
 

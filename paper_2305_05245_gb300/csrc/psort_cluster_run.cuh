@@ -42,6 +42,28 @@ template <typename K> struct ClusterSort {
         return cudaLaunchKernelEx(&cfg, f, j.src, j.dst, j.in, j.n_B, share, j.own, j.keep);
     }
 
+    // Whether a cluster of so many CTAs of the widest shape fits the current device.
+    static bool placeable(int ctas)
+    {
+        using SB = typename TileBuf<K, 8>::type;
+        auto f = k_cluster_sort<1024, 8, K, 0, TW, 16>;
+        const size_t sm = SB::bytes(8192) * 2 + 64;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3(1024);
+        cfg.dynamicSmemBytes = sm;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)ctas;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (smem_attr(f, sm, true) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, f, &cfg) == cudaSuccess) return n > 0;
+        cudaGetLastError();
+        return false;
+    }
+
     // Small shapes first: one CTA while a tile holds the keys, then clusters of 4
     // and 16 (more, shorter shares sort sooner: 16384 keys in 4 x 4096, not 2 x 8192).
     template <int XF> static cudaError_t run_xf(const Job& j, int64_t n)

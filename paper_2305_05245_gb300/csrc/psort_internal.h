@@ -147,8 +147,15 @@ size_t radix_bytes_u64(const SortArgs& a);
 // radix: 131072 int32 46 / 46 us, 98304 int64 60 / 62, 131072 int64 70 / 64, 65536
 // records 67 / 75, 66000 records 85 / 72).
 constexpr int64_t CLUSTER_MAX = 131072;
+// CTAs of the largest cluster of such a sort that the current device can place
+// (16, 8, 4, 2 or 1: a process may see fewer SMs of a GPC than 16).  Longer sorts
+// than the placeable clusters take go the way of longer sorts.
+int cluster_placeable();
+void cluster_debug_cap(int ctas);
 inline int64_t cluster_max(int dtype)
 {
+    const int c = cluster_placeable();
+    if (c < 16) return c >= 4 ? 16384 : 8192;
     return dtype < 0 ? 65536 : dtype == PS_I32 || dtype == PS_F32 || dtype == PS_U32 ? CLUSTER_MAX : 98304;
 }
 int run_cluster_u32(const SortArgs& a);

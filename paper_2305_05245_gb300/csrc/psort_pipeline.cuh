@@ -377,6 +377,7 @@ static inline bool cluster_fits(int64_t blocks, int64_t L)
     if (L > CLUSTER_MAX) return false;
     int64_t cs = 1;
     while (cs * 8192 < L) cs *= 2;
+    if (cs > 1 && cs > cluster_placeable()) return false;
     return blocks * cs <= (cs == 1 ? 152 : 2 * 152);
 }
 
