@@ -326,6 +326,9 @@ int ps_debug_fail_alloc_after(int skip, int count);
  * exceed it (0 turns it off).  Call it while no sort is under way. */
 int ps_debug_limit_alloc(size_t bytes);
 
+/* Looks at an earlier tile's counts before a wait of the radix sort gives up
+ * (negative: the default, some ten seconds; 0: at the first that fails). */
+int ps_debug_radix_spins(int looks);
 /* As if the device could place thread-block clusters of at most `ctas` blocks
  * (0 turns it off): sorts that need larger ones take another way. */
 int ps_debug_max_cluster(int ctas);
@@ -338,7 +341,9 @@ int ps_debug_max_cluster(int ctas);
  * with (site + 100 * kernel family, index, bound, CTA) if a violation was seen,
  * 0 if none, or a negative status.  An ordinary build reports one thing only:
  * site 90 (index = tile), a radix pass's bounded wait for an earlier tile that
- * gave up (it never does in a correct run; the sort's output is then wrong). */
+ * gave up (it never does in a correct run; the sort's output is then wrong, and
+ * ps_sort_host and the server's requests, which wait for the device, report
+ * PS_ERR_TIMEOUT). */
 int ps_debug_violation(uint64_t* out);
 
 /* ---- profiling (library-wide, off by default) ---------------------------

@@ -25,7 +25,8 @@ EXPORTS = ["ps_sort", "ps_sort_ex", "ps_sort_pairs", "ps_sort_host", "ps_resolve
            "ps_server_open", "ps_server_submit", "ps_server_poll", "ps_server_close", "ps_sort_struct",
            "ps_autotune", "ps_autotune_get", "ps_autotune_set", "ps_server_debug_fail",
            "ps_batch_plan_create", "ps_batch_run", "ps_batch_plan_destroy", "ps_debug_fail_alloc",
-           "ps_debug_fail_alloc_after", "ps_debug_limit_alloc", "ps_debug_max_cluster"]
+           "ps_debug_fail_alloc_after", "ps_debug_limit_alloc", "ps_debug_max_cluster",
+           "ps_debug_radix_spins"]
 
 PS_NOALLOC_MAX_KEYS = 1 << 20
 PS_NOALLOC_SCRATCH_BYTES = 12 << 20
@@ -105,6 +106,7 @@ def load(path: str | None = None):
     lib.ps_debug_fail_alloc_after.argtypes = [i32, i32]
     lib.ps_debug_limit_alloc.argtypes = [ctypes.c_size_t]
     lib.ps_debug_max_cluster.argtypes = [i32]
+    lib.ps_debug_radix_spins.argtypes = [i32]
     lib.ps_debug_violation.argtypes = [ctypes.POINTER(ctypes.c_uint64)]
     lib.ps_profile_enable.argtypes = [i32]
     lib.ps_profile_read.argtypes = [ctypes.POINTER(PsKernelStat), i32, ctypes.POINTER(i32)]
@@ -115,7 +117,8 @@ def load(path: str | None = None):
                  "ps_server_submit", "ps_server_poll", "ps_server_close", "ps_sort_struct", "ps_autotune",
                  "ps_autotune_get", "ps_autotune_set", "ps_server_debug_fail", "ps_batch_plan_create",
                  "ps_batch_run", "ps_batch_plan_destroy", "ps_debug_fail_alloc",
-                 "ps_debug_fail_alloc_after", "ps_debug_limit_alloc", "ps_debug_max_cluster"):
+                 "ps_debug_fail_alloc_after", "ps_debug_limit_alloc", "ps_debug_max_cluster",
+                 "ps_debug_radix_spins"):
         getattr(lib, name).restype = i32
     if path is None:
         _lib = lib

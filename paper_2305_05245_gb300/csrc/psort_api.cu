@@ -109,6 +109,37 @@ void ws_free(void* p, cudaStream_t s)
     cudaFreeAsync(p, s);
 }
 
+// Words of one page-locked allocation, handed out again once given back.
+static std::mutex g_err_mu;
+static std::vector<unsigned*> g_err_free;
+
+unsigned* err_word_take()
+{
+    constexpr size_t WORDS = 64, STEP = 64;
+    std::lock_guard<std::mutex> lk(g_err_mu);
+    if (g_err_free.empty()) {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, WORDS * STEP, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        for (size_t i = WORDS; i-- > 0;) g_err_free.push_back((unsigned*)((char*)p + i * STEP));
+    }
+    unsigned* w = g_err_free.back();
+    g_err_free.pop_back();
+    *(volatile unsigned*)w = 0;
+    return w;
+}
+void err_word_give(unsigned* w)
+{
+    if (!w) return;
+    std::lock_guard<std::mutex> lk(g_err_mu);
+    g_err_free.push_back(w);
+}
+
+static std::atomic<unsigned> g_spins{1u << 24};
+unsigned radix_spins() { return g_spins.load(std::memory_order_relaxed); }
+
 // ---- profiling records
 struct ProfRec {
     std::string name;
@@ -385,7 +416,7 @@ static int dispatch(SortArgs& a)
 }
 
 static int sort_common(void* keys, uint32_t* payload, int64_t n, int dtype, int mode, const ps_params* params,
-                       const ps_trace* trace, ps_stream_t stream)
+                       const ps_trace* trace, ps_stream_t stream, unsigned* err = nullptr)
 {
     if (n < 0) return PS_ERR_INVALID_ARG;
     if (dtype < -1 || dtype > PS_U64) return PS_ERR_UNSUPPORTED;
@@ -412,6 +443,7 @@ static int sort_common(void* keys, uint32_t* payload, int64_t n, int dtype, int 
     a.trace = trace;
     a.stream = (cudaStream_t)stream;
     a.free_blocks = free_params(params, trace);
+    a.err = err;
     return dispatch(a);
 }
 
@@ -625,7 +657,7 @@ static bool narrow_dtype(int dtype) { return dtype == PS_I32 || dtype == PS_F32 
 // workspace from the pool; otherwise every one runs on ws (cap bytes) and
 // nothing is allocated.
 static int batch_launch(const BatchPlan& bp, const int64_t* dev_table, void* keys, cudaStream_t s, char* ws,
-                        size_t cap)
+                        size_t cap, unsigned* err)
 {
     const bool narrow = narrow_dtype(bp.dtype);
     int rc = PS_OK;
@@ -650,6 +682,7 @@ static int batch_launch(const BatchPlan& bp, const int64_t* dev_table, void* key
     for (size_t i = 0; i < bp.bins.size() && rc == PS_OK; i++) {
         if (bp.bins[i].front) continue;
         SortArgs a = batch_bin_args(bp, bp.bins[i], dev_table, keys, s);
+        a.err = err;
         if (bp.bins[i].cluster) {
             rc = narrow ? run_cluster_u32(a) : run_cluster_u64(a);
         } else if (ws && a.radix) {
@@ -696,7 +729,7 @@ size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const s
 // Batched sort of the segments [off[i], off[i+1]) of `keys` (host offsets):
 // bins by length, one multi-instance pipeline per bin, queued on s.
 int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
-               int64_t* pinned, size_t pinned_cap, const ps_params* force, const std::vector<void*>* own)
+               int64_t* pinned, size_t pinned_cap, const ps_params* force, const std::vector<void*>* own, unsigned* err)
 {
     if ((int64_t)off.size() - 1 <= 0) return PS_OK;
     if (dtype < PS_I32 || dtype > PS_U64) return PS_ERR_UNSUPPORTED;
@@ -725,7 +758,7 @@ int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode,
         ws_free(dev, s);
         return fail_cuda(e);
     }
-    rc = batch_launch(bp, (const int64_t*)dev, keys, s, nullptr, 0);
+    rc = batch_launch(bp, (const int64_t*)dev, keys, s, nullptr, 0, err);
     ws_free(dev, s);
     return rc;
 }
@@ -923,8 +956,16 @@ static ps_params host_free_blocks(size_t bytes)
     return r;
 }
 
+// Zeroes the n words of p if a wait of the sorts before gave up (*err): blocks that are
+// not sorted must not reach the merge, whose ranges would leave its buffers.
+__global__ void __launch_bounds__(256) k_clear_lost(const unsigned* err, uint32_t* p, int64_t n)
+{
+    if (*(const volatile unsigned*)err == 0) return;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) p[i] = 0;
+}
+
 static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t n, int dtype, int mode,
-                          const ps_params& r, bool free_blocks, cudaStream_t s)
+                          const ps_params& r, bool free_blocks, cudaStream_t s, unsigned* err)
 {
     const int64_t nb = r.n_blocks, L = (n + nb - 1) / nb;
     const size_t kb = dtype_size(dtype);
@@ -980,8 +1021,13 @@ static int host_pipelined(const void* host_keys, void* mapped, void* d, int64_t 
             a.keys = (char*)d + k0 * kb;
             a.extent = L;
             a.radix = true;
+            a.err = err;
         }
         rc = dispatch(a);
+    }
+    if (e == cudaSuccess && rc == PS_OK && free_blocks) {
+        k_clear_lost<<<152, 256, 0, s>>>(err, (uint32_t*)d, n * (int64_t)(kb / 4));
+        e = cudaGetLastError();
     }
     void* d2 = nullptr;  // the final merge's device output (exact splitting)
     if (e == cudaSuccess && rc == PS_OK && mode == PS_PIVOT_EXACT && PS_HOST_RANGES > 1) {
@@ -1121,7 +1167,7 @@ int ps_batch_run(const ps_batch_plan* plan, void* keys, ps_stream_t stream)
     if (!plan) return PS_ERR_INVALID_ARG;
     if (plan->plan.table.empty()) return PS_OK;
     if (!keys || (uintptr_t)keys % (narrow_dtype(plan->plan.dtype) ? 4 : 8) != 0) return PS_ERR_INVALID_ARG;
-    return batch_launch(plan->plan, plan->table, keys, (cudaStream_t)stream, plan->ws, plan->ws_bytes);
+    return batch_launch(plan->plan, plan->table, keys, (cudaStream_t)stream, plan->ws, plan->ws_bytes, nullptr);
 }
 
 int ps_batch_plan_destroy(ps_batch_plan* plan)
@@ -1162,11 +1208,12 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode, const ps
     cudaError_t e = cudaSuccess;
     ps_params r;
     resolve(n, dtype, params, &r);
+    unsigned* err = n > cluster_max(dtype) ? err_word_take() : nullptr;
     const bool free_blocks = free_params(params, nullptr) && r.merge_variant == PS_MERGE_TREE;
-    if (mapped && free_blocks && bytes >= HOST_FREE_MIN) {
-        rc = host_pipelined(host_keys, mapped, d, n, dtype, PS_PIVOT_EXACT, host_free_blocks(bytes), true, s);
+    if (mapped && free_blocks && bytes >= HOST_FREE_MIN && err) {
+        rc = host_pipelined(host_keys, mapped, d, n, dtype, PS_PIVOT_EXACT, host_free_blocks(bytes), true, s, err);
     } else if (mapped && !free_blocks && r.n_blocks > 1 && n >= HOST_PIPE_MIN) {
-        rc = host_pipelined(host_keys, mapped, d, n, dtype, pivot_mode, r, false, s);
+        rc = host_pipelined(host_keys, mapped, d, n, dtype, pivot_mode, r, false, s, err);
     } else if (mapped && !(free_blocks && n > cluster_max(dtype))) {
         SortArgs a;
         a.keys = d;
@@ -1188,16 +1235,19 @@ int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode, const ps
     } else {
         e = cudaMemcpyAsync(d, host_keys, bytes, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) {
-            rc = sort_common(d, nullptr, n, dtype, pivot_mode, params, nullptr, stream);
+            rc = sort_common(d, nullptr, n, dtype, pivot_mode, params, nullptr, stream, err);
             if (rc == PS_OK) e = cudaMemcpyAsync(host_keys, d, bytes, cudaMemcpyDeviceToHost, s);
         }
     }
     ws_free(d, s);
-    if (e != cudaSuccess) return fail_cuda(e);
-    if (rc != PS_OK) return rc;
-    e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return fail_cuda(e);
-    return PS_OK;
+    if (e != cudaSuccess) rc = fail_cuda(e);
+    if (rc == PS_OK || err) {  // (after a failure, sorts that were queued may still write *err)
+        e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess && rc == PS_OK) rc = fail_cuda(e);
+    }
+    if (err && *(volatile unsigned*)err && rc == PS_OK) rc = PS_ERR_TIMEOUT;
+    err_word_give(err);
+    return rc;
 }
 
 int ps_resolve_params(int64_t n, int dtype, const ps_params* in, ps_params* out)
@@ -1327,6 +1377,12 @@ int ps_debug_limit_alloc(size_t bytes)
     g_held.clear();
     g_held_bytes = 0;
     g_limit_alloc.store(bytes);
+    return PS_OK;
+}
+
+int ps_debug_radix_spins(int looks)
+{
+    g_spins.store(looks < 0 ? 1u << 24 : (unsigned)looks);
     return PS_OK;
 }
 

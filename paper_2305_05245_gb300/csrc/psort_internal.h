@@ -66,12 +66,20 @@ struct SortArgs {
     bool free_blocks = false;
     // Several instances, each sorted as one block by radix.
     bool radix = false;
+    // Host word the device can write: set when a bounded wait of the radix sort gave up.
+    unsigned* err = nullptr;
 };
 
 // Workspace from the library's stream-ordered pool.
 int ws_alloc(void** p, size_t bytes, cudaStream_t s);
 void ws_free(void* p, cudaStream_t s);
 int fail_cuda(cudaError_t e);
+// A zeroed word of page-locked host memory that kernels can write (SortArgs::err);
+// nullptr if there is no memory for it.
+unsigned* err_word_take();
+void err_word_give(unsigned* w);
+// Looks at one predecessor before a wait of the radix sort gives up (some ten seconds).
+unsigned radix_spins();
 
 // Profiling: when enabled (ps_profile_enable), a ProfScope records a CUDA
 // event before and after the launch it brackets.
@@ -112,7 +120,7 @@ int viol_read_radix_rec(unsigned long long* out);
 // table then holds 3 int64 per segment instead of 2.
 int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
                int64_t* pinned, size_t pinned_cap, const ps_params* force = nullptr,
-               const std::vector<void*>* own = nullptr);
+               const std::vector<void*>* own = nullptr, unsigned* err = nullptr);
 // Device bytes that batch_sort takes for such a call (instance table and workspace).
 size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const std::vector<void*>* own);
 // The size heuristic alone (no tuned entries), with every field automatic.

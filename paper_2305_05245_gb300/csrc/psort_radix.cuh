@@ -160,6 +160,9 @@ template <typename K> struct RxArgs {
     RxBad* bad;              // [2 * fix tiles]: the list
     unsigned* bads;          // [4]: its entries, rows of dtab given out; listing tasks taken and finished
     void* dtab;              // digit table, 256 counts a row (CT)
+    unsigned rows;           // its size
+    unsigned spins;          // looks in vain at one predecessor (or count) before a wait gives up
+    unsigned* err;           // set when one did (host memory, where someone waits for the sort)
     int min_pass;            // least number of passes (a sort between two buffers needs some)
     bool keep;               // the last pass leaves order keys
 };
@@ -207,9 +210,16 @@ template <int XF> __device__ __forceinline__ Rec rx_ld_digits(const GBuf<Rec>& b
     return g0 < 4 ? Rec{0, b.p[i]} : Rec{b.k[i], 0};
 }
 
-// The first look-back wait that gave up (tile + 1), recorded like an index
-// violation; 0 in every correct run.
+// The first wait that gave up (its tile + 1), recorded like an index violation;
+// 0 in every correct run.
 static __device__ unsigned long long rx_stall;
+// A wait gave up: the result is wrong, and whoever waits for the sort is told.  (The
+// kernels after it stay inside their buffers whatever order the keys are in.)
+template <typename K> __device__ __forceinline__ void rx_give_up(const RxArgs<K>& A, unsigned long long what)
+{
+    atomicExch(&rx_stall, what + 1);
+    *(volatile unsigned*)A.err = 1;
+}
 
 // ------------------------------------------------------------ sampling
 // How many low bytes the passes may leave out (64-bit keys and records).
@@ -612,8 +622,6 @@ template <typename K, typename CT, int NT, int E> constexpr size_t rx_smem()
     return RxTile<K>::bytes(NT * E) + (NT / 32) * 1024 + 256 * sizeof(CT) + 64;
 }
 
-constexpr unsigned RX_SPINS = 1u << 24;  // looks at one predecessor before a wait gives up
-
 // One digit pass.  Persistent CTAs take tiles in order from a counter, so
 // every tile before a waiting one is running or done and the look-back ends.
 //
@@ -797,12 +805,13 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
                     for (int q = 0; q < LB; q++) {
                         if (!more) break;
                         if ((v[q] & Lb<CT>::FLAGS) == 0) {
-                            if (++spins > RX_SPINS) {
-                                atomicExch(&rx_stall, (unsigned long long)tile + 1);
+                            if (++spins > A.spins) {
+                                rx_give_up(A, (unsigned long long)tile);
                                 more = false;
                             }
                             break;
                         }
+                        spins = 0;
                         excl += v[q] & ~Lb<CT>::FLAGS;
                         p -= 256;
                         left--;
@@ -1039,7 +1048,7 @@ template <typename F> __device__ __forceinline__ int64_t rx_search(int64_t a, in
 // its tiles comes first.
 template <typename K, typename LD>
 __device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, unsigned flag, int seg, unsigned* started,
-                                        RxBad* bad, unsigned* nbad, unsigned* nslot)
+                                        RxBad* bad, unsigned* bads, unsigned maxrows)
 {
     const typename Rx<K>::M m = Rx<K>::mask(lo, Rx<K>::D - 1);
     const int64_t t1 = t0 + FT < len ? t0 + FT : len;
@@ -1049,7 +1058,9 @@ __device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, 
     auto list = [&](int64_t s, int64_t e, int inside) {
         if (!one) return;
         const unsigned rows = e - s > LONG_ONE ? (unsigned)((e - s + LONG_T - 1) / LONG_T) : 0;
-        bad[atomicAdd(nbad, 1u)] = RxBad{s, e, seg, inside, rows ? atomicAdd(nslot, rows) : 0u, 0, 0, 0, 0};
+        const unsigned slot = rows ? atomicAdd(bads + 1, rows) : 0u;
+        if ((unsigned long long)slot + rows > maxrows) return;  // (only of keys that an abandoned wait left out of order)
+        bad[atomicAdd(bads, 1u)] = RxBad{s, e, seg, inside, slot, 0, 0, 0, 0};
     };
     auto spans = [&](int64_t s, int64_t e) {
         const unsigned was = one ? atomicExch(&started[s / FT], 1u) : 0;
@@ -1060,7 +1071,7 @@ __device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, 
     const int64_t in = t0 > 0 && Rx<K>::same(ld(t0 - 1), head, m) ? rx_search(t0, t1, upto(head)) : t0;
     if (flag & 1) spans(rx_search(0, t0, below(head)), in < t1 ? in : rx_search(t1, len, upto(head)));
     const int64_t out = t1 < len && Rx<K>::same(ld(t1), tail, m) ? rx_search(in, t1, below(tail)) : t1;
-    if (flag & 2) spans(out, rx_search(t1, len, upto(tail)));
+    if ((flag & 2) && out < t1) spans(out, rx_search(t1, len, upto(tail)));
     if (flag & 4) list(in, out, 1);
 }
 // The bits in which a key differs from another, and the same as a key.
@@ -1204,16 +1215,15 @@ __device__ __forceinline__ void rx_range_scatter(LD ld, ST st, int64_t a, int64_
     __syncthreads();
 }
 
-// Waits until *done reaches `need` (thread 0; bounded).
-__device__ __forceinline__ bool rx_reached(const unsigned* done, unsigned need, unsigned long long what)
+// Waits until *done reaches `need` (one thread; at most so many looks).
+__device__ __forceinline__ bool rx_reached(const unsigned* done, unsigned need, unsigned looks)
 {
-    for (unsigned spins = 0; spins <= RX_SPINS; spins++) {
+    for (unsigned spins = 0; spins <= looks; spins++) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
         if (v >= need) return true;
         __nanosleep(100);
     }
-    atomicExch(&rx_stall, what + 1);
     return false;
 }
 
@@ -1266,6 +1276,16 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
         x = rx_global(A.iptr ? rx_own(A.iptr, (int64_t)q.seg, 0, len) : rx_sub(A.last, off, len));
         y = rx_global(rx_sub(A.b, off, len));
     };
+    auto reached = [&](const unsigned* done, unsigned need, unsigned what) {
+        if (tid == 0) {
+            s_ok = rx_reached(done, need, A.spins);
+            if (!s_ok) rx_give_up(A, what);
+        }
+        __syncthreads();
+        const bool ok = s_ok;
+        __syncthreads();
+        return ok;
+    };
     // keys of x, or of y once they are swapped
     auto from = [&](bool swapped) {
         return [&, swapped](int64_t i) {
@@ -1298,15 +1318,13 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
                 q.seg = A.nseg == 1 ? 0 : A.fix_seg[f];
                 const int fix0 = rx_at(A, q.seg).fix0;
                 open(q);
-                rx_list<K>(from(false), len, (f - fix0) * FT, lo, flag, q.seg, A.started + fix0, A.bad, A.bads, A.bads + 1);
+                rx_list<K>(from(false), len, (f - fix0) * FT, lo, flag, q.seg, A.started + fix0, A.bad, A.bads, A.rows);
             }
             __threadfence();
             __syncthreads();
             if (tid == 0) atomicAdd(&A.bads[3], 1u);
         }
-        if (tid == 0) s_ok = rx_reached(&A.bads[3], tasks, ~0ull - 1);
-        __syncthreads();
-        if (!s_ok) return;
+        if (!reached(&A.bads[3], tasks, tasks)) return;
     }
     const unsigned nbad = __ldcg(A.bads);
     for (unsigned r = blockIdx.x; r < nbad; r += gridDim.x) {
@@ -1375,9 +1393,7 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
                     rx_range_bits<NT, K>(ld, a, b, ld(s), &bad->dk, &bad->dp);
                 } else {
                     if (digits < 0) {
-                        if (tid == 0) s_ok = rx_reached(&bad->done, nt, bad->slot);
-                        __syncthreads();
-                        if (!s_ok) return;
+                        if (!reached(&bad->done, nt, bad->slot)) return;
                         bits = rx_bits<K>(__ldcg(&bad->dk), __ldcg(&bad->dp));
                         digits = 0;
                         for (int d = first; d < lo; d++) digits += Rx<K>::dig(bits, d) != 0;
@@ -1388,9 +1404,7 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
                     if ((int)di > digits || (back && (!(digits & 1) || sub >= nt))) break;
                     const unsigned kind = back || sub < nt ? 0 : sub < nt + 16 ? 1 : 2;
                     const unsigned before = nt + di * per + (kind == 0 ? 0 : kind == 1 ? nt : nt + 16);
-                    if (tid == 0) s_ok = rx_reached(&bad->done, before, bad->slot);
-                    __syncthreads();
-                    if (!s_ok) return;
+                    if (!reached(&bad->done, before, bad->slot)) return;
                     int d = first;  // the byte
                     for (unsigned c = 0; d < lo; d++)
                         if (Rx<K>::dig(bits, d) != 0 && c++ == di) break;

@@ -223,7 +223,10 @@ template <typename K> struct Radix {
         A.started = (unsigned*)(ws + y.o_started);
         // the look-back tables serve k_rx_long once the passes are over
         A.dtab = ws + y.o_lb0;
+        A.rows = (unsigned)std::min<int64_t>(y.tiles, 0x7FFFFFFF);
         A.bad = (RxBad*)(ws + y.o_lb1);
+        A.spins = radix_spins();
+        A.err = a.err ? a.err : (unsigned*)(ws + y.o_misc + 40);
         A.keep = a.keep_order_keys;
         // a sort between two buffers, or one that leaves order keys, moves
         // (and transforms) the keys even when they are all equal

@@ -59,6 +59,7 @@ struct Slot {
     Round* cur = nullptr;       // the slot's last round (kept until replaced)
     int64_t* pinned = nullptr;  // page-locked staging of the round's instance tables
     size_t pinned_cap = 0;      // in int64
+    unsigned* err = nullptr;    // set by a kernel of the round whose bounded wait gave up
 };
 
 struct Done {
@@ -109,7 +110,9 @@ struct Server {
     static void CUDART_CB retire(void* p)
     {
         Round* r = (Round*)p;
-        retire_with(r, r->status);
+        const unsigned* err = r->srv->slots[r->slot].err;
+        const bool gave_up = err && *(volatile const unsigned*)err;
+        retire_with(r, r->status == PS_OK && gave_up ? PS_ERR_TIMEOUT : r->status);
     }
 
     // A round's requests of one (dtype, mode): one batched sort.
@@ -166,6 +169,7 @@ struct Server {
             else sl.pinned = nullptr;
         }
         size_t pin_at = 0;
+        if (sl.err) *(volatile unsigned*)sl.err = 0;  // (the slot's last round has retired)
         if (inject) rc = PS_ERR_CUDA;  // as if a launch had failed: nothing is queued
         for (const Group& g : groups(r->reqs)) {
             if (rc != PS_OK) break;
@@ -175,7 +179,7 @@ struct Server {
             void* stage = nullptr;  // the passes between the first and the last
             rc = ws_alloc(&stage, g.stage(), st);
             if (rc != PS_OK) break;
-            rc = batch_sort(g.off, stage, g.dtype, g.mode, st, pin, pin_cap, nullptr, &g.own);
+            rc = batch_sort(g.off, stage, g.dtype, g.mode, st, pin, pin_cap, nullptr, &g.own, sl.err);
             ws_free(stage, st);
         }
         r->status = rc;
@@ -327,6 +331,7 @@ int ps_server_open(size_t mem_budget_bytes, int max_inflight, ps_server** out)
         delete p;
         return fail_cuda(e);
     }
+    for (Slot& sl : s.slots) sl.err = err_word_take();
     s.worker = std::thread([&s] { s.run(); });
     *out = p;
     return PS_OK;
@@ -401,6 +406,7 @@ int ps_server_close(ps_server* p)
             cudaStreamDestroy(s.slots[i].stream);
         }
         if (s.slots[i].pinned) cudaFreeHost(s.slots[i].pinned);
+        err_word_give(s.slots[i].err);
         delete s.slots[i].cur;
     }
     delete p;

@@ -52,15 +52,17 @@ __global__ void __launch_bounds__(NT) k_struct_split(const W* rec, W* copy, int6
 }
 
 // records[i] = copy[pos[i]], W-sized words (8 or 16 bytes), one thread per
-// word of the output (coalesced stores; each record is read contiguously).
+// word of the output (coalesced stores; each record is read contiguously).  A
+// position is below n unless the sort before lost keys (a wait that gave up).
 template <typename W>
-__global__ void k_struct_gather(const W* copy, W* rec, const uint32_t* pos, int64_t words_total, int words)
+__global__ void k_struct_gather(const W* copy, W* rec, const uint32_t* pos, int64_t words_total, int words, uint32_t n)
 {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < words_total;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / words;
         const int w = (int)(t - i * words);
-        rec[t] = copy[(int64_t)pos[i] * words + w];
+        const uint32_t at = pos[i];
+        rec[t] = copy[(int64_t)(at < n ? at : 0) * words + w];
     }
 }
 
@@ -103,9 +105,9 @@ int struct_sort(void* records, int64_t n, int64_t rb, int64_t ko, int mode, cons
         if (rc == PS_OK) {
             ProfScope ps_("struct_gather", s);
             if (wide)
-                k_struct_gather<uint4><<<grid_for(wt), 256, 0, s>>>((const uint4*)ws, (uint4*)records, pos, wt, words);
+                k_struct_gather<uint4><<<grid_for(wt), 256, 0, s>>>((const uint4*)ws, (uint4*)records, pos, wt, words, (uint32_t)n);
             else
-                k_struct_gather<uint64_t><<<grid_for(wt), 256, 0, s>>>((const uint64_t*)ws, (uint64_t*)records, pos, wt, words);
+                k_struct_gather<uint64_t><<<grid_for(wt), 256, 0, s>>>((const uint64_t*)ws, (uint64_t*)records, pos, wt, words, (uint32_t)n);
             e = cudaGetLastError();
         }
     }
