@@ -60,6 +60,7 @@ static int get_pool(cudaMemPool_t* out)
 // after g_skip_alloc more workspace allocations the next g_fail_alloc of them
 // fail with PS_ERR_NO_MEMORY before any CUDA call.
 static std::atomic<int> g_skip_alloc{0}, g_fail_alloc{0};
+static thread_local bool g_injected = false;  // this thread's last allocation failed so
 static bool take_one(std::atomic<int>& c)
 {
     for (int k = c.load(); k > 0;)
@@ -76,7 +77,8 @@ static size_t g_held_bytes = 0;
 
 int ws_alloc(void** p, size_t bytes, cudaStream_t s)
 {
-    if (g_fail_alloc.load() > 0 && !take_one(g_skip_alloc) && take_one(g_fail_alloc)) return PS_ERR_NO_MEMORY;
+    g_injected = g_fail_alloc.load() > 0 && !take_one(g_skip_alloc) && take_one(g_fail_alloc);
+    if (g_injected) return PS_ERR_NO_MEMORY;
     const size_t limit = g_limit_alloc.load();
     if (limit) {
         std::lock_guard<std::mutex> lk(g_held_mu);
@@ -404,8 +406,14 @@ static int dispatch(SortArgs& a)
     if (rc != PS_OK) return rc;
     if (cluster_takes(a))
         return a.dtype < 0 ? run_cluster_rec(a) : tune_family(a.dtype) == 0 ? run_cluster_u32(a) : run_cluster_u64(a);
-    if (radix_takes(a))
-        return a.dtype < 0 ? run_radix_rec(a) : tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
+    if (radix_takes(a)) {
+        rc = a.dtype < 0 ? run_radix_rec(a) : tune_family(a.dtype) == 0 ? run_radix_u32(a) : run_radix_u64(a);
+        // its tables take more than the merges' at most sizes (2^30 keys, bytes a key: 0.33
+        // against 0.08 for 32 bits, 0.45 against 0.18 for 64, 0.67 against 0.37 for
+        // records): where they do not fit, the merges may
+        if (rc != PS_ERR_NO_MEMORY || g_injected || a.inst_base) return rc;
+        rc = PS_OK;
+    }
     if (sh) return sh->run(a);
     switch (a.dtype) {
     case PS_I32: case PS_F32: case PS_U32: return run_sort_u32(a);
@@ -535,9 +543,10 @@ static constexpr int64_t BATCH_CLUSTER_CTAS = 176;
 static int64_t cluster_ctas(int64_t n) { return n <= 8192 ? 1 : n <= 16384 ? 4 : 16; }
 
 // own (optional): one device pointer per segment; segment i then lives in its
-// own buffer, and off only lays the segments out for the workspace.
+// own buffer, and off only lays the segments out for the workspace.  radix: long
+// segments may take the radix run.
 static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode, const ps_params* force,
-                           BatchPlan* bp, const std::vector<void*>* own = nullptr)
+                           BatchPlan* bp, const std::vector<void*>* own = nullptr, bool radix = true)
 {
     const int64_t n_segs = (int64_t)off.size() - 1;
     if (dtype < PS_I32 || dtype > PS_U64) return PS_ERR_UNSUPPORTED;
@@ -563,11 +572,11 @@ static int batch_make_plan(const std::vector<int64_t>& off, int dtype, int mode,
         int b = 1;
         if (len <= SMALL_SEG) b = 0;
         while (len > (tile << (b - 1)) && b > 0) b++;
-        if (!force && len > rmin) b = (int)bins.size() - 1;
+        if (!force && radix && len > rmin) b = (int)bins.size() - 1;
         bins[b].push_back(i);
         sum[b] += len;
     }
-    if (!force) {
+    if (!force && radix) {
         const size_t last = bins.size() - 1;
         int few = 0;
         for (size_t b = 2; b < last; b++) few += sum[b] > 0 && sum[b] <= BATCH_FEW_ALONE;
@@ -728,15 +737,15 @@ size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const s
 
 // Batched sort of the segments [off[i], off[i+1]) of `keys` (host offsets):
 // bins by length, one multi-instance pipeline per bin, queued on s.
-int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
-               int64_t* pinned, size_t pinned_cap, const ps_params* force, const std::vector<void*>* own, unsigned* err)
+static int batch_sort_as(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s, int64_t* pinned,
+                         size_t pinned_cap, const ps_params* force, const std::vector<void*>* own, unsigned* err, bool radix)
 {
     if ((int64_t)off.size() - 1 <= 0) return PS_OK;
     if (dtype < PS_I32 || dtype > PS_U64) return PS_ERR_UNSUPPORTED;
     if (!keys) return PS_ERR_INVALID_ARG;
     if ((uintptr_t)keys % (narrow_dtype(dtype) ? 4 : 8) != 0) return PS_ERR_INVALID_ARG;
     BatchPlan bp;
-    int rc = batch_make_plan(off, dtype, mode, force, &bp, own);
+    int rc = batch_make_plan(off, dtype, mode, force, &bp, own, radix);
     if (rc != PS_OK) return rc;
     const size_t total = bp.table.size();
     if (total == 0) return PS_OK;
@@ -760,6 +769,17 @@ int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode,
     }
     rc = batch_launch(bp, (const int64_t*)dev, keys, s, nullptr, 0, err);
     ws_free(dev, s);
+    return rc;
+}
+
+int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode, cudaStream_t s,
+               int64_t* pinned, size_t pinned_cap, const ps_params* force, const std::vector<void*>* own, unsigned* err)
+{
+    int rc = batch_sort_as(off, keys, dtype, mode, s, pinned, pinned_cap, force, own, err, true);
+    // as in dispatch; bins that are sorted already are sorted once more (pinned may
+    // still be read by the first table's copy)
+    if (rc == PS_ERR_NO_MEMORY && !g_injected && !force)
+        rc = batch_sort_as(off, keys, dtype, mode, s, nullptr, 0, force, own, err, false);
     return rc;
 }
 
@@ -1143,15 +1163,24 @@ int ps_batch_plan_create(const int64_t* host_seg_offsets, int64_t n_segs, int dt
     if (off.empty()) off.push_back(0);
     ps_batch_plan* p = new (std::nothrow) ps_batch_plan();
     if (!p) return PS_ERR_NO_MEMORY;
-    int rc = batch_make_plan(off, dtype, pivot_mode, nullptr, &p->plan);
-    const size_t ws = plan_ws_bytes(p->plan, &rc);
+    int rc = PS_OK;
     cudaError_t e = cudaSuccess;
-    if (rc == PS_OK && !p->plan.table.empty()) {
+    for (const bool radix : {true, false}) {  // (without: as in dispatch)
+        rc = batch_make_plan(off, dtype, pivot_mode, nullptr, &p->plan, nullptr, radix);
+        const size_t ws = plan_ws_bytes(p->plan, &rc);
+        if (rc != PS_OK || p->plan.table.empty()) break;
         e = cudaMalloc((void**)&p->table, p->plan.table.size() * 8);
         if (e == cudaSuccess)
             e = cudaMemcpy(p->table, p->plan.table.data(), p->plan.table.size() * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess && ws > 0) e = cudaMalloc((void**)&p->ws, ws);
         p->ws_bytes = ws;
+        if (e != cudaErrorMemoryAllocation) break;
+        if (radix) {
+            e = cudaSuccess;
+            cudaGetLastError();
+            if (p->table) cudaFree(p->table);
+            p->table = nullptr;
+        }
     }
     if (rc == PS_OK && e != cudaSuccess) rc = fail_cuda(e);
     if (rc != PS_OK) {
