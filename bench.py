@@ -169,6 +169,16 @@ def radix_passes(prof, workload: str):
     return ncu_traffic("radix_pass", workload, "active_launches_per_sort")
 
 
+def sorted_by(prof, nb, np_):
+    """What the timed sorts did, from their kernels: (method, n_B, n_P).  Sorts whose
+    blocks are the library's choice sort their input as one block, without pivots."""
+    if "radix_pass" in prof:
+        return "one block, radix digit passes (no pivots, nothing to merge)", 1, 1
+    if set(prof) == {"cluster_sort"}:
+        return "one block, one thread-block cluster (no pivots)", 1, 1
+    return "blocks, pivots and multiway merges", nb, np_
+
+
 def host_cpu():
     """nproc and the CPU model of this host (x86 "model name"; on Arm, lscpu's
     model name, else the implementer/part codes of /proc/cpuinfo)."""
@@ -615,7 +625,7 @@ def run_records(a):
         ach = per_launch / (dms / dl / 1e3) / 1e9
         roof = {"bound": "hbm", "kernel": dname, "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
                 "peak_source": src_peak, "traffic": None, "algorithmic_bytes_per_launch": per_launch}
-    nb, np_ = ps.resolve_params(n, -1, a.n_blocks, a.n_parts)
+    method, nb, np_ = sorted_by(prof, *ps.resolve_params(n, -1, a.n_blocks, a.n_parts))
     inblock = prof.get("merge_inblock", (0, 0))[0] // max(a.steps, 1)
     passes = None if "radix_pass" in prof else 2 + inblock
     line = {
@@ -624,7 +634,7 @@ def run_records(a):
         "dtype": "u64 key + u32 payload", "data": "synthetic (SplitMix64 keys, index payloads), resident in HBM",
         "config": {"workload": "single sort N=2^%d records (uint64 key, uint32 payload), %s splitting"
                                % (n.bit_length() - 1, a.pivot), "n": n, "n_blocks": nb, "n_parts": np_,
-                   "l2": "inputs larger than L2 (no flush needed)", "in_block_merge_passes": inblock},
+                   "sorted_by": method, "l2": "inputs larger than L2 (no flush needed)", "in_block_merge_passes": inblock},
         "roofline": roof,
         "sort_roofline": {"algorithmic_bytes_per_key": 48, "achieved_gbs": 48 * n / (ms / 1e3) / 1e9,
                           "frac": 48 * n / (ms / 1e3) / 1e9 / hbm, "passes_made": passes,
@@ -836,8 +846,9 @@ def main():
     keys = torch.empty_like(pristine)
     stream = torch.cuda.current_stream()
     tuned = False
-    if not a.no_autotune and not a.n_blocks and not a.n_parts and n >= (1 << 14):
-        # untimed: the library's autotuner picks n_B, n_P for this size
+    if not a.no_autotune and not a.n_blocks and not a.n_parts and n >= (1 << 14) and a.merge_variant != "tree":
+        # untimed: the library's autotuner picks n_B, n_P for this size (a plain sort
+        # is sorted as one block and reads no tuned entry)
         ps.autotune(a.dtype, a.pivot, n, n)
         tuned = True
     nb, np_ = ps.resolve_params(n, {"int32": 0, "int64": 1, "float32": 2, "float64": 3,
@@ -910,6 +921,7 @@ def main():
     s = BYTES[a.dtype]
     hbm, src_peak = peaks()
     launches = sum(v[0] for v in prof.values())
+    method, nb, np_ = sorted_by(prof, nb, np_)
     # dominant kernel by device time
     dom = max(prof.items(), key=lambda kv: kv[1][1]) if prof else ("none", (1, 1.0))
     dname, (dl, dms) = dom
@@ -942,8 +954,9 @@ def main():
         "data": "synthetic (SplitMix64, seeded), resident in HBM",
         "config": {"workload": wl, "n": n, "dist": a.dist, "pivot": a.pivot, "n_blocks": nb,
                    "n_parts": np_, "launch_shape": shape,
+                   "sorted_by": method,
                    "params": "autotuned (ps_autotune, untimed)" if tuned else
-                   ("explicit" if a.n_blocks or a.n_parts else "library defaults (measured size table)"),
+                   ("explicit" if a.n_blocks or a.n_parts else "automatic"),
                    "parallelism": "replicas" if world > 1 else "single GPU",
                    "l2": "inputs larger than L2 (no flush needed)",
                    "restore": "keys restored from a pristine device copy before each step, outside the timed events",
