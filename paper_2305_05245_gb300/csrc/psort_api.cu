@@ -261,8 +261,6 @@ static void resolve_heuristic(int64_t n, int dtype, const ps_params* in, ps_para
     *out = r;
 }
 
-void resolve_default(int64_t n, int dtype, ps_params* out) { resolve_heuristic(n, dtype, nullptr, out); }
-
 // Defaults measured on GB300 with ps_autotune (exact splitting, uniform keys):
 // (n_B, n_P) per round(log2 n) from 2^14 on, for single sorts and for the size
 // bins of batched sorts, 32-bit and 64-bit keys.  Up to 2^19-2^20 keys one
@@ -525,13 +523,7 @@ struct BatchPlan {
 // int32, k = 17: 1.21 / 1.35 ms, 18: 1.54 / 1.35, 21: 2.04 / 1.37; int64, k = 16:
 // 2.02 / 2.07, 17: 2.12 / 2.04, 21: 3.35 / 2.09.  (Up to these lengths one merge
 // pass after the tiles finishes a segment.)
-#ifndef PS_BATCH_RADIX32
-#define PS_BATCH_RADIX32 262144
-#endif
-#ifndef PS_BATCH_RADIX64
-#define PS_BATCH_RADIX64 131072
-#endif
-static int64_t batch_radix_min(int dtype) { return tune_family(dtype) == 0 ? PS_BATCH_RADIX32 : PS_BATCH_RADIX64; }
+static int64_t batch_radix_min(int dtype) { return tune_family(dtype) == 0 ? 262144 : 131072; }
 // Size bins of few keys below that cost their launches (75-110 us each).  They
 // join the radix run when there is one (2^23 keys add 0.17 ms to it) or when three
 // or more of them would run one by one; else a bin whose clusters fit the GPU at
@@ -958,7 +950,6 @@ static constexpr int64_t HOST_PIPE_MIN = int64_t(1) << 24;
 #define PS_HOST_RANGES 8   // partition ranges copied out while later ones merge
 #endif
 
-//
 // Blocks that are the library's choice (free) are as few as the transfers want:
 // one block per copy group, sorted by radix, and as many partitions, so that the
 // final merge has a small fan-in; both pivot modes then split exactly (the result

@@ -123,8 +123,6 @@ int batch_sort(const std::vector<int64_t>& off, void* keys, int dtype, int mode,
                const std::vector<void*>* own = nullptr, unsigned* err = nullptr);
 // Device bytes that batch_sort takes for such a call (instance table and workspace).
 size_t batch_bytes(const std::vector<int64_t>& off, int dtype, int mode, const std::vector<void*>* own);
-// The size heuristic alone (no tuned entries), with every field automatic.
-void resolve_default(int64_t n, int dtype, ps_params* out);
 // Records (uint64 key, uint32 payload) through the validated record path.
 int sort_records(uint64_t* keys, uint32_t* payload, int64_t n, int mode, const ps_params* params, cudaStream_t s);
 // Fixed-size records sorted by an embedded uint64 key (arguments validated).

@@ -52,11 +52,12 @@ static __device__ __noinline__ void ps_violation(int site, long long idx, long l
 #endif
 
 // ---------------------------------------------------------------- launches
-// First statement of every kernel: the library's kernels are launched with
-// programmatic stream serialization (launch_next), so a kernel's CTAs may be
+// First statement of every kernel that launch_next (or the cluster sort's launch)
+// starts: they allow programmatic stream serialization, so a kernel's CTAs may be
 // scheduled while the kernel before them ends; they wait here until all its work
 // is done and visible, and let the kernel after them be scheduled in turn.  Hides
-// launch latency between the many short kernels of a sort.
+// launch latency between the many short kernels of a sort.  (A kernel launched
+// without it, such as the record split, starts when the one before it has ended.)
 __device__ __forceinline__ void kernel_entry()
 {
     asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");

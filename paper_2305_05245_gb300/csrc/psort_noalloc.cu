@@ -98,9 +98,6 @@ extern "C" int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode,
     if (n <= 1) return PS_OK;
     const bool narrow = dtype == PS_I32 || dtype == PS_F32 || dtype == PS_U32;
     if (!keys || (uintptr_t)keys % (narrow ? 4 : 8) != 0) return PS_ERR_INVALID_ARG;
-    // the size heuristic, not tuned entries: the scratch is sized for it
-    ps_params r;
-    resolve_default(n, dtype, &r);
     void* ws = nullptr;
     int rc = noalloc_scratch(&ws);
     if (rc != PS_OK) return rc;
@@ -110,16 +107,11 @@ extern "C" int ps_sort_noalloc(void* keys, int64_t n, int dtype, int pivot_mode,
     a.n = n;
     a.dtype = dtype;
     a.mode = pivot_mode;
-    a.n_B = r.n_blocks;
-    a.n_P = r.n_parts;
+    a.n_B = a.n_P = 1;
     a.trace = nullptr;
     a.stream = (cudaStream_t)stream;
-    // short: one cluster, no workspace; else by radix where its workspace fits
-    // (it does up to PS_NOALLOC_MAX_KEYS)
+    // short: one cluster, no workspace; else by radix, whose workspace fits the array
+    // (8.5 MiB for PS_NOALLOC_MAX_KEYS 64-bit keys; the call checks it)
     if (n <= cluster_max(dtype)) return narrow ? run_cluster_u32(a) : run_cluster_u64(a);
-    if ((narrow ? radix_bytes_u32(a) : radix_bytes_u64(a)) <= PS_NOALLOC_SCRATCH_BYTES)
-        return narrow ? run_radix_u32(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES)
-                      : run_radix_u64(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);
-    return narrow ? run_sort_u32_on(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES)
-                  : run_sort_u64_on(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);
+    return narrow ? run_radix_u32(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES) : run_radix_u64(a, (char*)ws, PS_NOALLOC_SCRATCH_BYTES);
 }

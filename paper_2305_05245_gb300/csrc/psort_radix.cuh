@@ -127,15 +127,14 @@ struct RxBad {
     unsigned dp;              // bits that differ among its payloads and keys (the same)
     unsigned long long dk;
 };
-// Device tables and buffers of one radix sort.  Pass 0 reads `first`, pass i
-// writes b (i even) or a (i odd); a last pass of odd index writes `last`
-// instead of a.  (A last pass of even index leaves the keys in b: only when
-// low digits were left out, k_rx_fix then moves them to `last`.)
+// Device tables and buffers of one radix sort.  Pass 0 reads a, pass i writes b (i
+// even) or a (i odd).  (A last pass of even index leaves the keys in b: only when
+// low digits were left out, k_rx_fix then moves them to a.)
 template <typename K> struct RxArgs {
-    GBuf<K> first, a, b, last;
+    GBuf<K> a, b;
     Inst in;
     int64_t nseg;            // segments (instances)
-    K* const* iptr;          // instances in buffers of their own (first, a and last)
+    K* const* iptr;          // instances in buffers of their own, in place of a
     unsigned long long* hist;  // [nseg][D][256]: digit counts, then their exclusive sums
     RxPlan* plan;            // [nseg]
     unsigned* done;          // [nseg]: finished counting chunks
@@ -163,7 +162,6 @@ template <typename K> struct RxArgs {
     unsigned rows;           // its size
     unsigned spins;          // looks in vain at one predecessor (or count) before a wait gives up
     unsigned* err;           // set when one did (host memory, where someone waits for the sort)
-    int min_pass;            // least number of passes (a sort between two buffers needs some)
     bool keep;               // the last pass leaves order keys
 };
 constexpr int FT = 4096;  // positions of a fix tile (k_rx_fix)
@@ -231,7 +229,7 @@ template <typename K> __device__ __forceinline__ void rx_give_up(const RxArgs<K>
 // lo and above); a key that meets an earlier, different one of the same leading
 // bytes counts as a hit.  S keys have S^2/2 pairs, so a key has about
 // 2 * hits * n / S^2 different ones in its run; the smallest number of leading
-// bytes that keeps this at PS_RX_RUN or less wins.  Hits count whatever order
+// bytes that keeps this at RX_RUN or less wins.  Hits count whatever order
 // the two keys come in: nearly sorted input has long runs too.  A guess can be
 // wrong (one value makes up a large share of the input and few of its
 // neighbours share its leading bytes: the sample sees none of them); it then
@@ -243,9 +241,7 @@ template <typename K> __device__ __forceinline__ void rx_give_up(const RxArgs<K>
 // leave them in order, and such pairs are no hits.
 // The choices are RX_TRY numbers of leading bytes from the fewest that could
 // tell as many uniform keys apart.
-#ifndef PS_RX_RUN
-#define PS_RX_RUN 1
-#endif
+constexpr int RX_RUN = 1;
 constexpr int RX_SAMPLE_MAX = 1 << 16, RX_TRY = 4, RX_SLOTS = 4;  // (table slots per sampled key)
 // sqrt(8 n) sampled keys: runs with one other key each then give four hits.
 __host__ __device__ inline int rx_samples(int64_t n)
@@ -313,7 +309,7 @@ __global__ void __launch_bounds__(128) k_rx_sample(RxArgs<K> A)
     if (lo < 1) return;
     int64_t off, n;
     rx_seg(A, seg, off, n);
-    const GBuf<K> src = A.iptr ? rx_own(A.iptr, seg, 0, n) : rx_sub(A.first, off, n);
+    const GBuf<K> src = A.iptr ? rx_own(A.iptr, seg, 0, n) : rx_sub(A.a, off, n);
     auto pos = [&](int j) { return (int64_t)__umul64hi(rx_mix((uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull), (uint64_t)n); };
     const typename Rx<K>::M m = Rx<K>::mask(lo, D - 1);
     const bool asc = *A.descents == 0;
@@ -349,7 +345,7 @@ template <typename K> __device__ __forceinline__ int rx_choose_lo(const RxArgs<K
     if (at.S == 0) return 0;
     const int q = threadIdx.x & 31;
     const double h = q < RX_TRY ? (double)__ldcg(&A.hits[seg * RX_TRY + q]) : 0.0;
-    const bool ok = q < RX_TRY && h * 2.0 * (double)n <= (double)PS_RX_RUN * (double)at.S * (double)at.S;
+    const bool ok = q < RX_TRY && h * 2.0 * (double)n <= (double)RX_RUN * (double)at.S * (double)at.S;
     const unsigned b = __ballot_sync(0xFFFFFFFFu, ok);
     const int lo = b ? D - at.b0 - (__ffs(b) - 1) : 0;
     return lo < 0 ? 0 : lo;
@@ -436,7 +432,7 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
     for (int i = threadIdx.x; i < G * 4096; i += NT) cnt[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const GBuf<K> src = rx_global(A.iptr ? rx_own(A.iptr, seg, c0, (int64_t)n) : rx_sub(A.first, off + c0, (int64_t)n));
+    const GBuf<K> src = rx_global(A.iptr ? rx_own(A.iptr, seg, c0, (int64_t)n) : rx_sub(A.a, off + c0, (int64_t)n));
     auto add = [&](const K& k) {
 #pragma unroll
         for (int d = 0; d < G; d++) {
@@ -537,7 +533,7 @@ __global__ void __launch_bounds__(NT) k_rx_count(RxArgs<K> A)
         // filled up with digits that change nothing, unless k_rx_fix can move
         // the keys
         int want = lo0 ? act : act + (act & 1);
-        if (want < A.min_pass) want = A.min_pass;
+        if (A.keep && want < 2) want = 2;  // (they also turn the keys into order keys)
         int fill = want - act;
         p.npass = 0;
         for (int d = lo0; d < D; d++) {
@@ -603,13 +599,12 @@ __device__ __forceinline__ void rx_seg_pass(const RxArgs<K>& A, int64_t seg, int
     sg.npass = len > 0 ? pl.npass : 0;
     if (slot >= sg.npass) return;
     const int d = pl.dig[slot];
-    const bool tail = slot + 1 == sg.npass;
     const GBuf<K> own = A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.a, off, len);
     const GBuf<K> oth = rx_sub(A.b, off, len);
     sg.d = d;
-    sg.src = slot == 0 ? (A.iptr ? own : rx_sub(A.first, off, len)) : (slot & 1) ? oth : own;
-    sg.dst = !(slot & 1) ? oth : (tail && !A.iptr) ? rx_sub(A.last, off, len) : own;
-    sg.inv = tail && !A.keep;
+    sg.src = (slot & 1) ? oth : own;
+    sg.dst = (slot & 1) ? own : oth;
+    sg.inv = slot + 1 == sg.npass && !A.keep;
     sg.m = Rx<K>::mask(pl.lo, d);
     sg.mb = d > pl.lo ? Rx<K>::mask(pl.lo, d - 1) : typename Rx<K>::M{};
     rx_keep_ties(sg.m, sg.mb, pl.lo >= 4 && *A.descents == 0);
@@ -908,8 +903,8 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
 // even in place.  Longer runs are left to k_rx_long: a tile in which one of
 // them is out of order gets a flag (1: a run from an earlier tile, 2: one that
 // starts here and goes on into the next tile, 4: one inside the tile).
-// An odd number of passes left the keys in b: every key is then moved to
-// `last`.  Measured on 2^28 uniform uint64 keys, in place: 0.64 ms (every
+// An odd number of passes left the keys in b: every key is then moved to a.
+// Measured on 2^28 uniform uint64 keys, in place: 0.64 ms (every
 // position tested by its own thread with run scans of its own: 1.0 ms).
 constexpr int FN = 256, FL = 64;
 template <typename K, int XF>
@@ -928,7 +923,7 @@ __global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
     int64_t off, len;
     rx_seg(A, seg, off, len);
     const bool move = pl.npass & 1;
-    const GBuf<K> dst = rx_global(A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.last, off, len));
+    const GBuf<K> dst = rx_global(A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.a, off, len));
     const GBuf<K> src = rx_global(move ? rx_sub(A.b, off, len) : dst);
     const typename Rx<K>::M m = Rx<K>::mask(pl.lo, Rx<K>::D - 1);
     const bool inv = !A.keep;
@@ -1273,7 +1268,7 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
         rx_seg(A, (int64_t)q.seg, off, len);
         lo = A.plan[q.seg].lo;
         first = ascending && lo >= 4 ? 4 : 0;
-        x = rx_global(A.iptr ? rx_own(A.iptr, (int64_t)q.seg, 0, len) : rx_sub(A.last, off, len));
+        x = rx_global(A.iptr ? rx_own(A.iptr, (int64_t)q.seg, 0, len) : rx_sub(A.a, off, len));
         y = rx_global(rx_sub(A.b, off, len));
     };
     auto reached = [&](const unsigned* done, unsigned need, unsigned what) {

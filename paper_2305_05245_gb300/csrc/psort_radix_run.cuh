@@ -139,7 +139,7 @@ template <typename K> struct Radix {
         if constexpr (std::is_same<K, Rec>::value) {
             ProfScope ps_("radix_descents", s);
             const int64_t g = (A.in.n0 + 4095) / 4096;
-            launch_next(k_rx_descents<512>, (unsigned)std::min<int64_t>(g, grid_sms * 4), 512, 0, s, A.first.p, A.in.n0, A.descents);
+            launch_next(k_rx_descents<512>, (unsigned)std::min<int64_t>(g, grid_sms * 4), 512, 0, s, A.a.p, A.in.n0, A.descents);
         }
         if constexpr (D > 4) {
             ProfScope ps_("radix_sample", s);
@@ -191,8 +191,6 @@ template <typename K> struct Radix {
         RxArgs<K> A;
         A.a = gbuf_user<K>(a);
         A.b = gbuf_at<K>(ws + y.o_data, a.inst_base ? a.extent : a.n);
-        A.first = gbuf_ext<K>(a.src_keys, A.a);
-        A.last = gbuf_ext<K>(a.dst_keys, A.a);
         A.in.base = a.inst_base;
         A.in.n = a.inst_n;
         A.in.count = a.n_inst;
@@ -228,9 +226,6 @@ template <typename K> struct Radix {
         A.spins = radix_spins();
         A.err = a.err ? a.err : (unsigned*)(ws + y.o_misc + 40);
         A.keep = a.keep_order_keys;
-        // a sort between two buffers, or one that leaves order keys, moves
-        // (and transforms) the keys even when they are all equal
-        A.min_pass = (A.keep || a.src_keys || a.dst_keys) ? 2 : 0;
         return y.wide ? passes<XF, uint64_t>(a, y, A, ws, sms) : passes<XF, uint32_t>(a, y, A, ws, sms);
     }
 
