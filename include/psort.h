@@ -70,9 +70,12 @@ typedef enum {
 
 /* Tuning parameters.  0 in a field means "choose automatically" (a tuned
  * entry from ps_autotune, else the library's size-binned default).
- * A keys-only sort with every field automatic and no trace may sort its input
- * as one block whatever ps_resolve_params reports (the result is the same);
- * n_B and n_P then matter to sorts that fix them or ask for a trace.
+ * A sort (keys, pairs or structs) with automatic block counts and launch shape,
+ * the tree merge and no trace sorts its input as one block whatever
+ * ps_resolve_params reports (the result is the same; where the workspace for that
+ * does not fit the device, in the reported blocks), and so does one that gives
+ * n_blocks = n_parts = 1 without a launch shape or trace; n_B and n_P matter to
+ * the others.
  * n_blocks = n_B and n_parts = n_P of Sec. 2; both may exceed n (empty blocks
  * or partitions are legal).  Limits: 1 <= n_blocks <= 4096,
  * 1 <= n_parts <= 1048576.
@@ -206,7 +209,8 @@ int ps_batch_plan_destroy(ps_batch_plan* plan);
  * sorted, and with exact splitting (or automatic parameters) copy the result back
  * in partition ranges while later ranges merge.  Other memory, and automatic
  * sorts in between, are copied to a device buffer and back.  Device buffers come
- * from the library's pool. */
+ * from the library's pool.  PS_ERR_TIMEOUT: a bounded wait inside the sort gave up
+ * and the keys are lost (never in a correct run). */
 int ps_sort_host(void* host_keys, int64_t n, int dtype, int pivot_mode,
                  const ps_params* params, ps_stream_t stream);
 
@@ -298,8 +302,8 @@ int ps_server_debug_fail(ps_server* server, int what, int count);
  * result bit-identical) but takes all of its workspace from one static device
  * array of PS_NOALLOC_SCRATCH_BYTES that the library reserves on every GPU it
  * is loaded on, for the life of the process (short sorts need none of it).
- *   - n above PS_NOALLOC_MAX_KEYS (or a shape whose workspace would not fit
- *     the array) is rejected with PS_ERR_INVALID_ARG before any work is queued.
+ *   - n above PS_NOALLOC_MAX_KEYS is rejected with PS_ERR_INVALID_ARG before any
+ *     work is queued (up to there the workspace fits the array).
  *   - It calls no cudaMalloc, cudaFree or pool allocation.  (Keep profiling
  *     off: ps_profile_enable makes every launch create CUDA events.)
  *   - The first call in each CUDA context (per device: its primary context,

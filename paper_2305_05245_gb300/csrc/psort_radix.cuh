@@ -1223,17 +1223,19 @@ __device__ __forceinline__ bool rx_reached(const unsigned* done, unsigned need, 
 }
 
 // What k_rx_fix flagged.  All CTAs first list it (a task per LIST fix tiles, taken
-// in order from a counter) and wait until the list is whole.  The runs inside a tile are sorted together in shared
-// memory, by one CTA (they lie in order of their leading bytes already).  A run
-// that spans tiles is sorted by the bytes left out of the passes that vary in it,
-// lowest first, one CTA alone for up to LONG_ONE keys, all CTAs together for more:
-// its work is cut into tasks, taken in order from a counter:
+// in order from a counter) and wait until the list is whole.  (Listing in k_rx_fix
+// cost that kernel 3% where there is nothing to list.)  The runs inside a tile are
+// sorted together in shared memory, by one CTA (they lie in order of their leading
+// bytes already).  A run that spans tiles is sorted by the bytes left out of the
+// passes that vary in it, lowest first, by one CTA alone for up to LONG_ONE keys, by
+// all CTAs together for more: its work is cut into tasks, taken in order from a
+// counter:
 //   differing bits (a task per LONG_T keys); then for each varying byte: counts
 //   (the same), running sums of them (16), moves (the same); if the moves are odd
 //   in number, the way back.
 // A task waits until all tasks of the kinds before it are finished; those were
 // taken by CTAs that are running, so the waits end whatever share of the grid is
-// on the GPU.  (Listing in k_rx_fix costs that kernel 3% where there is nothing to list.)  So a sample that misjudged the input costs at most the passes it
+// on the GPU.  So a sample that misjudged the input costs at most the passes it
 // saved, each at a grid's full width, and a counting pass each.  Measured, a whole
 // sort (one CTA per run before / this kernel; uniform keys in brackets): 2^20 float64
 // of which 30% are the mean 34.9 / 0.23 ms (0.11), 2^24 uint64 of which half are zero
