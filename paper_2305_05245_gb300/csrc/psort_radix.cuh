@@ -1021,8 +1021,13 @@ __global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
 }
 
 // --------------------------------------------------------------- long runs
-// Keys of one task of k_rx_long, and the longest run that one CTA sorts alone.
-constexpr int LONG_T = 16384, LONG_ONE = 2 * LONG_T;
+// Keys of one task of k_rx_long, the longest run that one CTA sorts alone, and CTAs
+// per SM.  Tasks of short runs are short, so that all CTAs have some, and those of
+// long ones long: each costs some 3 us beside its keys (LONG_T / 2 LONG_T for all runs:
+// 2^20 float64 with 30% of the mean 204 / 245 us, 2^24 uint64, half zeros, 831 / 790
+// us; 4 LONG_T for 2^30 zeros with rare values below 2^16 16.9 ms, 2 LONG_T 18.4).
+constexpr int LONG_T = 8192, LONG_ONE = 2 * LONG_T, LONG_CTAS = 2;
+__device__ __forceinline__ int rx_task(int64_t m) { return m < (1 << 22) ? LONG_T : m < (1 << 25) ? 2 * LONG_T : 4 * LONG_T; }
 // The first position of [a, b) for which pred fails (it holds for those before),
 // by one warp, 32 probes a round.
 template <typename F> __device__ __forceinline__ int64_t rx_search(int64_t a, int64_t b, F pred)
@@ -1052,7 +1057,7 @@ __device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, 
     auto upto = [&](const K& v) { return [&](int64_t i) { return !Rx<K>::lt(v, ld(i), m); }; };
     auto list = [&](int64_t s, int64_t e, int inside) {
         if (!one) return;
-        const unsigned rows = e - s > LONG_ONE ? (unsigned)((e - s + LONG_T - 1) / LONG_T) : 0;
+        const unsigned rows = e - s > LONG_ONE ? (unsigned)((e - s + rx_task(e - s) - 1) / rx_task(e - s)) : 0;
         const unsigned slot = rows ? atomicAdd(bads + 1, rows) : 0u;
         if ((unsigned long long)slot + rows > maxrows) return;  // (only of keys that an abandoned wait left out of order)
         bad[atomicAdd(bads, 1u)] = RxBad{s, e, seg, inside, slot, 0, 0, 0, 0};
@@ -1094,8 +1099,19 @@ __device__ __forceinline__ void rx_range_bits(LD ld, int64_t a, int64_t b, const
         if (vp) atomicOr(dp, vp);
     }
 }
+// Whether every thread's digits v[U] are the same in a whole warp.
+template <int U> __device__ __forceinline__ bool rx_one_value(const unsigned (&v)[U])
+{
+    bool same = true;
+#pragma unroll
+    for (int u = 1; u < U; u++) same &= v[u] == v[0];
+    int one;
+    __match_all_sync(0xFFFFFFFFu, same ? v[0] : 256u, &one);
+    return __all_sync(0xFFFFFFFFu, same) && one;
+}
 // How often each value of digit d occurs in [a, b), into cnt[256] (one CTA; wt: a
-// table per warp).  Mostly one value, so a warp adds its lanes' equal digits as one.
+// table per warp).  Long runs mostly hold one value: a warp whose keys all have the
+// same digit adds them as one.
 template <int NT, typename K, typename LD>
 __device__ __forceinline__ void rx_range_count(LD ld, int64_t a, int64_t b, int d, uint32_t* wt, uint32_t* cnt)
 {
@@ -1111,18 +1127,13 @@ __device__ __forceinline__ void rx_range_count(LD ld, int64_t a, int64_t b, int 
             const int64_t i = c + u * NT + tid;
             v[u] = Rx<K>::dig(ld(i < b ? i : a), d);
         }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const bool in = c + u * NT + tid < b;
-            const unsigned act = __ballot_sync(0xFFFFFFFFu, in), v0 = __shfl_sync(0xFFFFFFFFu, v[u], 0);
-            int one;
-            __match_all_sync(0xFFFFFFFFu, in ? v[u] : v0, &one);  // (lane 0 is in if any lane is)
-            if (one && act) {
-                if (lane == 0) atomicAdd(&my[v[u]], (uint32_t)__popc(act));
-            } else if (in) {
-                atomicAdd(&my[v[u]], 1u);
-            }
+        if (c + NT * U <= b && rx_one_value(v)) {
+            if (lane == 0) atomicAdd(&my[v[0]], 32u * U);
+            continue;
         }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (c + u * NT + tid < b) atomicAdd(&my[v[u]], 1u);
     }
     __syncthreads();
     if (tid < 256) {
@@ -1168,8 +1179,18 @@ __device__ __forceinline__ void rx_range_scatter(LD ld, ST st, int64_t a, int64_
         uint32_t rk[E];
 #pragma unroll
         for (int j = 0; j < E; j++) k[j] = ld(p0 + j * 32 < b ? p0 + j * 32 : a);
+        unsigned dv[E];
+#pragma unroll
+        for (int j = 0; j < E; j++) dv[j] = Rx<K>::dig(k[j], d);
+        const bool one = c + NT * E <= b && rx_one_value(dv);
+        if (one) {
+            if (lane == 0) my[dv[0]] = 32 * E;
+#pragma unroll
+            for (int j = 0; j < E; j++) rk[j] = j * 32 + lane;
+        }
 #pragma unroll
         for (int j = 0; j < E; j++) {
+            if (one) break;
             const bool in = p0 + j * 32 < b;
             const unsigned v = Rx<K>::dig(k[j], d);
             unsigned mt = __ballot_sync(0xFFFFFFFFu, in);
@@ -1230,21 +1251,24 @@ __device__ __forceinline__ bool rx_reached(const unsigned* done, unsigned need, 
 // passes that vary in it, lowest first, by one CTA alone for up to LONG_ONE keys, by
 // all CTAs together for more: its work is cut into tasks, taken in order from a
 // counter:
-//   differing bits (a task per LONG_T keys); then for each varying byte: counts
+//   differing bits (a task per rx_task keys); then for each varying byte: counts
 //   (the same), running sums of them (16), moves (the same); if the moves are odd
 //   in number, the way back.
 // A task waits until all tasks of the kinds before it are finished; those were
 // taken by CTAs that are running, so the waits end whatever share of the grid is
 // on the GPU.  So a sample that misjudged the input costs at most the passes it
-// saved, each at a grid's full width, and a counting pass each.  Measured, a whole
-// sort (one CTA per run before / this kernel; uniform keys in brackets): 2^20 float64
-// of which 30% are the mean 34.9 / 0.23 ms (0.11), 2^24 uint64 of which half are zero
-// 1171 / 1.05 ms (0.42), 2^26 int64 zeros with 1e-4 small values 7288 / 2.1 ms (1.44),
-// 2^26 records of such keys 8622 / 3.0 ms (2.4).
+// saved, each at a grid's full width, and a counting pass each.  A warp whose keys all
+// have the same digit, as most of such a run's have, counts and ranks them without
+// looking at them one by one; two CTAs per SM hide each other's barriers (one, and every
+// key ranked by ballots: 2^30 zeros with rare values below 2^24 50.7 ms, now 25.1).
+// Measured, a whole sort (one CTA per run before / this kernel; uniform keys in
+// brackets): 2^20 float64 of which 30% are the mean 34.9 / 0.20 ms (0.11), 2^24 uint64
+// of which half are zero 1171 / 0.79 ms (0.41), 2^26 int64 zeros with 1e-4 small values
+// 7288 / 1.26 ms (1.44), 2^26 records of such keys 8622 / 2.3 ms (2.4).
 // Records whose payloads ascend keep that order in a run: equal keys need no
 // payload digits.
 template <typename K, int XF, typename CT>
-__global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
+__global__ void __launch_bounds__(512, LONG_CTAS) k_rx_long(RxArgs<K> A)
 {
     kernel_entry();
     constexpr int NT = 512, E = 8, W = NT / 32;
@@ -1375,7 +1399,8 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
             RxBad* bad = A.bad + (start + pick) % nbad;
             open(*bad);
             const int64_t s = bad->s, e = bad->e;
-            const unsigned nt = (unsigned)((e - s + LONG_T - 1) / LONG_T);
+            const int T = rx_task(e - s);
+            const unsigned nt = (unsigned)((e - s + T - 1) / T);
             CT* table = (CT*)A.dtab + (size_t)bad->slot * 256;  // [256][nt]: counts, then their running sums
             K bits{};
             int digits = -1;  // varying bytes, once known
@@ -1386,7 +1411,7 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
                 const unsigned t = s_t;
                 if (t < nt) {
                     const auto ld = from(false);
-                    const int64_t a = s + (int64_t)t * LONG_T, b = a + LONG_T < e ? a + LONG_T : e;
+                    const int64_t a = s + (int64_t)t * T, b = a + T < e ? a + T : e;
                     rx_range_bits<NT, K>(ld, a, b, ld(s), &bad->dk, &bad->dp);
                 } else {
                     if (digits < 0) {
@@ -1407,27 +1432,42 @@ __global__ void __launch_bounds__(512) k_rx_long(RxArgs<K> A)
                         if (Rx<K>::dig(bits, d) != 0 && c++ == di) break;
                     const bool swapped = di & 1;
                     const unsigned tile = kind == 2 ? sub - nt - 16 : sub;
-                    const int64_t a = s + (int64_t)tile * LONG_T, b = a + LONG_T < e ? a + LONG_T : e;
+                    const int64_t a = s + (int64_t)tile * T, b = a + T < e ? a + T : e;
                     if (back) {
-                        for (int64_t i = a + tid; i < b; i += NT) x.st(i, y.ld(i));
+                        constexpr int U = 8;
+                        for (int64_t i = a + tid; i < b; i += NT * U) {
+                            K v[U];
+#pragma unroll
+                            for (int u = 0; u < U; u++)
+                                if (i + u * NT < b) v[u] = y.ld(i + u * NT);
+#pragma unroll
+                            for (int u = 0; u < U; u++)
+                                if (i + u * NT < b) x.st(i + u * NT, v[u]);
+                        }
                     } else if (kind == 0) {
                         rx_range_count<NT, K>(from(swapped), a, b, d, wt, cnt);
                         if (tid < 256) table[(size_t)tid * nt + tile] = cnt[tid];
                     } else if (kind == 1) {
                         // a warp per value: inclusive sums of its tiles' counts
                         CT* row = table + (size_t)((sub - nt) * W + (tid >> 5)) * nt;
+                        constexpr int U = 8;
                         CT sum = 0;
-                        for (unsigned i0 = 0; i0 < nt; i0 += 32) {
+                        for (unsigned i0 = 0; i0 < nt; i0 += 32 * U) {
                             const unsigned i = i0 + (tid & 31);
-                            CT v = i < nt ? __ldcg(row + i) : (CT)0;
+                            CT v[U];
 #pragma unroll
-                            for (int o = 1; o < 32; o <<= 1) {
-                                const CT u = __shfl_up_sync(0xFFFFFFFFu, v, o);
-                                if ((tid & 31) >= o) v += u;
+                            for (int u = 0; u < U; u++) v[u] = i + 32 * u < nt ? __ldcg(row + i + 32 * u) : (CT)0;
+#pragma unroll
+                            for (int u = 0; u < U; u++) {
+#pragma unroll
+                                for (int o = 1; o < 32; o <<= 1) {
+                                    const CT w = __shfl_up_sync(0xFFFFFFFFu, v[u], o);
+                                    if ((tid & 31) >= o) v[u] += w;
+                                }
+                                v[u] += sum;
+                                sum = __shfl_sync(0xFFFFFFFFu, v[u], 31);
+                                if (i + 32 * u < nt) row[i + 32 * u] = v[u];
                             }
-                            v += sum;
-                            if (i < nt) row[i] = v;
-                            sum = __shfl_sync(0xFFFFFFFFu, v, 31);
                         }
                     } else {
                         unsigned long long mine = 0, all = 0;

@@ -170,13 +170,15 @@ template <typename K> struct Radix {
             }
             auto fl = k_rx_long<K, XF, CT>;
             const size_t lb = std::max(TileBuf<K, 8>::type::bytes(FT), (size_t)(16 * 256 * 4 + 256 * 8 + 256 * 4 + 64));
-            // at most 1.5 rows per LONG_T keys, in the look-back tables of 1 row per tile
-            static_assert(3 * C::Large::T <= 2 * LONG_T && 3 * C::Mid::T <= 2 * LONG_T && 3 * C::Small::T <= 2 * LONG_T,
-                          "the digit table fits the look-back tables");
-            static_assert(sizeof(RxBad) * 2 * C::Large::T <= 1024 * FT, "and so does the list");
+            // the digit table (at most 1.5 rows of 1 KiB per LONG_T keys) and the list (two
+            // entries per fix tile) share the look-back tables (two rows per tile)
+            static_assert(2048.0 / C::Large::T >= 1.5 * 1024 / LONG_T + 2.0 * sizeof(RxBad) / FT &&
+                              2048.0 / C::Mid::T >= 1.5 * 1024 / LONG_T + 2.0 * sizeof(RxBad) / FT &&
+                              2048.0 / C::Small::T >= 1.5 * 1024 / LONG_T + 2.0 * sizeof(RxBad) / FT,
+                          "the digit table and the list fit the look-back tables");
             if ((e = smem_attr(fl, lb)) != cudaSuccess) return e;
             ProfScope ps_("radix_long", s);
-            launch_next(fl, (unsigned)grid_sms, 512, lb, s, A);
+            launch_next(fl, (unsigned)grid_sms * LONG_CTAS, 512, lb, s, A);
         }
         return cudaGetLastError();
     }
@@ -220,9 +222,10 @@ template <typename K> struct Radix {
         A.flags = (uint8_t*)(ws + y.o_flags);
         A.started = (unsigned*)(ws + y.o_started);
         // the look-back tables serve k_rx_long once the passes are over
+        const size_t list = align256((size_t)y.fixes * 2 * sizeof(RxBad));
         A.dtab = ws + y.o_lb0;
-        A.rows = (unsigned)std::min<int64_t>(y.tiles, 0x7FFFFFFF);
-        A.bad = (RxBad*)(ws + y.o_lb1);
+        A.rows = (unsigned)std::min<size_t>((y.o_plan - y.o_lb0 - list) / (y.wide ? 2048 : 1024), 0x7FFFFFFF);
+        A.bad = (RxBad*)(ws + y.o_plan - list);
         A.spins = radix_spins();
         A.err = a.err ? a.err : (unsigned*)(ws + y.o_misc + 40);
         A.keep = a.keep_order_keys;

@@ -11,7 +11,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-TILE, TASK, ALONE = 4096, 16384, 32768  # fix tile, keys of a task, longest run of one CTA
+TILE, TASK, ALONE = 4096, 8192, 16384  # fix tile, keys of a task, longest run of one CTA
 
 
 @pytest.fixture(scope="module")
@@ -63,7 +63,7 @@ def check(ps, u, view=np.int64):
 
 
 EDGES = [(65,), (TILE - 1,), (TILE,), (TILE + 1,), (ALONE - 1,), (ALONE,), (ALONE + 1,), (3 * TASK - 1,), (3 * TASK,),
-         (3 * TASK + 1,), (9 * TASK + 77,), (200000, 100000, 33000, 32768, 5000, 100, 70)]
+         (3 * TASK + 1,), (9 * TASK + 77,), (200000, 100000, 33000, 16384, 5000, 100, 70)]
 
 
 @pytest.mark.parametrize("runs", EDGES)
