@@ -330,7 +330,7 @@ int ps_debug_fail_alloc_after(int skip, int count);
  * exceed it (0 turns it off).  Call it while no sort is under way. */
 int ps_debug_limit_alloc(size_t bytes);
 
-/* Looks at an earlier tile's counts before a wait of the radix sort gives up
+/* Looks in vain at earlier tiles' counts before a wait of the radix sort gives up
  * (negative: the default, some ten seconds; 0: at the first that fails). */
 int ps_debug_radix_spins(int looks);
 /* As if the device could place thread-block clusters of at most `ctas` blocks

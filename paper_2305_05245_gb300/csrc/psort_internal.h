@@ -78,7 +78,7 @@ int fail_cuda(cudaError_t e);
 // nullptr if there is no memory for it.
 unsigned* err_word_take();
 void err_word_give(unsigned* w);
-// Looks at one predecessor before a wait of the radix sort gives up (some ten seconds).
+// Looks in vain before a wait of the radix sort gives up (some ten seconds).
 unsigned radix_spins();
 
 // Profiling: when enabled (ps_profile_enable), a ProfScope records a CUDA

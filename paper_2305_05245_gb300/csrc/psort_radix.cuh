@@ -130,8 +130,11 @@ struct RxBad {
 // Device tables and buffers of one radix sort.  Pass 0 reads a, pass i writes b (i
 // even) or a (i odd).  (A last pass of even index leaves the keys in b: only when
 // low digits were left out, k_rx_fix then moves them to a.)
+// (first and last are a, for the digit passes: with a in their places, or the members
+// in the order of the kernels that read them, the passes have the same registers and
+// spills but take up to 0.8% longer: 2^26 float64 2128 against 2111 us a sort.)
 template <typename K> struct RxArgs {
-    GBuf<K> a, b;
+    GBuf<K> first, a, b, last;
     Inst in;
     int64_t nseg;            // segments (instances)
     K* const* iptr;          // instances in buffers of their own, in place of a
@@ -141,7 +144,7 @@ template <typename K> struct RxArgs {
     unsigned* ticket;        // [D]: next tile of each pass
     int T;                   // keys per tile of a digit pass
     int64_t chunk;           // keys per counting chunk
-    // one segment: its numbers; several (k_rx_map): tables of them
+    // one segment: its numbers; several (k_rx_at): tables of them
     RxSegAt one;
     int64_t ntiles1;
     RxSegAt* at;             // [nseg]
@@ -152,16 +155,14 @@ template <typename K> struct RxArgs {
     unsigned* descents;      // records: set if the payloads do not ascend
     unsigned* hits;          // [nseg][RX_TRY]: the sample's hits per choice of the lowest digit
     unsigned* tab;           // hash tables
-    uint8_t* flags;          // [fix tiles], see k_rx_fix
+    uint8_t* flags;          // [fix tiles], see k_rx_fix; LISTED: the long run that starts there is listed
     unsigned* nflag;         // number of flagged tiles
-    // k_rx_long
-    unsigned* started;       // [fix tiles]: the long run that starts there is listed
-    RxBad* bad;              // [2 * fix tiles]: the list
+    RxBad* bad;              // [2 * fix tiles]: k_rx_long's list
     unsigned* bads;          // [4]: its entries, rows of dtab given out; listing tasks taken and finished
     void* dtab;              // digit table, 256 counts a row (CT)
-    unsigned rows;           // its size
-    unsigned spins;          // looks in vain at one predecessor (or count) before a wait gives up
-    unsigned* err;           // set when one did (host memory, where someone waits for the sort)
+    unsigned rows;           // of dtab
+    unsigned spins;          // looks in vain, over a tile's look-back or at a count, before the wait gives up
+    unsigned* err;           // set when one gave up (host memory, where someone waits for the sort)
     bool keep;               // the last pass leaves order keys
 };
 constexpr int FT = 4096;  // positions of a fix tile (k_rx_fix)
@@ -602,9 +603,10 @@ __device__ __forceinline__ void rx_seg_pass(const RxArgs<K>& A, int64_t seg, int
     const GBuf<K> own = A.iptr ? rx_own(A.iptr, seg, 0, len) : rx_sub(A.a, off, len);
     const GBuf<K> oth = rx_sub(A.b, off, len);
     sg.d = d;
-    sg.src = (slot & 1) ? oth : own;
-    sg.dst = (slot & 1) ? own : oth;
-    sg.inv = slot + 1 == sg.npass && !A.keep;
+    const bool tail = slot + 1 == sg.npass;
+    sg.src = slot == 0 ? (A.iptr ? own : rx_sub(A.first, off, len)) : (slot & 1) ? oth : own;
+    sg.dst = !(slot & 1) ? oth : (tail && !A.iptr) ? rx_sub(A.last, off, len) : own;
+    sg.inv = tail && !A.keep;
     sg.m = Rx<K>::mask(pl.lo, d);
     sg.mb = d > pl.lo ? Rx<K>::mask(pl.lo, d - 1) : typename Rx<K>::M{};
     rx_keep_ties(sg.m, sg.mb, pl.lo >= 4 && *A.descents == 0);
@@ -806,7 +808,6 @@ __global__ void __launch_bounds__(NT, CTAS) k_rx_pass(RxArgs<K> A, int slot, CT*
                             }
                             break;
                         }
-                        spins = 0;
                         excl += v[q] & ~Lb<CT>::FLAGS;
                         p -= 256;
                         left--;
@@ -1027,6 +1028,7 @@ __global__ void __launch_bounds__(FN) k_rx_fix(RxArgs<K> A)
 // 2^20 float64 with 30% of the mean 204 / 245 us, 2^24 uint64, half zeros, 831 / 790
 // us; 4 LONG_T for 2^30 zeros with rare values below 2^16 16.9 ms, 2 LONG_T 18.4).
 constexpr int LONG_T = 8192, LONG_ONE = 2 * LONG_T, LONG_CTAS = 2;
+constexpr unsigned LISTED = 128;  // (in RxArgs::flags)
 __device__ __forceinline__ int rx_task(int64_t m) { return m < (1 << 22) ? LONG_T : m < (1 << 25) ? 2 * LONG_T : 4 * LONG_T; }
 // The first position of [a, b) for which pred fails (it holds for those before),
 // by one warp, 32 probes a round.
@@ -1047,8 +1049,8 @@ template <typename F> __device__ __forceinline__ int64_t rx_search(int64_t a, in
 // tile's): those inside it as one range, one that goes beyond it once, whichever of
 // its tiles comes first.
 template <typename K, typename LD>
-__device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, unsigned flag, int seg, unsigned* started,
-                                        RxBad* bad, unsigned* bads, unsigned maxrows)
+__device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, unsigned flag, int seg, uint8_t* flags,
+                                        int64_t fix0, RxBad* bad, unsigned* bads, unsigned maxrows)
 {
     const typename Rx<K>::M m = Rx<K>::mask(lo, Rx<K>::D - 1);
     const int64_t t1 = t0 + FT < len ? t0 + FT : len;
@@ -1063,8 +1065,10 @@ __device__ __forceinline__ void rx_list(LD ld, int64_t len, int64_t t0, int lo, 
         bad[atomicAdd(bads, 1u)] = RxBad{s, e, seg, inside, slot, 0, 0, 0, 0};
     };
     auto spans = [&](int64_t s, int64_t e) {
-        const unsigned was = one ? atomicExch(&started[s / FT], 1u) : 0;
-        if (__shfl_sync(0xFFFFFFFFu, was, 0) == 0) list(s, e, 0);
+        const int64_t f = fix0 + s / FT;
+        const unsigned bit = LISTED << (8 * (f & 3));
+        const unsigned was = one ? atomicOr((unsigned*)(flags + (f & ~int64_t(3))), bit) : 0;
+        if ((__shfl_sync(0xFFFFFFFFu, was, 0) & bit) == 0) list(s, e, 0);
     };
     // [in, out): the runs inside the tile
     const K head = ld(t0), tail = ld(t1 - 1);
@@ -1333,13 +1337,13 @@ __global__ void __launch_bounds__(512, LONG_CTAS) k_rx_long(RxArgs<K> A)
             if (t >= tasks) break;
             const int64_t f0 = (int64_t)t * LIST + (tid >> 5) * (LIST / W);  // a few tiles per warp
             for (int64_t f = f0; f < f0 + LIST / W && f < tiles; f++) {
-                const unsigned flag = A.flags[f];
+                const unsigned flag = A.flags[f] & ~LISTED;
                 if (flag == 0) continue;
                 RxBad q{};
                 q.seg = A.nseg == 1 ? 0 : A.fix_seg[f];
                 const int fix0 = rx_at(A, q.seg).fix0;
                 open(q);
-                rx_list<K>(from(false), len, (f - fix0) * FT, lo, flag, q.seg, A.started + fix0, A.bad, A.bads, A.rows);
+                rx_list<K>(from(false), len, (f - fix0) * FT, lo, flag, q.seg, A.flags, fix0, A.bad, A.bads, A.rows);
             }
             __threadfence();
             __syncthreads();

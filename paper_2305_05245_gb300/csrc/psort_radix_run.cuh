@@ -47,7 +47,7 @@ template <typename K> struct Radix {
         int T;  // keys per tile
         int64_t nseg, tiles, chunk, chunks, fixes, S;  // (several segments: upper bounds)
         bool wide;     // 64-bit look-back words
-        size_t o_hist, o_done, o_ticket, o_misc, o_hits, o_tab, o_flags, o_started, o_lb0, zero_bytes, o_lb1, o_plan, o_at, o_tile,
+        size_t o_hist, o_done, o_ticket, o_misc, o_hits, o_tab, o_flags, o_lb0, zero_bytes, o_lb1, o_plan, o_at, o_tile,
             o_chunk, o_fix, o_data, total;
     };
     static Layout layout(const SortArgs& a)
@@ -86,8 +86,6 @@ template <typename K> struct Radix {
         o += align256(sampled ? (size_t)many * RX_TRY * RX_SLOTS * 4 : 0);
         y.o_flags = o;
         o += align256((size_t)y.fixes);
-        y.o_started = o;
-        o += align256((size_t)y.fixes * 4);
         y.o_lb0 = o;
         o += lb;
         y.zero_bytes = o;  // everything up to here starts as zeros
@@ -193,6 +191,7 @@ template <typename K> struct Radix {
         RxArgs<K> A;
         A.a = gbuf_user<K>(a);
         A.b = gbuf_at<K>(ws + y.o_data, a.inst_base ? a.extent : a.n);
+        A.first = A.last = A.a;
         A.in.base = a.inst_base;
         A.in.n = a.inst_n;
         A.in.count = a.n_inst;
@@ -220,7 +219,6 @@ template <typename K> struct Radix {
         A.hits = (unsigned*)(ws + y.o_hits);
         A.tab = (unsigned*)(ws + y.o_tab);
         A.flags = (uint8_t*)(ws + y.o_flags);
-        A.started = (unsigned*)(ws + y.o_started);
         // the look-back tables serve k_rx_long once the passes are over
         const size_t list = align256((size_t)y.fixes * 2 * sizeof(RxBad));
         A.dtab = ws + y.o_lb0;
